@@ -13,18 +13,24 @@
 // a few dozen rows, so it is bound by HBM and everything else hides under
 // that stream:
 //  * lm_head_kernel: one CTA per SM, each owning an equal contiguous range
-//    of vocabulary rows (floor or ceil of V / G), cut into 128-row tiles; a
+//    of vocabulary rows (floor or ceil of V / G), cut into 256-row tiles; a
 //    range's last tile is loaded with a box of exactly its remaining height
 //    (two extra tensor maps), so every SM streams the same number of weight
-//    bytes.  Warp 5 streams 128 x 64 weight boxes and
+//    bytes.  Warp 9 streams 256 x 64 weight boxes and
 //    the matching 64-column box of the hidden states (rows padded to NP, a
-//    multiple of 16, by the copy's zero fill) into a deep ring; warp 4 issues
-//    logits^T = W H^T as tcgen05 MMAs of M = 128 (vocabulary), N = NP (draft
-//    rows), K = 16, accumulating in tensor memory, double-buffered per tile;
-//    warps 0-3 read a finished tile back (one vocabulary row per lane),
-//    store the fp32 logits coalesced along the vocabulary and, for the fused
-//    path, reduce each draft row over the tile to (max, first argmax,
-//    float-float sum of exp((x - max)/tau)), merged across the CTA's tiles.
+//    multiple of 16, by the copy's zero fill) into a deep ring; warp 8 issues
+//    logits^T = W H^T as tcgen05 MMAs of M = 128 (a half tile of the
+//    vocabulary), N = NP (draft rows), K = 16, accumulating in tensor memory,
+//    double-buffered per tile where that fits; warps 0-7 (four per half) read
+//    a finished tile back (one vocabulary row per lane), store the fp32 logits
+//    coalesced along the vocabulary and, for the fused path, reduce each
+//    draft row over the tile to (max, first argmax, float-float sum of
+//    exp((x - max)/tau)), merged across the CTA's tiles.
+//    Tiles of 256 rows, not 128: the hidden-state box is re-read from L2 for
+//    every tile, and a CTA of V = 32000 (210 rows) has one tile and one
+//    exposed epilogue instead of two.  Measured with 128 and 256 rows:
+//    5 rows x 32000 x 4096 50.8 -> 41.1 us (6.4 TB/s), 36 x 152064 x 3584
+//    171.0 -> 161.7, 128 x 152064 x 3584 195.7 -> 183 us.
 //    Weight copies run before griddepcontrol.wait (the weights are constant);
 //    the hidden states are copied after it.
 //  * sample_stats_kernel (sf_sample only): the same per-chunk statistics
@@ -54,19 +60,21 @@
 
 namespace sf {
 
-constexpr int kLmThreads = 192;
-constexpr int kLmEpiThreads = 128;
-constexpr int kLmMmaWarp = 4;
-constexpr int kLmProducerWarp = 5;
-constexpr int kLmTileV = 128;                          // vocabulary rows per tile (MMA M)
+constexpr int kLmThreads = 320;
+constexpr int kLmHalf = 128;                           // vocabulary rows per MMA (M), threads per epilogue group
+constexpr int kLmEpiThreads = 2 * kLmHalf;             // one group per half tile
+constexpr int kLmMmaWarp = 8;
+constexpr int kLmProducerWarp = 9;
+constexpr int kLmTileV = 2 * kLmHalf;                  // vocabulary rows per tile: two MMAs share a hidden-state box
 constexpr int kLmChunkK = 64;                          // hidden columns per ring slot
-constexpr uint32_t kLmWBytes = kLmTileV * kLmChunkK * 2;  // 16 KB weight box
-constexpr int kLmMaxStages = 12;
+constexpr int kLmMaxStages = 32;
+constexpr int kLmEpiWarps = kLmEpiThreads / 32;
 constexpr int kLmColGroup = 16;                        // draft rows per epilogue step
-constexpr int kLmTStride = 136;                        // floats per transposed row (8 mod 32 banks)
-constexpr int kLmTBufFloats = 2 * kLmColGroup * kLmTStride;
+constexpr int kLmTStride = 34;                         // floats per transposed row (2 mod 32 banks)
+constexpr int kLmTBufFloats = kLmColGroup * kLmTStride;  // per epilogue warp
 constexpr int kSampleUnit = 2048;                      // tokens per statistics chunk (sf_sample)
-constexpr int kSampleSpan = 4096;                      // least tokens per finishing CTA
+constexpr int kSampleSpan = 1024;                      // least tokens per finishing CTA (4 per thread)
+constexpr int kFinishCtasPerSm = 5;                    // resident finishing CTAs (registers)
 constexpr int kMaxStatChunks = 4096;                   // statistics chunks per row
 
 struct LmParams {
@@ -78,7 +86,10 @@ struct LmParams {
   int G;             // CTAs; CTA c owns vocabulary rows [c*V/G, (c+1)*V/G)
   int ha, hb;        // box heights of the two last-tile weight maps
   int KC;            // hidden chunks of 64
+  int halves;        // 128-row halves of a tile in use (1: no CTA owns more than 128 rows)
+  int nbuf;          // accumulator buffers in tensor memory (2, or 1)
   int stages;
+  uint32_t w_bytes;      // weight box of the tallest tile
   uint32_t stage_bytes;  // weight box + NP * 128 bytes of hidden states
   uint32_t tmem_cols;
   uint32_t idesc;
@@ -108,8 +119,16 @@ struct SampleParams {
 // ---------------------------------------------------------------------------
 struct LmSmem {
   static size_t bytes(int stages, uint32_t stage_bytes, int NP) {
-    return 1024 + static_cast<size_t>(stages) * stage_bytes + 4 * kLmTBufFloats +
-           static_cast<size_t>(NP) * (sizeof(SampStat) + 4) + 8 * (2 * stages + 5) + 64;
+    // ring | transposed values and running statistics of every epilogue warp |
+    // temperatures | barriers | misc.  An MMA reads 128 rows from its half's
+    // first row, whatever the box's height: what lies behind the last slot
+    // covers the rest of a tile, so that those reads stay inside the allocation.
+    const size_t behind = kLmEpiWarps * 4 * kLmTBufFloats +
+                          static_cast<size_t>(NP) * (kLmEpiWarps * sizeof(SampStat) + 4) +
+                          8 * (2 * stages + 5) + 64;
+    const size_t tile = kLmTileV * kLmChunkK * 2;
+    return 1024 + static_cast<size_t>(stages) * stage_bytes +
+           (behind + stage_bytes > tile ? behind : tile - stage_bytes);
   }
 };
 
@@ -125,12 +144,90 @@ __device__ __forceinline__ void stat_merge(SampStat &run, float m, int arg, ff s
                                            bool greedy) {
   if (better(m, arg, run.m, run.arg)) {
     if (!greedy)
-      run.S = run.m == -INFINITY ? s : ff_add(ff_mul(run.S, exp_diff_accurate(run.m, m, tau)), s);
+      run.S = ff_add(run.m == -INFINITY ? run.S : ff_mul(run.S, exp_diff_accurate(run.m, m, tau)), s);
     run.m = m;
     run.arg = arg;
   } else if (!greedy) {
     run.S = ff_add(run.S, ff_mul(s, term_of(m, run.m, tau)));
   }
+}
+
+// One epilogue step of a warp: 16 draft rows (TMEM columns from `taddr`) of
+// its 32 vocabulary rows vbase .. vbase + 31 (one per lane).  The fp32 logits go
+// straight to global memory, coalesced along the vocabulary.  For the
+// statistics (wrun: the warp's running statistics of these draft rows) the
+// warp transposes the values through its own shared memory tb, so that two
+// lanes hold a draft row, 16 values each: the maximum, its first index and the
+// float-float sum of their terms as trees, so that a lane's exponentials
+// overlap; warps never wait for one another.
+__device__ __forceinline__ void lm_epilogue_step(uint32_t taddr, float *logits, int V, int vbase, bool vin,
+                                                 int cols_left, float *tb, const float *tau_row,
+                                                 SampStat *wrun) {
+  const int lane = threadIdx.x & 31;
+  uint32_t x[16];
+  tmem_ld_32x32b_x16(taddr, x);
+  if (vin) {
+    float *dst = logits + vbase + lane;
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (j < cols_left) dst[static_cast<size_t>(j) * V] = __uint_as_float(x[j]);
+  }
+  if (!wrun) return;
+  __syncwarp();  // the previous step's reads are done
+#pragma unroll
+  for (int j = 0; j < 16; ++j) tb[j * kLmTStride + lane] = vin ? __uint_as_float(x[j]) : -INFINITY;
+  __syncwarp();
+  const int part = lane & 1, r = lane >> 1;
+  const float *col = tb + r * kLmTStride + part;
+  float xv[16];
+#pragma unroll
+  for (int e = 0; e < 16; ++e) xv[e] = col[2 * e];
+  float mx[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) mx[e] = fmaxf(xv[e], xv[e + 8]);
+#pragma unroll
+  for (int w = 4; w >= 1; w >>= 1) {
+#pragma unroll
+    for (int e = 0; e < w; ++e) mx[e] = fmaxf(mx[e], mx[e + w]);
+  }
+  float bv = fmaxf(mx[0], -INFINITY);  // NaN values only: -inf
+  unsigned hits = 0u;
+#pragma unroll
+  for (int e = 0; e < 16; ++e) hits |= xv[e] == bv ? 1u << e : 0u;
+  int bi = hits ? vbase + part + 2 * (__ffs(hits) - 1) : INT_MAX;  // first index of the maximum
+  {
+    const float ov = __shfl_xor_sync(0xffffffffu, bv, 1);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, 1);
+    if (better(ov, oi, bv, bi)) {
+      bv = ov;
+      bi = oi;
+    }
+  }
+  const float tau = tau_row[r];
+  const bool greedy = !(tau > 0.f);
+  ff s = ff_of(0.f);
+  if (!greedy) {
+    // terms exp((x - bv) / tau), the argument carried to float-float
+    const float ref = bv == -INFINITY ? 0.f : bv;  // all masked: every term is 0
+    if (tau == 1.f) {  // one branch for all: the divisions are skipped together
+#pragma unroll
+      for (int e = 0; e < 16; ++e) xv[e] = term_of(xv[e], ref, 1.f);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 16; ++e) xv[e] = term_of(xv[e], ref, tau);
+    }
+    ff t[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) t[e] = two_sum(xv[e], xv[e + 8]);
+#pragma unroll
+    for (int w = 4; w >= 1; w >>= 1) {
+#pragma unroll
+      for (int e = 0; e < w; ++e) t[e] = ff_add(t[e], t[e + w]);
+    }
+    s = t[0];
+  }
+  s = ff_add(s, shfl_xor_ff(s, 1));
+  if (part == 0) stat_merge(*(wrun + r), bv, bi, s, tau, greedy);
 }
 
 __global__ void __launch_bounds__(kLmThreads, 1)
@@ -143,8 +240,8 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
   const int S = p.stages;
   const uint32_t ring = smem_addr(smem);
   float *tbuf = reinterpret_cast<float *>(smem + static_cast<size_t>(S) * p.stage_bytes);
-  SampStat *run = reinterpret_cast<SampStat *>(tbuf + kLmTBufFloats);
-  float *s_tau = reinterpret_cast<float *>(run + p.NP);
+  SampStat *run = reinterpret_cast<SampStat *>(tbuf + kLmEpiWarps * kLmTBufFloats);
+  float *s_tau = reinterpret_cast<float *>(run + kLmEpiWarps * p.NP);
   uint64_t *bar_mem = reinterpret_cast<uint64_t *>(s_tau + p.NP);
   int *s_misc = reinterpret_cast<int *>(bar_mem + 2 * S + 5);
   // s_misc: [0] TMEM base, [1] abort word, [2] chunks issued, [3] chunks consumed
@@ -178,7 +275,7 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     }
     for (int x = 0; x < 2; ++x) {
       mbar_init(bar(DFULL + x), 1);
-      mbar_init(bar(DEMPTY + x), kLmEpiThreads);
+      mbar_init(bar(DEMPTY + x), static_cast<uint32_t>(p.halves * kLmHalf));
     }
     mbar_init(bar(FIN), 1);
     fence_mbar_init();
@@ -204,7 +301,7 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
       tmem_relinquish_alloc_permit();
       tc_fence_before_sync();
     }
-    named_bar_sync(3, kLmEpiThreads + 32);
+    named_bar_sync(2, kLmEpiThreads + 32);
     tc_fence_after_sync();
     tmem = static_cast<uint32_t>(s_misc[0]);
   }
@@ -228,7 +325,7 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
       if (!p.w_after_wait) grid_dependency_wait();
       for (uint32_t q = 0; q < prime; ++q) {
         const int kc = kc0 + static_cast<int>(q) % nkc;
-        tma_load_2d(ring + q * p.stage_bytes + kLmWBytes, &tmap_h, kc * kLmChunkK, 0, bar(FULL + q),
+        tma_load_2d(ring + q * p.stage_bytes + p.w_bytes, &tmap_h, kc * kLmChunkK, 0, bar(FULL + q),
                     pol_h);
       }
       uint32_t q = prime;
@@ -241,29 +338,31 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         const CUtensorMap *mw = tile_map(i, bytes);
         mbar_arrive_expect_tx(bar(FULL + slot), bytes);
         tma_load_2d(dst, mw, kc * kLmChunkK, v0 + i * kLmTileV, bar(FULL + slot), pol_w);
-        tma_load_2d(dst + kLmWBytes, &tmap_h, kc * kLmChunkK, 0, bar(FULL + slot), pol_h);
+        tma_load_2d(dst + p.w_bytes, &tmap_h, kc * kLmChunkK, 0, bar(FULL + slot), pol_h);
       }
       s_misc[2] = static_cast<int>(q);
     }
     __syncwarp();
   } else if (warp == kLmMmaWarp) {
     // ------------------------------------------------------------------
-    // MMA issue: per 64-column chunk four MMAs (K = 16 each, +32 bytes
-    // along the 128-byte swizzled rows); the slot is released by a commit.
-    // Rows of a short last tile beyond its box hold stale data; their
-    // accumulator rows are never stored.
+    // MMA issue: per 64-column chunk four K steps (16 columns, +32 bytes along
+    // the 128-byte swizzled rows) for each 128-row half of the tile, the halves
+    // sharing the hidden-state box; the slot is released by a commit.  Rows
+    // beyond a short tile's box hold stale data; their accumulator rows are
+    // never stored.
     // ------------------------------------------------------------------
     uint32_t q = 0;
     bool ok = true;
     for (int i = 0; i < n_tiles && ok; ++i) {
-      const uint32_t buf = static_cast<uint32_t>(i) & 1u;
-      if (i >= 2) {
+      const int buf = i % p.nbuf;
+      const int halves = (i == n_tiles - 1 ? last_h : kLmTileV) > kLmHalf ? 2 : 1;
+      if (i >= p.nbuf) {
         int w = 1;
-        if (lane == 0) w = mbar_wait_or_abort(bar(DEMPTY + buf), ((i - 2) >> 1) & 1, s_abort);
+        if (lane == 0) w = mbar_wait_or_abort(bar(DEMPTY + buf), (i / p.nbuf - 1) & 1, s_abort);
         if (!__shfl_sync(0xffffffffu, w, 0)) break;
       }
       tc_fence_after_sync();
-      const uint32_t d = tmem + buf * static_cast<uint32_t>(p.NP);
+      const uint32_t d = tmem + static_cast<uint32_t>(buf * p.halves * p.NP);
       for (int kc = 0; kc < nkc; ++kc, ++q) {
         const uint32_t slot = q % S;
         int w = 1;
@@ -275,13 +374,15 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         tc_fence_after_sync();
         if (lane == 0) s_misc[3] = static_cast<int>(q + 1);
         const uint32_t wa = ring + slot * p.stage_bytes;
-        const uint32_t hb = wa + kLmWBytes;
+        const uint32_t hb = wa + p.w_bytes;
         if (elect_one()) {
+          for (int hf = 0; hf < halves; ++hf) {
 #pragma unroll
-          for (int kk = 0; kk < kLmChunkK / 16; ++kk) {
-            const uint64_t a = smem_desc_sw128(wa + kk * 32, 16, 1024);
-            const uint64_t b = smem_desc_sw128(hb + kk * 32, 16, 1024);
-            tc_mma_ss(d, a, b, p.idesc, (kc > 0 || kk > 0) ? 1u : 0u);
+            for (int kk = 0; kk < kLmChunkK / 16; ++kk) {
+              const uint64_t a = smem_desc_sw128(wa + hf * (kLmHalf * kLmChunkK * 2) + kk * 32, 16, 1024);
+              const uint64_t b = smem_desc_sw128(hb + kk * 32, 16, 1024);
+              tc_mma_ss(d + static_cast<uint32_t>(hf * p.NP), a, b, p.idesc, (kc > 0 || kk > 0) ? 1u : 0u);
+            }
           }
           tc_commit(bar(EMPTY + slot));
         }
@@ -296,85 +397,66 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     (void)mbar_wait_bounded(bar(FIN), 0);
   } else {
     // ------------------------------------------------------------------
-    // epilogue: thread = vocabulary row of the tile (TMEM lane), 16 draft
-    // rows (TMEM columns) per step.  Logits go straight to global memory;
-    // for the statistics the step is transposed through shared memory and
-    // each draft row is reduced by 8 threads (128 values / 8, interleaved).
+    // epilogue: warps 0-3 take the tile's first 128 vocabulary rows, warps
+    // 4-7 the others; 16 draft rows per step.  The last tile's epilogue is
+    // exposed: at 128 draft rows the statistics added 30 us with a 128-thread
+    // transpose and chains of float-float adds on four warps.
     // ------------------------------------------------------------------
     const bool stats = p.stats != nullptr;
-    grid_dependency_wait();  // outputs and temperatures follow the previous kernel
+    const int hf = warp >> 2;  // half of the tile
+    grid_dependency_wait();    // outputs and temperatures follow the previous kernel
     if (stats) {
-      for (int c = tid; c < p.NP; c += kLmEpiThreads) {
-        s_tau[c] = c < p.R ? p.tau[c / p.tau_div] : 1.f;
-        run[c] = SampStat{-INFINITY, INT_MAX, ff_of(0.f)};
-      }
+      for (int c = tid; c < p.NP; c += kLmEpiThreads) s_tau[c] = c < p.R ? p.tau[c / p.tau_div] : 1.f;
+      for (int c = tid; c < kLmEpiWarps * p.NP; c += kLmEpiThreads) run[c] = SampStat{-INFINITY, INT_MAX, ff_of(0.f)};
+      named_bar_sync(1, kLmEpiThreads);
     }
-    named_bar_sync(1, kLmEpiThreads);
-    const uint32_t lane_base = tmem + (static_cast<uint32_t>(32 * warp) << 16);
-    const int groups = p.NP / kLmColGroup;
-    uint32_t g_count = 0;
-    for (int i = 0; i < n_tiles; ++i) {
-      const uint32_t buf = static_cast<uint32_t>(i) & 1u;
-      bool ok = mbar_wait_or_abort(bar(DFULL + buf), (i >> 1) & 1, s_abort);
-      if (!named_bar_and(2, kLmEpiThreads, ok)) break;
+    const uint32_t lane_base = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16);
+    float *tb = tbuf + warp * kLmTBufFloats;
+    SampStat *wrun = stats ? run + warp * p.NP : nullptr;
+    for (int i = 0; i < n_tiles && hf < p.halves; ++i) {
+      const int buf = i % p.nbuf;
+      const bool ok = mbar_wait_or_abort(bar(DFULL + buf), (i / p.nbuf) & 1, s_abort);
+      if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after_sync();
-      const int vbase = v0 + i * kLmTileV;
-      const int v = vbase + 32 * warp + lane;
-      const bool vin = v < v1;
-      for (int g = 0; g < groups; ++g, ++g_count) {
-        const int c0 = g * kLmColGroup;
-        uint32_t x[16];
-        tmem_ld_32x32b_x16(lane_base + buf * static_cast<uint32_t>(p.NP) + c0, x);
-        if (vin) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (c0 + j < p.R) logits[static_cast<size_t>(c0 + j) * p.V + v] = __uint_as_float(x[j]);
-        }
-        if (!stats) continue;
-        float *tb = tbuf + (g_count & 1u) * (kLmColGroup * kLmTStride);
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-          tb[j * kLmTStride + 32 * warp + lane] = vin ? __uint_as_float(x[j]) : -INFINITY;
-        named_bar_sync(1, kLmEpiThreads);
-        const int cl = tid >> 3, part = tid & 7, r = c0 + cl;
-        const float *col = tb + cl * kLmTStride + part;
-        float bv = -INFINITY;
-        int bi = INT_MAX;
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          const float val = col[8 * e];
-          if (better(val, vbase + part + 8 * e, bv, bi)) {
-            bv = val;
-            bi = vbase + part + 8 * e;
-          }
-        }
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) {
-          const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-          const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-          if (better(ov, oi, bv, bi)) {
-            bv = ov;
-            bi = oi;
-          }
-        }
-        const float tau = s_tau[r];
-        const bool greedy = !(tau > 0.f);
-        ff s = ff_of(0.f);
-        if (!greedy) {
-#pragma unroll 4
-          for (int e = 0; e < 16; ++e) s = ff_add(s, ff_of(term_of(col[8 * e], bv, tau)));
-        }
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) s = ff_add(s, shfl_xor_ff(s, o));
-        if (part == 0) stat_merge(run[r], bv, bi, s, tau, greedy);
-      }
+      const int vbase = v0 + i * kLmTileV + 32 * warp;  // the warp's vocabulary rows
+      const bool vin = vbase + lane < v1;
+      const uint32_t acc = lane_base + static_cast<uint32_t>((buf * p.halves + hf) * p.NP);
+#pragma unroll 1
+      for (int c0 = 0; c0 < p.NP && vbase < v1; c0 += kLmColGroup)
+        lm_epilogue_step(acc + static_cast<uint32_t>(c0), logits + static_cast<size_t>(c0) * p.V, p.V, vbase, vin,
+                         p.R - c0, tb, s_tau + c0, stats ? wrun + c0 : nullptr);
       tc_fence_before_sync();
       mbar_arrive(bar(DEMPTY + buf));
     }
     if (stats) {
       named_bar_sync(1, kLmEpiThreads);
-      for (int c = tid; c < p.R; c += kLmEpiThreads)
-        p.stats[static_cast<size_t>(c) * p.G + grp] = run[c];
+      // the eight warps' statistics of a draft row, all rescaled at once
+      for (int c = tid; c < p.R; c += kLmEpiThreads) {
+        SampStat st{-INFINITY, INT_MAX, ff_of(0.f)};
+#pragma unroll
+        for (int w = 0; w < kLmEpiWarps; ++w) {
+          const SampStat o = run[w * p.NP + c];
+          if (better(o.m, o.arg, st.m, st.arg)) {
+            st.m = o.m;
+            st.arg = o.arg;
+          }
+        }
+        if (s_tau[c] > 0.f) {
+          ff t[kLmEpiWarps];
+#pragma unroll
+          for (int w = 0; w < kLmEpiWarps; ++w) {
+            const SampStat o = run[w * p.NP + c];
+            t[w] = o.m == -INFINITY || o.m == st.m ? o.S : ff_mul(o.S, exp_diff_accurate(o.m, st.m, s_tau[c]));
+          }
+#pragma unroll
+          for (int n = kLmEpiWarps / 2; n >= 1; n >>= 1) {
+#pragma unroll
+            for (int w = 0; w < n; ++w) t[w] = ff_add(t[w], t[w + n]);
+          }
+          st.S = t[0];
+        }
+        p.stats[static_cast<size_t>(c) * p.G + grp] = st;
+      }
     }
   }
 
@@ -457,108 +539,149 @@ __global__ void __launch_bounds__(kFfThreads) sample_stats_kernel(const __grid_c
 // tokens and, in the CTA holding the crossing chunk's first
 // token, draws T'.  grid (ceil(V / span), R); dynamic shared memory
 // holds the row's Cn statistics.
-__global__ void __launch_bounds__(kFfThreads) sample_finish_kernel(const __grid_constant__ SampleParams p) {
+//
+// Warp 0 of every CTA combines the statistics alone, with shuffles instead of
+// block barriers (all lanes' loads in one round trip, one barrier in all),
+// while the other warps' first logits are in flight: with a block-wide
+// combine of ten barriers a wave of CTAs spent 10 us before its first store.
+__global__ void __launch_bounds__(kFfThreads, kFinishCtasPerSm)
+sample_finish_kernel(const __grid_constant__ SampleParams p) {
   extern __shared__ SampStat s_st[];
   __shared__ ff s_scan[kFfWarps + 1];
-  __shared__ float s_v[32];
-  __shared__ int s_i[32];
-  __shared__ int s_c, s_tok, s_last;
-  __shared__ ff s_base;
+  __shared__ float s_m, s_inv;
+  __shared__ int s_arg, s_cross, s_crossed, s_tok, s_last;
+  __shared__ ff s_base, s_target;
+  constexpr int kBatch = 4;
+  constexpr unsigned kAll = 0xffffffffu;
   grid_dependency_wait();  // the statistics and logits come from the previous kernels
   grid_launch_dependents();
   const int r = blockIdx.y, tid = threadIdx.x;
   const float *row = p.logits + static_cast<size_t>(r) * p.V;
   float *prow = p.probs + static_cast<size_t>(r) * p.V;
-  const SampStat *st = p.stats + static_cast<size_t>(r) * p.Cn;
-  for (int c = tid; c < p.Cn; c += kFfThreads) s_st[c] = st[c];
-  if (tid == 0) {
-    s_c = INT_MAX;
-    s_tok = INT_MAX;
-    s_last = -1;
-  }
-  __syncthreads();
-
-  // row maximum and its first index
-  float m = -INFINITY;
-  int arg = INT_MAX;
-  for (int c = tid; c < p.Cn; c += kFfThreads)
-    if (better(s_st[c].m, s_st[c].arg, m, arg)) {
-      m = s_st[c].m;
-      arg = s_st[c].arg;
-    }
-  block_argmax(m, arg, s_v, s_i);
-
   const float tau = p.tau[r];
+  const bool greedy = !(tau > 0.f);
   const int x0 = blockIdx.x * p.span;
   const int x1 = min(p.V, x0 + p.span);
-  if (!(tau > 0.f)) {
-    // greedy: one-hot P', T' = the first argmax
+  float4 f[kBatch];  // the vector path's first tokens
+  if (p.vec4 && !greedy) {
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) {
+      const int x = x0 + 4 * tid + j * 4 * kFfThreads;
+      if (x < x1) f[j] = __ldcs(reinterpret_cast<const float4 *>(row + x));
+    }
+  }
+  if (tid < 32) {
+    const int lane = tid;
+    const SampStat *st = p.stats + static_cast<size_t>(r) * p.Cn;
+#pragma unroll 4
+    for (int c = lane; c < p.Cn; c += 32) s_st[c] = st[c];
+    __syncwarp();
+    // lane l owns chunks [c_lo, c_hi), in order
+    const int c_lo = lane * p.Cn / 32, c_hi = (lane + 1) * p.Cn / 32;
+    // row maximum and its first index
+    float m = -INFINITY;
+    int arg = INT_MAX;
+    for (int c = c_lo; c < c_hi; ++c)
+      if (better(s_st[c].m, s_st[c].arg, m, arg)) {
+        m = s_st[c].m;
+        arg = s_st[c].arg;
+      }
+    warp_argmax(m, arg);
+    if (!greedy) {
+      // chunk masses relative to m, and their prefix over the lanes: excl of a
+      // lane is, bit for bit, incl of the lane before
+      ff incl = ff_of(0.f);
+      for (int c = c_lo; c < c_hi; ++c) {
+        const ff w = s_st[c].m == -INFINITY ? ff_of(0.f) : ff_mul(s_st[c].S, term_of(s_st[c].m, m, tau));
+        s_st[c].S = w;
+        incl = ff_add(incl, w);
+      }
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const ff n = shfl_up_ff(incl, o);
+        if (lane >= o) incl = ff_add(n, incl);
+      }
+      const ff prev = shfl_up_ff(incl, 1);
+      const ff total = ff{__shfl_sync(kAll, incl.hi, 31), __shfl_sync(kAll, incl.lo, 31)};
+      const ff target = ff_mul(total, p.u[r]);
+      // the first chunk whose inclusive prefix exceeds the target
+      ff cum = lane > 0 ? prev : ff_of(0.f);
+      ff base = cum;
+      int cand = INT_MAX, lastpos = -1;
+      for (int c = c_lo; c < c_hi; ++c) {
+        const ff w = s_st[c].S;
+        const ff nxt = ff_add(cum, w);
+        if (ff_pos(w)) lastpos = c;
+        if (cand == INT_MAX && ff_lt(target, nxt)) {
+          cand = c;
+          base = cum;
+        }
+        cum = nxt;
+      }
+      const unsigned any = __ballot_sync(kAll, cand != INT_MAX);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) lastpos = max(lastpos, __shfl_xor_sync(kAll, lastpos, o));
+      if (lane == (any ? __ffs(any) - 1 : 0)) {
+        s_crossed = any != 0u;
+        s_cross = any ? cand : lastpos;  // no crossing (u >= 1 or NaN): last positive chunk
+        s_base = base;
+        s_target = target;
+        s_inv = ff_div_to_f(1.f, total);
+      }
+    }
+    if (lane == 0) {
+      s_m = m;
+      s_arg = arg;
+      s_tok = INT_MAX;
+      s_last = -1;
+    }
+  }
+  __syncthreads();
+  if (greedy) {
+    // one-hot P', T' = the first argmax
+    const int arg = s_arg;
     for (int x = x0 + tid; x < x1; x += kFfThreads) prow[x] = x == arg ? 1.f : 0.f;
     if (tid == 0 && arg >= x0 && arg < x1) p.tokens[r] = arg;
     return;
   }
-
-  // chunk masses relative to m; thread t sums chunks [c_lo, c_hi) in order
-  const int c_lo = static_cast<int>(static_cast<long long>(tid) * p.Cn / kFfThreads);
-  const int c_hi = static_cast<int>(static_cast<long long>(tid + 1) * p.Cn / kFfThreads);
-  auto mass = [&](int c) -> ff {
-    return s_st[c].m == -INFINITY ? ff_of(0.f)
-                                  : ff_mul(s_st[c].S, term_of(s_st[c].m, m, tau));
-  };
-  ff mine = ff_of(0.f);
-  for (int c = c_lo; c < c_hi; ++c) mine = ff_add(mine, mass(c));
-  ff excl, Stot;
-  block_inclusive_scan(mine, s_scan, &excl, &Stot);
-  const ff target = ff_mul(Stot, p.u[r]);
-  // the first chunk whose inclusive prefix exceeds the target
-  {
-    ff cum = excl;
-    int cand = INT_MAX, lastpos = -1;
-    ff cand_base = ff_of(0.f);
-    for (int c = c_lo; c < c_hi; ++c) {
-      const ff w = mass(c);
-      const ff nxt = ff_add(cum, w);
-      if (ff_pos(w)) lastpos = c;
-      if (cand == INT_MAX && ff_lt(target, nxt)) {
-        cand = c;
-        cand_base = cum;
-      }
-      cum = nxt;
-    }
-    if (cand != INT_MAX) atomicMin(&s_c, cand);
-    if (lastpos >= 0) atomicMax(&s_last, lastpos);
-    __syncthreads();
-    if (cand != INT_MAX && cand == s_c) s_base = cand_base;
-    __syncthreads();
-  }
-  const bool crossed = s_c != INT_MAX;
-  const int cs = crossed ? s_c : s_last;  // no crossing (u >= 1 or NaN): last positive chunk
+  const float m = s_m;
+  const ff target = s_target;
+  const bool crossed = s_crossed != 0;
+  const int cs = s_cross;
 
   // P' for this CTA's span.  Rows are 16-byte aligned and the span a
   // multiple of 4 in the vector path, so a float4 is either wholly inside
-  // the span or wholly outside; each thread issues kBatch loads before
-  // the arithmetic and stores that depend on them.
-  const float invS = ff_div_to_f(1.f, Stot);
+  // the span or wholly outside; each thread issues the next kBatch loads
+  // before the arithmetic and stores of the current ones.
+  const float invS = s_inv;
   if (p.vec4) {
-    constexpr int kBatch = 4;
-    for (int base = x0 + 4 * tid; base < x1; base += 4 * kFfThreads * kBatch) {
-      float4 f[kBatch];
+    constexpr int kStep = 4 * kFfThreads * kBatch;
+    for (int base = x0 + 4 * tid; base < x1; base += kStep) {
+      float4 g[kBatch];
 #pragma unroll
       for (int j = 0; j < kBatch; ++j) {
-        const int x = base + j * 4 * kFfThreads;
-        if (x < x1) f[j] = __ldcs(reinterpret_cast<const float4 *>(row + x));
+        const int x = base + kStep + j * 4 * kFfThreads;
+        if (x < x1) g[j] = __ldcs(reinterpret_cast<const float4 *>(row + x));
       }
 #pragma unroll
       for (int j = 0; j < kBatch; ++j) {
         const int x = base + j * 4 * kFfThreads;
         if (x < x1) {
           float4 o;
-          o.x = __fmul_rn(term_of(f[j].x, m, tau), invS);
-          o.y = __fmul_rn(term_of(f[j].y, m, tau), invS);
-          o.z = __fmul_rn(term_of(f[j].z, m, tau), invS);
-          o.w = __fmul_rn(term_of(f[j].w, m, tau), invS);
+          if (tau == 1.f) {  // constant, so that the divisions are branched over once
+            o.x = __fmul_rn(term_of(f[j].x, m, 1.f), invS);
+            o.y = __fmul_rn(term_of(f[j].y, m, 1.f), invS);
+            o.z = __fmul_rn(term_of(f[j].z, m, 1.f), invS);
+            o.w = __fmul_rn(term_of(f[j].w, m, 1.f), invS);
+          } else {
+            o.x = __fmul_rn(term_of(f[j].x, m, tau), invS);
+            o.y = __fmul_rn(term_of(f[j].y, m, tau), invS);
+            o.z = __fmul_rn(term_of(f[j].z, m, tau), invS);
+            o.w = __fmul_rn(term_of(f[j].w, m, tau), invS);
+          }
           *reinterpret_cast<float4 *>(prow + x) = o;
         }
+        f[j] = g[j];
       }
     }
   } else {
@@ -571,9 +694,6 @@ __global__ void __launch_bounds__(kFfThreads) sample_finish_kernel(const __grid_
   if (e0 < x0 || e0 >= x1) return;
 
   // scan the chunk in ascending order, 4 consecutive tokens per thread
-  __syncthreads();
-  if (tid == 0) s_last = -1;
-  __syncthreads();
   ff base = s_base;
   int lastpos = -1;
   for (int s0 = e0; s0 < e1; s0 += 4 * kFfThreads) {
@@ -613,6 +733,8 @@ __global__ void __launch_bounds__(kFfThreads) sample_finish_kernel(const __grid_
 // ---------------------------------------------------------------------------
 static int np_of(int R) { return (R + 15) / 16 * 16; }
 
+// As many slots as fit: the weight stream needs ~200 KB in flight per SM
+// (152064 x 3584, 128 draft rows: 183 us with four 48 KB slots, 196 with three).
 static int lm_stages(const DeviceInfo &dev, uint32_t stage_bytes, int NP) {
   int s = kLmMaxStages;
   while (s > 2 && LmSmem::bytes(s, stage_bytes, NP) > static_cast<size_t>(dev.max_smem_optin)) --s;
@@ -727,16 +849,20 @@ static int launch_lm_head(const void *hidden, const void *weight, int R, int hid
   prm.R = R;
   prm.V = V;
   prm.NP = NP;
-  const int tiles = (V + kLmTileV - 1) / kLmTileV;
-  prm.G = tiles < dev.sm_count ? tiles : dev.sm_count;
+  prm.G = projection_groups(V, dev.sm_count);
   const int q = V / prm.G;  // every CTA owns q or q + 1 rows
+  const int tallest = q + (V % prm.G ? 1 : 0) < kLmTileV ? q + (V % prm.G ? 1 : 0) : kLmTileV;
+  prm.halves = tallest > kLmHalf ? 2 : 1;
+  prm.w_bytes = static_cast<uint32_t>((tallest + 7) / 8 * 8) * (kLmChunkK * 2);
   prm.ha = (q - 1) % kLmTileV + 1;
   prm.hb = q % kLmTileV + 1;
   prm.KC = (hidden_size + kLmChunkK - 1) / kLmChunkK;
-  prm.stage_bytes = kLmWBytes + static_cast<uint32_t>(NP) * 128u;
+  prm.stage_bytes = prm.w_bytes + static_cast<uint32_t>(NP) * 128u;
   prm.stages = lm_stages(dev, prm.stage_bytes, NP);
+  const uint32_t acc = static_cast<uint32_t>(prm.halves * NP);  // columns of one tile's accumulators
+  prm.nbuf = 2 * acc <= 512 ? 2 : 1;
   uint32_t cols = 32;
-  while (cols < 2u * static_cast<uint32_t>(NP)) cols <<= 1;
+  while (cols < static_cast<uint32_t>(prm.nbuf) * acc) cols <<= 1;
   prm.tmem_cols = cols;
   prm.idesc = idesc_bf16_f32(128, NP, 0, 0);
   prm.w_after_wait = w_after_wait ? 1 : 0;
@@ -765,21 +891,22 @@ static int launch_lm_head(const void *hidden, const void *weight, int R, int hid
   return SF_OK;
 }
 
-// Span per finishing CTA: about one wave of CTAs (8 per SM) over all rows,
-// at least kSampleSpan tokens, a multiple of kSampleSpan.
-static int finish_span(int R, int V) {
-  DeviceInfo dev;
-  const int sms = current_device(&dev) == SF_OK ? dev.sm_count : 148;
-  const long long per = ((long long)R * V + 8LL * sms - 1) / (8LL * sms);
-  long long span = (per + kSampleSpan - 1) / kSampleSpan * kSampleSpan;
-  if (span < kSampleSpan) span = kSampleSpan;
-  if (span > V) span = (V + 3) / 4 * 4;
-  return static_cast<int>(span);
+// Span per finishing CTA: the CTAs of all rows fit the GPU at once (a second,
+// nearly empty wave cost 128 rows of 152064 tokens a third of the kernel),
+// at least kSampleSpan tokens each, a multiple of kSampleSpan.
+static int finish_span(int R, int V, int sm_count) {
+  const long long slots = static_cast<long long>(kFinishCtasPerSm) * sm_count;
+  const long long spans = slots / R > 1 ? slots / R : 1;
+  const long long span = ((V + spans - 1) / spans + kSampleSpan - 1) / kSampleSpan * kSampleSpan;
+  return static_cast<int>(span < V ? span : (V + 3) / 4 * 4);
 }
 
 static int launch_finish(SampleParams prm, cudaStream_t stream) {
   cudaLaunchAttribute attr[1];
-  prm.span = finish_span(prm.R, prm.V);
+  DeviceInfo dev;
+  const int st = current_device(&dev);
+  if (st != SF_OK) return st;
+  prm.span = finish_span(prm.R, prm.V, dev.sm_count);
   const int spans = (prm.V + prm.span - 1) / prm.span;
   cudaLaunchConfig_t cfg = pdl_config(dim3(spans, prm.R), dim3(kFfThreads),
                                       static_cast<size_t>(prm.Cn) * sizeof(SampStat), stream, attr);
@@ -798,13 +925,12 @@ int launch_projection_stats(const void *hidden, const void *weight, int R, int h
 }
 
 int projection_groups(int V, int sm_count) {
-  const int tiles = (V + kLmTileV - 1) / kLmTileV;
-  return tiles < sm_count ? tiles : sm_count;
+  const int g = (V + kLmHalf - 1) / kLmHalf;
+  return g < sm_count ? g : sm_count;
 }
 
 int projection_splits(int V, int hidden_size, int sm_count) {
-  const int tiles = (V + kLmTileV - 1) / kLmTileV;
-  const int G = tiles < sm_count ? tiles : sm_count;
+  const int G = projection_groups(V, sm_count);
   const int KC = (hidden_size + kLmChunkK - 1) / kLmChunkK;
   int ks = sm_count / G;
   if (ks > KC) ks = KC;

@@ -38,6 +38,13 @@ __device__ __forceinline__ bool better(float v, int i, float bv, int bi) {
 // explicit _rn intrinsics keep the compiler from contracting or reordering.
 __device__ __forceinline__ ff ff_of(float x) { return ff{x, 0.f}; }
 
+// a + b exactly, as a float-float number.
+__device__ __forceinline__ ff two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b);
+  const float v = __fsub_rn(s, a);
+  return ff{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v))};
+}
+
 __device__ __forceinline__ ff ff_add(ff a, ff b) {
   const float s = __fadd_rn(a.hi, b.hi);
   const float v = __fsub_rn(s, a.hi);

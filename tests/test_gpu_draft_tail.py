@@ -115,6 +115,27 @@ def test_lm_head_exact_on_small_integer_inputs(oracle_mod, R, Hd, V):
                           oracle_mod.lm_head_logits(case.hidden, case.weight))
 
 
+@pytest.mark.parametrize("R,rows,extra", [
+    (16, 128, 0),     # one full half tile per CTA
+    (5, 128, 1),      # one CTA with a second half of one row
+    (33, 256, 0),     # one full tile per CTA (NP = 48)
+    (128, 256, 3),    # a last tile of one row in some CTAs; double-buffered accumulators
+    (129, 300, 7),    # NP = 144: a single accumulator buffer
+    (256, 513, 5),    # three tiles, single-buffered, the largest N
+])
+def test_projection_and_sampling_at_tile_edges(oracle_mod, R, rows, extra):
+    """Vocabulary sizes at which the CTAs' row ranges (V / SM count) meet the
+    edges of the 128-row halves and 256-row tiles, with the statistics of
+    every range: logits exact, samples as in check_sampler."""
+    V = rows * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    tau = np.where(np.arange(R) % 3 == 1, 0.0, np.where(np.arange(R) % 3 == 2, 0.6, 1.0)).astype(np.float32)
+    case = make_draft_tail_case(R, 72, V, seed=[R, rows, extra], temperature=tau, exact=True)
+    logits, probs, tokens = run_fused(case)
+    assert np.array_equal(logits.astype(np.float64), oracle_mod.lm_head_logits(case.hidden, case.weight))
+    some = np.unique(np.linspace(0, R - 1, 12).astype(int))
+    check_sampler(oracle_mod, logits[some], case.uniforms[some], tau[some], probs[some], tokens[some])
+
+
 def test_lm_head_is_deterministic():
     case = make_draft_tail_case(40, 1024, 9000, seed=7)
     h, w = bf16_tensor(case.hidden), bf16_tensor(case.weight)
