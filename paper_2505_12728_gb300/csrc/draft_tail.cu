@@ -250,7 +250,7 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
   const int FULL = 0, EMPTY = S, DFULL = 2 * S, DEMPTY = 2 * S + 2, FIN = 2 * S + 4;
   auto bar = [&](int i) -> uint32_t { return bars + 8u * static_cast<uint32_t>(i); };
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp_id(), lane = tid & 31;
   const int grp = static_cast<int>(blockIdx.x) % p.G, split = static_cast<int>(blockIdx.x) / p.G;
   const int v0 = static_cast<int>(static_cast<long long>(grp) * p.V / p.G);
   const int v1 = static_cast<int>(static_cast<long long>(grp + 1) * p.V / p.G);
@@ -307,41 +307,59 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
   }
 
   if (warp == kLmProducerWarp) {
-    if (lane == 0) {
-      const uint64_t pol_w = p.w_keep ? l2_policy_evict_last() : l2_policy_evict_first();
-      const uint64_t pol_h = l2_policy_evict_last();
-      const uint32_t prime = total < static_cast<uint32_t>(S) ? total : static_cast<uint32_t>(S);
-      // the first ring fill: weights before the dependency wait (unless
-      // they may come from the previous kernel), hidden states after it
-      if (p.w_after_wait) grid_dependency_wait();
-      for (uint32_t q = 0; q < prime; ++q) {
-        const int i = static_cast<int>(q) / nkc, kc = kc0 + static_cast<int>(q) % nkc;
-        uint32_t bytes;
-        const CUtensorMap *mw = tile_map(i, bytes);
+    // The whole warp runs the loop and an elected lane issues, so that the
+    // copies' operands are warp-uniform (see smem_desc_sw128).
+    const uint64_t pol_w = p.w_keep ? l2_policy_evict_last() : l2_policy_evict_first();
+    const uint64_t pol_h = l2_policy_evict_last();
+    const int prime = total < static_cast<uint32_t>(S) ? static_cast<int>(total) : S;
+    int i = 0, kc = 0;  // tile and hidden chunk of the next slot
+    auto next = [&]() {
+      if (++kc == nkc) {
+        kc = 0;
+        ++i;
+      }
+    };
+    // the first ring fill: weights before the dependency wait (unless
+    // they may come from the previous kernel), hidden states after it
+    if (p.w_after_wait) grid_dependency_wait();
+    for (int q = 0; q < prime; ++q, next()) {
+      uint32_t bytes;
+      const CUtensorMap *mw = tile_map(i, bytes);
+      if (elect_one()) {
         mbar_arrive_expect_tx(bar(FULL + q), bytes);
-        tma_load_2d(ring + q * p.stage_bytes, mw, kc * kLmChunkK, v0 + i * kLmTileV, bar(FULL + q),
-                    pol_w);
+        tma_load_2d(ring + static_cast<uint32_t>(q) * p.stage_bytes, mw, (kc0 + kc) * kLmChunkK, v0 + i * kLmTileV,
+                    bar(FULL + q), pol_w);
       }
-      if (!p.w_after_wait) grid_dependency_wait();
-      for (uint32_t q = 0; q < prime; ++q) {
-        const int kc = kc0 + static_cast<int>(q) % nkc;
-        tma_load_2d(ring + q * p.stage_bytes + p.w_bytes, &tmap_h, kc * kLmChunkK, 0, bar(FULL + q),
-                    pol_h);
-      }
-      uint32_t q = prime;
-      for (; q < total; ++q) {
-        const uint32_t slot = q % S;
-        if (!mbar_wait_or_abort(bar(EMPTY + slot), ((q / S) - 1) & 1u, s_abort)) break;
-        const int i = static_cast<int>(q) / nkc, kc = kc0 + static_cast<int>(q) % nkc;
-        const uint32_t dst = ring + slot * p.stage_bytes;
-        uint32_t bytes;
-        const CUtensorMap *mw = tile_map(i, bytes);
-        mbar_arrive_expect_tx(bar(FULL + slot), bytes);
-        tma_load_2d(dst, mw, kc * kLmChunkK, v0 + i * kLmTileV, bar(FULL + slot), pol_w);
-        tma_load_2d(dst + p.w_bytes, &tmap_h, kc * kLmChunkK, 0, bar(FULL + slot), pol_h);
-      }
-      s_misc[2] = static_cast<int>(q);
+      __syncwarp();
     }
+    if (!p.w_after_wait) grid_dependency_wait();
+    for (int q = 0, hc = 0; q < prime; ++q) {
+      if (elect_one())
+        tma_load_2d(ring + static_cast<uint32_t>(q) * p.stage_bytes + p.w_bytes, &tmap_h, (kc0 + hc) * kLmChunkK, 0,
+                    bar(FULL + q), pol_h);
+      __syncwarp();
+      if (++hc == nkc) hc = 0;
+    }
+    uint32_t q = static_cast<uint32_t>(prime), lap = 0;  // earlier passes over the ring
+    int slot = 0;
+    for (; q < total; ++q, next()) {
+      const bool w = mbar_wait_or_abort(bar(EMPTY + slot), lap & 1u, s_abort);
+      if (!__all_sync(0xffffffffu, w)) break;
+      const uint32_t dst = ring + static_cast<uint32_t>(slot) * p.stage_bytes;
+      uint32_t bytes;
+      const CUtensorMap *mw = tile_map(i, bytes);
+      if (elect_one()) {
+        mbar_arrive_expect_tx(bar(FULL + slot), bytes);
+        tma_load_2d(dst, mw, (kc0 + kc) * kLmChunkK, v0 + i * kLmTileV, bar(FULL + slot), pol_w);
+        tma_load_2d(dst + p.w_bytes, &tmap_h, (kc0 + kc) * kLmChunkK, 0, bar(FULL + slot), pol_h);
+      }
+      __syncwarp();
+      if (++slot == S) {
+        slot = 0;
+        ++lap;
+      }
+    }
+    if (lane == 0) s_misc[2] = static_cast<int>(q);
     __syncwarp();
   } else if (warp == kLmMmaWarp) {
     // ------------------------------------------------------------------
@@ -351,7 +369,8 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     // beyond a short tile's box hold stale data; their accumulator rows are
     // never stored.
     // ------------------------------------------------------------------
-    uint32_t q = 0;
+    uint32_t q = 0, lap = 0;
+    int slot = 0;
     bool ok = true;
     for (int i = 0; i < n_tiles && ok; ++i) {
       const int buf = i % p.nbuf;
@@ -364,29 +383,32 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
       tc_fence_after_sync();
       const uint32_t d = tmem + static_cast<uint32_t>(buf * p.halves * p.NP);
       for (int kc = 0; kc < nkc; ++kc, ++q) {
-        const uint32_t slot = q % S;
-        int w = 1;
-        if (lane == 0) w = mbar_wait_or_abort(bar(FULL + slot), (q / S) & 1u, s_abort);
-        if (!__shfl_sync(0xffffffffu, w, 0)) {
+        const bool w = mbar_wait_or_abort(bar(FULL + slot), lap & 1u, s_abort);
+        if (!__all_sync(0xffffffffu, w)) {
           ok = false;
           break;
         }
         tc_fence_after_sync();
         if (lane == 0) s_misc[3] = static_cast<int>(q + 1);
-        const uint32_t wa = ring + slot * p.stage_bytes;
-        const uint32_t hb = wa + p.w_bytes;
+        const uint32_t wa = ring + static_cast<uint32_t>(slot) * p.stage_bytes;
+        const uint64_t a0 = smem_desc_sw128(wa, 16, 1024), b0 = smem_desc_sw128(wa + p.w_bytes, 16, 1024);
+        const uint32_t acc = kc > 0 ? 1u : 0u;
         if (elect_one()) {
-          for (int hf = 0; hf < halves; ++hf) {
 #pragma unroll
-            for (int kk = 0; kk < kLmChunkK / 16; ++kk) {
-              const uint64_t a = smem_desc_sw128(wa + hf * (kLmHalf * kLmChunkK * 2) + kk * 32, 16, 1024);
-              const uint64_t b = smem_desc_sw128(hb + kk * 32, 16, 1024);
-              tc_mma_ss(d + static_cast<uint32_t>(hf * p.NP), a, b, p.idesc, (kc > 0 || kk > 0) ? 1u : 0u);
-            }
+          for (int kk = 0; kk < kLmChunkK / 16; ++kk) tc_mma_ss(d, a0 + 2 * kk, b0 + 2 * kk, p.idesc, kk > 0 ? 1u : acc);
+          if (halves > 1) {
+#pragma unroll
+            for (int kk = 0; kk < kLmChunkK / 16; ++kk)
+              tc_mma_ss(d + static_cast<uint32_t>(p.NP), a0 + (kLmHalf * kLmChunkK * 2 >> 4) + 2 * kk, b0 + 2 * kk,
+                        p.idesc, kk > 0 ? 1u : acc);
           }
           tc_commit(bar(EMPTY + slot));
         }
         __syncwarp();
+        if (++slot == S) {
+          slot = 0;
+          ++lap;
+        }
       }
       if (!ok) break;
       if (elect_one()) tc_commit(bar(DFULL + buf));

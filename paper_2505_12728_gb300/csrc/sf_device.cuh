@@ -197,6 +197,15 @@ __device__ __forceinline__ void cluster_sync() {
                "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// The two halves of a cluster barrier phase, for a phase that opens early and
+// closes later (every thread of every CTA of the cluster arrives, then waits).
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // Loads from the shared memory of CTA `rank` of the cluster, at the address
 // that `local` has in this CTA's shared memory (distributed shared memory).
 __device__ __forceinline__ uint32_t dsmem_addr(uint32_t local, uint32_t rank) {
@@ -231,6 +240,24 @@ __device__ __forceinline__ void st_dsmem_f32x2(uint32_t remote, float a, float b
                : "memory");
 }
 
+__device__ __forceinline__ void st_dsmem_u32(uint32_t remote, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
+}
+
+// Arrival on an mbarrier of another CTA of the cluster (an address obtained
+// with dsmem_addr), releasing this thread's earlier writes, and those ordered
+// before it by a CTA barrier, at cluster scope; mbar_wait_or_abort_cluster
+// acquires them.
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t remote) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
+}
+
+// Orders this thread's generic accesses to shared memory, of any CTA of the
+// cluster, with later accesses through the async proxy (tcgen05, TMA).
+__device__ __forceinline__ void fence_proxy_async() {
+  asm volatile("fence.proxy.async;" ::: "memory");
+}
+
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -246,6 +273,36 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint32_t bar, uint32_t parity
 #pragma unroll 1
     for (int i = 0; i < 64; ++i)
       if (mbar_try_wait(bar, parity)) return true;
+    if (*abort_word) return false;
+    if (global_timer_ns() - t0 > kWaitBudgetNs) {
+      *abort_word = 1;
+      return false;
+    }
+  }
+}
+
+// The same with cluster-scope acquire, for barriers that other CTAs of the
+// cluster arrive on.
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+__device__ __forceinline__ bool mbar_wait_or_abort_cluster(uint32_t bar, uint32_t parity,
+                                                           volatile int *abort_word) {
+  if (mbar_try_wait_cluster(bar, parity)) return true;
+  const unsigned long long t0 = global_timer_ns();
+  while (true) {
+#pragma unroll 1
+    for (int i = 0; i < 64; ++i)
+      if (mbar_try_wait_cluster(bar, parity)) return true;
     if (*abort_word) return false;
     if (global_timer_ns() - t0 > kWaitBudgetNs) {
       *abort_word = 1;
@@ -287,18 +344,24 @@ __device__ __forceinline__ void tc_fence_after_sync() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// Shared-memory matrix descriptor (tcgen05 format): start address, leading-
-// and stride-dimension byte offsets (all >> 4), descriptor version 1 at bit
-// 46, base offset 0 (every swizzle atom is 1024-byte aligned), 128-byte
-// swizzle (layout type 2 at bits 61..63).
+// Shared-memory matrix descriptor (tcgen05 format): start address (its low 18
+// bits: in a cluster the address carries the CTA's rank above them), leading-
+// and stride-dimension byte offsets (all >> 4), descriptor version 1 at bit 46, base offset 0 (every swizzle atom is 1024-byte aligned), 128-byte
+// swizzle (layout type 2 at bits 61..63).  Adding bytes >> 4 to a descriptor
+// moves its start address: code that issues several MMAs makes one
+// descriptor per operand outside the elected thread's branch, where it is
+// warp-uniform, and adds compile-time offsets (40-49 cycles per M128 MMA;
+// descriptors made inside a loop of that branch took 150-360).
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((addr & 0x3FFFFu) >> 4);
-  d |= static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16;
-  d |= static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32;
-  d |= static_cast<uint64_t>(1) << 46;
-  d |= static_cast<uint64_t>(2) << 61;
-  return d;
+  return static_cast<uint64_t>((addr & 0x3FFFFu) >> 4) | static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16 |
+         static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32 | static_cast<uint64_t>(1) << 46 |
+         static_cast<uint64_t>(2) << 61;
+}
+
+// The thread's warp as a value the compiler knows to be warp-uniform, so that
+// the operands of a warp's role can live in uniform registers.
+__device__ __forceinline__ int uniform_warp_id() {
+  return __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
 }
 
 // Instruction descriptor of kind::f16: bf16 A and B, fp32 accumulator,
