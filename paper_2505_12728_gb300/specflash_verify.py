@@ -54,6 +54,8 @@ def library_path() -> str:
 def load_library(path: str | None = None):
     """Load (once) the compiled library; raises if it has not been built."""
     global _lib
+    if _lib is not None:  # the lock guards the loading only
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -124,13 +126,24 @@ def _check(status: int):
                               f"{lib.sf_last_error().decode()}")
 
 
+# The marshalling of a call is host time that a small call waits for (17
+# tensors and two calls for one layer and its acceptance): pointers go to ctypes
+# as integers, the current stream is read without building a Stream object
+# (2.8 us a call), and a tensor that is as it should be takes one expression.
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream_handle(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(_device())
+    return torch.cuda.current_stream().cuda_stream
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
 
 
 def _need_workspace(workspace):
@@ -140,6 +153,9 @@ def _need_workspace(workspace):
 
 
 def _need(t, name, dtype, shape=None):
+    if (type(t) is torch.Tensor and t.dtype is dtype and t.is_cuda and t.is_contiguous()
+            and (shape is None or t.shape == shape)):
+        return
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.dtype != dtype:
