@@ -24,12 +24,18 @@
 //     unnormalised weights exp(s - max) rounded to bf16 into P [C][F][Np]
 //     (Np = N rounded up to 64, zeros past N) and the sum of the rounded
 //     weights into l [F][C];
-//  3. compress_apply_kernel, one CTA per (128 output columns, frame): the
-//     transposed product O^T = F_V^T P^T as a pipelined tcgen05 GEMM with
-//     M = 128 feature columns (A = the frame's features, MN-major, two
-//     64-column boxes per 64 tokens), N = C padded to 16 (B = P, K-major) and
-//     K = 64 tokens per ring slot, the accumulator in tensor memory; warps 0-3
-//     (lane = feature column) divide by l and store bf16, coalesced along d.
+//  3. compress_apply_kernel, up to two CTAs per SM, each with some of a frame's
+//     groups of 128 columns: the transposed product O^T = F_V^T P^T as a
+//     pipelined tcgen05 GEMM with M = 128 feature columns (A = the frame's
+//     features, MN-major), N = C padded to 16 (B = P, K-major) and K = 16
+//     tokens, two accumulators in tensor memory.
+// Measured per call (graph of calls over three inputs): 5 x 576 x 4096, C 64:
+// 24.2 -> 17.4 us; 128 x 144 x 3584, C 16: 55.9 -> 47 us; 1 x 576 x 4096:
+// 37.3 -> 14.9 us.  A single launch with a cluster per frame, the scores
+// exchanged through distributed shared memory, was slower (31.7 and 48.9 us):
+// a CTA's 147 KB of partial scores and 74 KB of weights move at ~13 bytes per
+// clock.  Computing the weights in the third kernel instead of the second:
+// 46.1 us for the video shape, 66.6 for the images.
 // N is at most 768 and C at most 128.  Every wait is bounded
 // (SF_DEVICE_TIMEOUT).
 #include <cmath>
@@ -40,16 +46,17 @@
 
 namespace sf {
 
-constexpr int kVcThreads = 192;
-constexpr int kVcMmaWarp = 4;
-constexpr int kVcProducerWarp = 5;
-constexpr int kVcCols = 128;        // output columns per CTA (MMA M)
-constexpr int kVcTokens = 64;       // tokens per ring slot (K)
+constexpr int kVcThreads = 320;
+constexpr int kVcEpiThreads = 256;  // two warps per lane quarter of tensor memory
+constexpr int kVcMmaWarp = 8;
+constexpr int kVcProducerWarp = 9;
+constexpr int kVcCols = 128;        // feature columns per group (MMA M)
+constexpr int kVcTokens = 64;       // tokens per box of weights (128 bytes)
 constexpr int kVcMaxTokens = 768;   // N
 constexpr int kVcMaxQueries = 128;  // C
-constexpr int kVcMaxStages = 4;
-constexpr uint32_t kVcFBytes = 2 * kVcTokens * 128;  // 64 tokens x 128 columns of features
-constexpr int kVcSoftmaxWarps = 8;
+constexpr int kVcMaxStages = 8;
+constexpr int kVcMaxSplits = 4;      // partial scores that the softmax adds
+constexpr int kVcSoftmaxWarps = 2;
 
 struct VcSoftmaxParams {
   const float *scores;  // [ks][C][F*N]
@@ -64,58 +71,79 @@ struct VcParams {
   __nv_bfloat16 *out;   // [F][C][d]
   uint32_t *status;
   int F, N, C, Cp, d, Np;
-  int KT;               // Np / 64 ring slots per CTA
+  int groups, per_frame;  // d / 128 column groups, split over per_frame CTAs
+  int T, slots;           // tokens per ring slot (a multiple of 16), slots per group
   int stages;
-  uint32_t stage_bytes;
+  uint32_t stage_bytes;   // 2 x T x 128 bytes of features, then T / 64 boxes of weights
   uint32_t tmem_cols;
 };
 
 static size_t vc_smem_bytes(int stages, uint32_t stage_bytes, int C) {
-  return 1024 + static_cast<size_t>(stages) * stage_bytes + 8 * (2 * stages + 1) + 64 + 4 * C;
+  return 1024 + static_cast<size_t>(stages) * stage_bytes + 8 * (2 * stages + 5) + 64 + 4 * C;
 }
 
-// grid (F, ceil(C / 8)), 256 threads: warp w handles query 8 * blockIdx.y + w
-// of frame blockIdx.x.
+// grid (F, ceil(C / 2)), 64 threads, one warp per query: the partial scores
+// summed in split order, then the unnormalised weights exp(s - max) rounded to
+// bf16, two tokens (64 i + 2 lane and the next) at a time, zeros past N.
+// Bound by memory round trips: every load of the row is in flight at once
+// (loads of one partial behind the sums of the one before: 17.6 us alone for
+// 5 x 576 x 4096, C 64, against 6.5), so there are at most kVcMaxSplits
+// partials; with up to 30 per score a single image took 31 us instead of 15.
 __global__ void __launch_bounds__(32 * kVcSoftmaxWarps)
 compress_softmax_kernel(const __grid_constant__ VcSoftmaxParams p) {
-  constexpr int kPer = kVcMaxTokens / 32;  // scores per lane
+  constexpr int kPairs = kVcMaxTokens / 64, kFly = kVcMaxSplits - 1;
   grid_dependency_wait();  // the partial scores come from the projection
   grid_launch_dependents();
   const int f = blockIdx.x, c = blockIdx.y * kVcSoftmaxWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (c >= p.C) return;
-  const long long row = static_cast<long long>(c) * p.F * p.N + static_cast<long long>(f) * p.N;
-  float x[kPer];
+  const float *row = p.scores + static_cast<long long>(c) * p.F * p.N + static_cast<long long>(f) * p.N;
+  float x[kPairs], y[kPairs];
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    const int n = lane + 32 * i;
-    x[i] = n < p.N ? __ldg(p.scores + row + n) : -INFINITY;
+  for (int i = 0; i < kPairs; ++i) {
+    const int n = 64 * i + 2 * lane;
+    x[i] = n < p.N ? __ldg(row + n) : -INFINITY;
+    y[i] = n + 1 < p.N ? __ldg(row + n + 1) : -INFINITY;
   }
-  // the other hidden-range partials, added in split order
-  for (int s = 1; s < p.ks; ++s) {
-    const float *part = p.scores + s * p.part_stride + row;
+  for (int s0 = 1; s0 < p.ks; s0 += kFly) {
+    float vx[kFly][kPairs], vy[kFly][kPairs];
 #pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-      const int n = lane + 32 * i;
-      if (n < p.N) x[i] += __ldg(part + n);
+    for (int u = 0; u < kFly; ++u) {
+      const float *part = row + (s0 + u) * p.part_stride;
+#pragma unroll
+      for (int i = 0; i < kPairs; ++i) {
+        const int n = 64 * i + 2 * lane;
+        vx[u][i] = s0 + u < p.ks && n < p.N ? __ldg(part + n) : 0.f;
+        vy[u][i] = s0 + u < p.ks && n + 1 < p.N ? __ldg(part + n + 1) : 0.f;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kFly; ++u) {
+#pragma unroll
+      for (int i = 0; i < kPairs; ++i) {
+        x[i] += vx[u][i];
+        y[i] += vy[u][i];
+      }
     }
   }
   float m = -INFINITY;
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) m = fmaxf(m, x[i]);
+  for (int i = 0; i < kPairs; ++i) m = fmaxf(m, fmaxf(x[i], y[i]));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   constexpr float kLog2e = 1.4426950408889634f;
   const float mb = m * kLog2e;
-  __nv_bfloat16 *prow = p.P + static_cast<long long>(c) * p.F * p.Np + static_cast<long long>(f) * p.Np;
+  uint32_t *prow = reinterpret_cast<uint32_t *>(p.P + static_cast<long long>(c) * p.F * p.Np +
+                                                static_cast<long long>(f) * p.Np);
   float l = 0.f;
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    const int n = lane + 32 * i;
-    if (n < p.Np) {
-      const __nv_bfloat16 b = __float2bfloat16_rn(n < p.N ? fast_exp2(fmaf(x[i], kLog2e, -mb)) : 0.f);
-      l += __bfloat162float(b);
-      prow[n] = b;
+  for (int i = 0; i < kPairs; ++i) {
+    const int n = 64 * i + 2 * lane;
+    if (64 * i < p.Np) {
+      const __nv_bfloat162 w = __floats2bfloat162_rn(n < p.N ? fast_exp2(fmaf(x[i], kLog2e, -mb)) : 0.f,
+                                                     n + 1 < p.N ? fast_exp2(fmaf(y[i], kLog2e, -mb)) : 0.f);
+      l += __low2float(w) + __high2float(w);
+      prow[32 * i + lane] = *reinterpret_cast<const uint32_t *>(&w);
     }
   }
 #pragma unroll
@@ -123,7 +151,14 @@ compress_softmax_kernel(const __grid_constant__ VcSoftmaxParams p) {
   if (lane == 0) p.l[f * p.C + c] = l;
 }
 
-__global__ void __launch_bounds__(kVcThreads, 1)
+// O^T = F_V^T P^T of a frame: CTA (part, f) takes its share of the frame's
+// groups of 128 columns, M = 128 columns, N = C padded to 16, K = 16 tokens.
+// Warp 9 streams the features (MN-major A) and the weights (K-major B) of T
+// tokens per ring slot, warp 8 issues the MMAs into one of two accumulators,
+// warps 0-7 divide by l and store bf16.  One CTA per 128 columns and copies
+// issued from a one-lane branch (~500 cycles each, three per slot) took 10.4 us
+// for 5 x 576 x 4096 and 28.8 us for 128 x 144 x 3584 alone.
+__global__ void __launch_bounds__(kVcThreads)
 compress_apply_kernel(const __grid_constant__ CUtensorMap tmap_f, const __grid_constant__ CUtensorMap tmap_p,
                       const __grid_constant__ VcParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -132,15 +167,19 @@ compress_apply_kernel(const __grid_constant__ CUtensorMap tmap_f, const __grid_c
   const int S = p.stages;
   const uint32_t ring = smem_addr(smem);
   uint64_t *bar_mem = reinterpret_cast<uint64_t *>(smem + static_cast<size_t>(S) * p.stage_bytes);
-  int *s_misc = reinterpret_cast<int *>(bar_mem + 2 * S + 1);  // [0] TMEM, [1] abort, [2] issued, [3] consumed
+  int *s_misc = reinterpret_cast<int *>(bar_mem + 2 * S + 5);  // [0] TMEM, [1] abort, [2] issued, [3] consumed
   float *s_inv = reinterpret_cast<float *>(s_misc + 16);       // 1 / l of the frame's queries
   volatile int *s_abort = s_misc + 1;
   const uint32_t bars = smem_addr(bar_mem);
-  const int FULL = 0, EMPTY = S, DONE = 2 * S;
+  const int FULL = 0, EMPTY = S, OFULL = 2 * S, OEMPTY = 2 * S + 2, FIN = 2 * S + 4;
   auto bar = [&](int i) -> uint32_t { return bars + 8u * static_cast<uint32_t>(i); };
 
-  const int chunk = blockIdx.x, f = blockIdx.y;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int f = blockIdx.y;
+  const int tid = threadIdx.x, warp = uniform_warp_id(), lane = tid & 31;
+  // this CTA's column groups, taken last first: the scores read the columns
+  // in ascending order, so the last ones are the likeliest to be in L2 still
+  const int part = blockIdx.x;
+  const int g0 = part * p.groups / p.per_frame, g1 = (part + 1) * p.groups / p.per_frame;
 
   grid_launch_dependents();
   if (tid == 0) {
@@ -148,7 +187,11 @@ compress_apply_kernel(const __grid_constant__ CUtensorMap tmap_f, const __grid_c
       mbar_init(bar(FULL + i), 1);
       mbar_init(bar(EMPTY + i), 1);
     }
-    mbar_init(bar(DONE), 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar(OFULL + i), 1);
+      mbar_init(bar(OEMPTY + i), kVcEpiThreads);
+    }
+    mbar_init(bar(FIN), 1);
     fence_mbar_init();
     prefetch_tensormap(&tmap_f);
     prefetch_tensormap(&tmap_p);
@@ -168,87 +211,126 @@ compress_apply_kernel(const __grid_constant__ CUtensorMap tmap_f, const __grid_c
       tmem_relinquish_alloc_permit();
       tc_fence_before_sync();
     }
-    named_bar_sync(3, 160);
+    named_bar_sync(3, kVcEpiThreads + 32);
     tc_fence_after_sync();
     tmem = static_cast<uint32_t>(s_misc[0]);
   }
 
+  const uint32_t half = static_cast<uint32_t>(p.T) * 128u;       // 64 columns of a slot's tokens
+  const uint32_t pbox = static_cast<uint32_t>(p.Cp) * 128u;      // the weights of 64 tokens
+  const int pboxes = (p.T + kVcTokens - 1) / kVcTokens;
   if (warp == kVcProducerWarp) {
-    if (lane == 0) {
-      grid_dependency_wait();  // P comes from the softmax kernel
-      const uint64_t pol = l2_policy_evict_first();
-      int k = 0;
-      for (; k < p.KT; ++k) {
-        const int slot = k % S;
-        if (k >= S && !mbar_wait_or_abort(bar(EMPTY + slot), ((k / S) - 1) & 1, s_abort)) break;
-        const uint32_t dst = ring + static_cast<uint32_t>(slot) * p.stage_bytes;
-        mbar_arrive_expect_tx(bar(FULL + slot), p.stage_bytes);
-        // features: tokens f*N + 64k .. +63 of columns [128 chunk, +64) and [+64, +128)
-        tma_load_2d(dst, &tmap_f, chunk * kVcCols, f * p.N + k * kVcTokens, bar(FULL + slot), pol);
-        tma_load_2d(dst + kVcFBytes / 2, &tmap_f, chunk * kVcCols + 64, f * p.N + k * kVcTokens,
-                    bar(FULL + slot), pol);
-        // weights of those tokens for every query (rows >= C are zero-filled)
-        tma_load_2d(dst + kVcFBytes, &tmap_p, f * p.Np + k * kVcTokens, 0, bar(FULL + slot), pol);
+    // the whole warp runs the loop and an elected lane issues, so that the
+    // copies' operands are warp-uniform (see smem_desc_sw128)
+    grid_dependency_wait();  // P comes from the softmax kernel
+    const uint64_t pol_f = l2_policy_evict_first(), pol_p = l2_policy_evict_last();
+    int slot = 0, q = 0;
+    uint32_t lap = 0;  // earlier passes over the ring
+    bool ok = true;
+    for (int g = g1 - 1; g >= g0 && ok; --g)
+      for (int t = 0; t < p.slots; ++t, ++q) {
+        bool w = true;
+        if (lap > 0) w = mbar_wait_or_abort(bar(EMPTY + slot), (lap - 1) & 1u, s_abort);
+        if (!(ok = __all_sync(0xffffffffu, w))) break;
+        const uint32_t dst = ring + static_cast<uint32_t>(slot) * p.stage_bytes, fb = bar(FULL + slot);
+        if (elect_one()) {
+          mbar_arrive_expect_tx(fb, p.stage_bytes);
+          // the slot's tokens of columns [128 g, +64) and [128 g + 64, +64);
+          // tokens past the frame are zero-filled
+          tma_load_3d(dst, &tmap_f, g * kVcCols, t * p.T, f, fb, pol_f);
+          tma_load_3d(dst + half, &tmap_f, g * kVcCols + 64, t * p.T, f, fb, pol_f);
+          // their weights for every query (rows >= C are zero-filled)
+          tma_load_2d(dst + 2 * half, &tmap_p, f * p.Np + t * p.T, 0, fb, pol_p);
+          if (pboxes > 1) tma_load_2d(dst + 2 * half + pbox, &tmap_p, f * p.Np + t * p.T + kVcTokens, 0, fb, pol_p);
+        }
+        __syncwarp();
+        if (++slot == S) {
+          slot = 0;
+          ++lap;
+        }
       }
-      s_misc[2] = k;
-    }
+    if (lane == 0) s_misc[2] = q;
     __syncwarp();
   } else if (warp == kVcMmaWarp) {
     const uint32_t idesc = idesc_bf16_f32(128, p.Cp, 1, 0);  // A MN-major, B K-major
+    int slot = 0, q = 0;
+    uint32_t lap = 0;
     bool ok = true;
-    for (int k = 0; k < p.KT; ++k) {
-      const int slot = k % S;
-      int w = 1;
-      if (lane == 0) w = mbar_wait_or_abort(bar(FULL + slot), (k / S) & 1, s_abort);
-      if (!__shfl_sync(0xffffffffu, w, 0)) {
-        ok = false;
-        break;
+    for (int g = g1 - 1, i = 0; g >= g0 && ok; --g, ++i) {
+      const int buf = i & 1;
+      if (i >= 2) {
+        const bool w = mbar_wait_or_abort(bar(OEMPTY + buf), (i / 2 - 1) & 1, s_abort);
+        if (!(ok = __all_sync(0xffffffffu, w))) break;
+        tc_fence_after_sync();
       }
-      tc_fence_after_sync();
-      if (lane == 0) s_misc[3] = k + 1;
-      const uint32_t base = ring + static_cast<uint32_t>(slot) * p.stage_bytes;
-      if (elect_one()) {
+      const uint32_t d = tmem + static_cast<uint32_t>(buf * p.Cp);
+      for (int t = 0; t < p.slots; ++t) {
+        const bool w = mbar_wait_or_abort(bar(FULL + slot), lap & 1u, s_abort);
+        if (!(ok = __all_sync(0xffffffffu, w))) break;
+        tc_fence_after_sync();
+        if (lane == 0) s_misc[3] = ++q;
+        const uint32_t base = ring + static_cast<uint32_t>(slot) * p.stage_bytes;
+        // A: 16 tokens = two 8-row atoms (2 KB) into each 64-column half, the
+        // halves (M) `half` apart.  B: 16 tokens = 32 bytes along the 128-byte
+        // swizzled rows of P, 8-row groups 1 KB apart.
+        const uint64_t a0 = smem_desc_sw128(base, half, 1024), b0 = smem_desc_sw128(base + 2 * half, 16, 1024);
+        const uint64_t b1 = b0 + (pbox >> 4);
+        const int steps = p.T / 16;
+        const uint32_t acc = t > 0 ? 1u : 0u;
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < kVcTokens / 16; ++kk) {
-          // A: 16 tokens = two 8-row atoms (2 KB) into each 64-column half;
-          // the halves (M) are kVcFBytes / 2 apart.  B: 16 tokens = 32 bytes
-          // along the 128-byte swizzled rows of P, 8-row groups 1 KB apart.
-          const uint64_t a = smem_desc_sw128(base + kk * 2048u, kVcFBytes / 2, 1024);
-          const uint64_t b = smem_desc_sw128(base + kVcFBytes + kk * 32u, 16, 1024);
-          tc_mma_ss(tmem, a, b, idesc, (k > 0 || kk > 0) ? 1u : 0u);
+          for (int k = 0; k < 4; ++k)
+            if (k < steps) tc_mma_ss(d, a0 + 128 * k, b0 + 2 * k, idesc, k > 0 ? 1u : acc);
+          if (steps > 4) {
+#pragma unroll
+            for (int k = 4; k < 8; ++k)
+              if (k < steps) tc_mma_ss(d, a0 + 128 * k, b1 + 2 * (k - 4), idesc, 1u);
+          }
+          tc_commit(bar(EMPTY + slot));
         }
-        tc_commit(bar(EMPTY + slot));
+        __syncwarp();
+        if (++slot == S) {
+          slot = 0;
+          ++lap;
+        }
       }
+      if (ok && elect_one()) tc_commit(bar(OFULL + buf));
       __syncwarp();
     }
-    if (ok && elect_one()) tc_commit(bar(DONE));
+    if (elect_one()) tc_commit(bar(FIN));
     __syncwarp();
-    if (ok) (void)mbar_wait_bounded(bar(DONE), 0);
+    (void)mbar_wait_bounded(bar(FIN), 0);  // every MMA issued has completed
   } else {
     // ------------------------------------------------------------------
-    // epilogue: lane = feature column 32 * warp + lane of the chunk, TMEM
-    // columns = queries
+    // epilogue: lane = feature column of the group, TMEM columns = queries;
+    // the two warps of a lane quarter take 16 queries in turn
     // ------------------------------------------------------------------
     grid_dependency_wait();  // l comes from the softmax kernel
-    for (int c = tid; c < p.C; c += 128) {
+    for (int c = tid; c < p.C; c += kVcEpiThreads) {
       const float l = p.l[f * p.C + c];
       s_inv[c] = l > 0.f ? 1.f / l : 0.f;
     }
-    named_bar_sync(1, 128);
-    bool ok = mbar_wait_or_abort(bar(DONE), 0, s_abort);
-    ok = __all_sync(0xffffffffu, ok);
-    if (ok) {
+    named_bar_sync(1, kVcEpiThreads);
+    const int quarter = warp & 3;
+    const uint32_t lane_base = tmem + (static_cast<uint32_t>(32 * quarter) << 16);
+    for (int g = g1 - 1, i = 0; g >= g0; --g, ++i) {
+      const int buf = i & 1;
+      const bool ok = mbar_wait_or_abort(bar(OFULL + buf), (i / 2) & 1, s_abort);
+      if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after_sync();
-      const uint32_t lane_base = tmem + (static_cast<uint32_t>(32 * warp) << 16);
-      __nv_bfloat16 *dst = p.out + static_cast<size_t>(f) * p.C * p.d + chunk * kVcCols + 32 * warp + lane;
-      for (int c0 = 0; c0 < p.Cp; c0 += 16) {
+      __nv_bfloat16 *dst =
+          p.out + static_cast<size_t>(f) * p.C * p.d + g * kVcCols + 32 * quarter + lane;
+#pragma unroll 1
+      for (int c0 = 16 * (warp >> 2); c0 < p.C; c0 += 32) {
         uint32_t v[16];
-        tmem_ld_32x32b_x16(lane_base + static_cast<uint32_t>(c0), v);
+        tmem_ld_32x32b_x16(lane_base + static_cast<uint32_t>(buf * p.Cp + c0), v);
 #pragma unroll
         for (int j = 0; j < 16; ++j)
           if (c0 + j < p.C)
             dst[static_cast<size_t>(c0 + j) * p.d] = __float2bfloat16_rn(__uint_as_float(v[j]) * s_inv[c0 + j]);
       }
+      tc_fence_before_sync();
+      mbar_arrive(bar(OEMPTY + buf));
     }
     tc_fence_before_sync();
   }
@@ -291,6 +373,7 @@ struct VcLayout {
 static VcLayout vc_layout(int F, int N, int C, int d, int sm_count) {
   VcLayout L;
   L.ks = projection_splits(F * N, d, sm_count);
+  if (L.ks > kVcMaxSplits) L.ks = kVcMaxSplits;
   const int Np = (N + kVcTokens - 1) / kVcTokens * kVcTokens;
   size_t off = 256;
   L.scores = off;
@@ -394,22 +477,37 @@ int sf_visual_compress(const void *queries, const void *features, int F, int N, 
   prm.Cp = (C + 15) / 16 * 16;
   prm.d = d;
   prm.Np = Np;
-  prm.KT = Np / kVcTokens;
-  prm.stage_bytes = kVcFBytes + static_cast<uint32_t>(prm.Cp) * 128u;
-  // a ring no deeper than the CTA's token chunks, and small enough for two
-  // or more CTAs per SM (the CTAs are short: prologue and epilogue overlap)
-  prm.stages = prm.KT < kVcMaxStages ? prm.KT : kVcMaxStages;
-  while (prm.stages > 2 && vc_smem_bytes(prm.stages, prm.stage_bytes, C) > static_cast<size_t>(dev.max_smem_optin) / 2)
+  prm.groups = d / kVcCols;
+  // CTAs per frame: at most two per SM, each with as many column groups as that
+  // leaves (one prologue for all of them), or one group each.  128 frames x
+  // 3584: 2 per frame 46.8 us for the whole call, 1 55.1, 3 50.9, 28 53.5
+  prm.per_frame = 2 * dev.sm_count / F;
+  if (prm.per_frame < 1) prm.per_frame = 1;
+  if (prm.per_frame > prm.groups) prm.per_frame = prm.groups;
+  // tokens per slot: the whole frame where it is short, else 64 (one box of
+  // weights)
+  const int n16 = (N + 15) / 16 * 16;
+  prm.T = n16 <= 96 ? n16 : kVcTokens;
+  prm.slots = (n16 + prm.T - 1) / prm.T;
+  const uint32_t boxes = static_cast<uint32_t>((prm.T + kVcTokens - 1) / kVcTokens);
+  prm.stage_bytes = static_cast<uint32_t>(prm.T) * 256u + boxes * static_cast<uint32_t>(prm.Cp) * 128u;
+  // a ring no deeper than the CTA's slots, and small enough for two CTAs per
+  // SM (prologue, softmax wait and epilogue of one under the other's stream)
+  const int slots = prm.slots * ((prm.groups + prm.per_frame - 1) / prm.per_frame);
+  prm.stages = slots < kVcMaxStages ? slots : kVcMaxStages;
+  while (prm.stages > 2 && vc_smem_bytes(prm.stages, prm.stage_bytes, C) > static_cast<size_t>(dev.max_smem_optin) / 2 - 1024)
     --prm.stages;
   uint32_t cols = 32;
-  while (cols < static_cast<uint32_t>(prm.Cp)) cols <<= 1;
+  while (cols < 2u * static_cast<uint32_t>(prm.Cp)) cols <<= 1;
   prm.tmem_cols = cols;
   CUtensorMap tmap_f, tmap_p;
   {
-    const uint64_t dims[2] = {static_cast<uint64_t>(d), static_cast<uint64_t>(F) * N};
-    const uint64_t strides[1] = {static_cast<uint64_t>(d) * 2};
-    const uint32_t box[2] = {64, static_cast<uint32_t>(kVcTokens)};
-    st = encode_tensor_map_bf16(&tmap_f, features, 2, dims, strides, box);
+    // frames as the third dimension: tokens past a frame's last are zero-filled
+    const uint64_t row = static_cast<uint64_t>(d) * 2;
+    const uint64_t dims[3] = {static_cast<uint64_t>(d), static_cast<uint64_t>(N), static_cast<uint64_t>(F)};
+    const uint64_t strides[2] = {row, row * static_cast<uint64_t>(N)};
+    const uint32_t box[3] = {64, static_cast<uint32_t>(prm.T), 1};
+    st = encode_tensor_map_bf16(&tmap_f, features, 3, dims, strides, box);
     if (st != SF_OK) return st;
   }
   {
@@ -419,7 +517,7 @@ int sf_visual_compress(const void *queries, const void *features, int F, int N, 
     st = encode_tensor_map_bf16(&tmap_p, P, 2, dims, strides, box);
     if (st != SF_OK) return st;
   }
-  cfg.gridDim = dim3(d / kVcCols, F);
+  cfg.gridDim = dim3(prm.per_frame, F);
   cfg.blockDim = dim3(kVcThreads);
   cfg.dynamicSmemBytes = vc_smem_bytes(prm.stages, prm.stage_bytes, C);
   e = cudaLaunchKernelEx(&cfg, compress_apply_kernel, tmap_f, tmap_p, prm);

@@ -66,6 +66,32 @@ def test_compressor_matches_oracle(oracle_mod, F, N, C, d):
         np.testing.assert_array_equal(got, np.repeat(bf16_bits_to_f32(f), C, axis=1))
 
 
+@pytest.mark.parametrize("F,N,C,d", [
+    (310, 20, 3, 768),      # more frames than two per SM: one CTA walks six column groups
+    (40, 97, 17, 1152),     # the first two-slot frame (a 64-token slot, then 33), 7 or 8 CTAs per frame
+    (2, 96, 16, 256),       # the longest one-slot frame (weights in two boxes)
+    (3, 65, 16, 128),       # one token in the second box of weights
+    (1, 129, 33, 4096),     # four hidden-range partials per score (the most)
+])
+def test_compressor_at_slot_and_split_edges(oracle_mod, F, N, C, d):
+    q, f = make_compress_case(F, N, C, d, seed=[F, N, C, d, 1])
+    got = run(q, f)
+    frames = np.unique(np.linspace(0, F - 1, 4).astype(int))
+    ref = oracle_mod.visual_compress(q, f[frames])
+    assert (np.abs(got[frames] - ref) <= bound(f[frames], ref)).all()
+
+
+def test_frames_do_not_reach_into_one_another():
+    # 50 tokens end inside a 16-token step of the copies: what lies behind them
+    # belongs to the next frame and must not count, NaN included
+    q, f = make_compress_case(3, 50, 4, 256, seed=9)
+    want = run(q, f)
+    f[1] = 0x7FC0  # bf16 NaN
+    got = run(q, f)
+    np.testing.assert_array_equal(got[[0, 2]], want[[0, 2]])
+    assert np.isnan(got[1]).all()
+
+
 @pytest.mark.parametrize("name", ["image7b", "gqa"])
 def test_named_workload_compressor_matches_oracle(oracle_mod, name):
     F, N, C, d = COMPRESS_SHAPES[name]
