@@ -116,380 +116,478 @@ __device__ __forceinline__ void draw_terms(float x, float qx, bool residual, flo
   r = residual ? fmaxf(__fsub_rn(pz, qx), 0.0f) : pz;
 }
 
-// The k accept/reject decisions of sequence b and its outputs, from the
-// combined rows in shared memory (row rr: max s_rm, first argmax s_rarg,
-// float-float sum s_rS, the draft token's logit s_rlx and draft probability
-// s_rqx, s_rhx = the token lies in [0, V)).  Called by every thread of the
-// block after the rows are visible; thread i < k tests draft i (my_tok,
-// my_u), threads <= k write out_tokens; j goes to num_accepted and seqs.
-__device__ void decide_sequence(const AccParams &p, int b, bool greedy, float tau, int my_tok,
-                                float my_u, const float *s_rm, const int *s_rarg, const ff *s_rS,
-                                const float *s_rlx, const float *s_rqx, const int *s_rhx,
-                                int *s_acc, bool write = true, int *s_j = nullptr) {
-  const int tid = threadIdx.x, k = p.k, V = p.V;
-  if (tid < k) {
-    const int i = tid, x = my_tok;
-    int acc = 0;
+// What the decisions leave to the draw: the first rejected position j (k if
+// none) and row j's largest logit and sum.
+struct Decision {
+  int j;
+  float m;
+  ff S;
+};
+
+// The k accept/reject decisions of sequence b by one warp.  Lane i <= k holds
+// the final statistics of row i (max rm, first argmax rarg, float-float sum rS);
+// lane i < k tests draft i: its token, uniform, the token's logit lx and draft
+// probability qx (0 outside the vocabulary).  With `write`, every output is
+// written except, for a sampled sequence, out_tokens[j], which the draw writes.
+__device__ __forceinline__ Decision decide_core(const AccParams &p, int b, float tau, float rm, int rarg, ff rS,
+                                                int tok, float u, float lx, float qx, bool write) {
+  const int lane = threadIdx.x & 31, k = p.k;
+  const bool greedy = !(tau > 0.0f);
+  const bool in_range = tok >= 0 && tok < p.V;
+  int acc = 0;
+  if (lane < k) {
     float ratio = 0.f;
-    if (x < 0 || x >= V || !s_rhx[i]) {
+    if (!in_range) {
       if (write) set_status(p.status, SF_DEVICE_BAD_TOKEN);  // treated as a rejection
     } else if (greedy) {
-      acc = (x == s_rarg[i]);
+      acc = tok == rarg;
       ratio = acc ? 1.f : 0.f;
     } else {
       // p(x) = exp((l_x - m) / tau) / S; accept iff u * q(x) < p(x), with the
       // product u * q kept exactly as float-float
-      const float px = ff_div_to_f(exp_diff_accurate(s_rlx[i], s_rm[i], tau), s_rS[i]);
-      const float qd = s_rqx[i];
-      const float uq = __fmul_rn(my_u, qd);
-      const ff uqf = ff{uq, __fmaf_rn(my_u, qd, -uq)};
+      const float px = ff_div_to_f(exp_diff_accurate(lx, rm, tau), rS);
+      const float uq = __fmul_rn(u, qx);
+      const ff uqf = ff{uq, __fmaf_rn(u, qx, -uq)};
       acc = ff_lt(uqf, ff_of(px)) ? 1 : 0;
-      ratio = qd > 0.f ? fminf(1.f, __fdiv_rn(px, qd)) : 1.f;
+      ratio = qx > 0.f ? fminf(1.f, __fdiv_rn(px, qx)) : 1.f;
     }
-    s_acc[i] = acc;
-    if (write && p.ratio) p.ratio[(size_t)b * k + i] = ratio;
+    if (write && p.ratio) p.ratio[(size_t)b * k + lane] = ratio;
   }
-  __syncthreads();
-  if (tid <= k) {
-    // every writer finds j in shared memory; thread i writes out_tokens[i]
-    int j = k;
-    for (int i = 0; i < k; ++i)
-      if (!s_acc[i]) { j = i; break; }
-    int32_t v = -1;
-    if (tid < j) v = my_tok;
-    else if (tid == j && greedy) v = s_rarg[j];
-    if (write && !(tid == j && !greedy)) p.out_tokens[(size_t)b * (k + 1) + tid] = v;
-    if (tid == 0) {
-      if (write) {
-        p.num_accepted[b] = j;
-        p.seqs[b] = SeqState{j, s_rm[j], s_rS[j]};
-      }
-      if (s_j) *s_j = j;
+  const unsigned rejected = __ballot_sync(0xffffffffu, lane < k && !acc);
+  const int j = rejected ? __ffs(rejected) - 1 : k;
+  const int arg_j = __shfl_sync(0xffffffffu, rarg, j);
+  const Decision d = {j, __shfl_sync(0xffffffffu, rm, j),
+                      ff{__shfl_sync(0xffffffffu, rS.hi, j), __shfl_sync(0xffffffffu, rS.lo, j)}};
+  if (write && lane <= k) {
+    int v = -1;
+    if (lane < j) v = tok;
+    else if (lane == j && greedy) v = arg_j;
+    if (!(lane == j && !greedy)) p.out_tokens[(size_t)b * (k + 1) + lane] = v;
+    if (lane == 0) p.num_accepted[b] = j;
+  }
+  return d;
+}
+
+// Lane i < k of a warp: draft token i of sequence b, its uniform, logit and
+// draft probability (0 outside the vocabulary).
+struct DraftEntry {
+  int tok;
+  float u, lx, qx;
+};
+
+__device__ __forceinline__ DraftEntry load_draft(const AccParams &p, int b) {
+  const int lane = threadIdx.x & 31, k = p.k;
+  DraftEntry d = {-1, 0.f, 0.f, 0.f};
+  if (lane < k) {
+    d.tok = p.tokens[(size_t)b * k + lane];
+    d.u = p.u[(size_t)b * (k + 1) + lane];
+    if (d.tok >= 0 && d.tok < p.V) {
+      d.lx = p.logits[((size_t)b * (k + 1) + lane) * p.V + d.tok];
+      d.qx = p.q[((size_t)b * k + lane) * p.V + d.tok];
     }
   }
+  return d;
 }
 
 // Single-kernel acceptance for V <= 16 * kClusterMaxSlice: one thread-block
 // cluster of cs CTAs per sequence, CTA `rank` owning tokens [rank * slice,
-// (rank + 1) * slice) of every row.  Phases, separated by cluster barriers
-// (the same number on every path; greedy clusters leave together after the
-// decision):
-//  1. each warp reduces one row of the CTA's slice to (max, first argmax,
-//     float-float sum of exp((x - max)/tau));
-//  2. CTA 0 combines the cs records of each row (read through distributed
-//     shared memory, in rank order), takes the decisions (decide_sequence)
-//     and publishes j and row j's (max, sum);
-//  3. sampled sequences: each CTA writes row j's residual (or bonus) terms
-//     of its slice to shared memory and their ordered sum;
-//  4. every CTA adds the cs slice sums in rank order, finds the slice
-//     holding u_k * S, and that CTA scans its terms in ascending order.
+// (rank + 1) * slice) of every row.  It is a chain of latencies (a row is 128 KB
+// at most), so the chain is short and its code, which runs once per launch and
+// is fetched cold, is rolled over the rows:
+//  1. every row's slice is copied to shared memory at once, or `bufs` rows at a
+//     time (one bulk copy per row; with q_ahead also the draft rows' slices, of
+//     which the draw needs one that is not known yet), and the draft tokens'
+//     logits and probabilities are on their way meanwhile;
+//  2. per row the slice's maximum and first index, then the float-float sum of
+//     exp((x - max)/tau), pushed into every CTA of the cluster;
+//  3. after the first cluster barrier every CTA combines the cs records of
+//     each row in rank order and takes the decisions, identically; CTA 0
+//     writes them.  Greedy clusters leave here;
+//  4. each thread forms the residual (or bonus) terms of 8 consecutive tokens of
+//     row j in registers; the slice's masses are pushed into every CTA;
+//  5. after the second cluster barrier the CTA holding u_k * S finds the token
+//     by a float-float scan over its threads' terms.
+// Nobody touches a peer's shared memory after the second barrier.  Measured
+// back to back (V = 32000): B = 1, k = 5 17.6 -> 11.3 us, greedy 5.4 -> 4.4; B = 16,
+// k = 8 31.1 -> 24.0; B = 64, k = 4 76 -> 40 us, against the same phases with
+// four barriers, the decisions in CTA 0 alone, row j read again from memory
+// and the sums combined warp by warp.
 constexpr int kClusterMax = 16;
-constexpr int kClusterMaxSlice = 2048;   // tokens per CTA: one row slice in a warp's registers
+constexpr int kClusterMaxSlice = 2048;
 constexpr int kClusterPerThread = kClusterMaxSlice / kAccThreads;  // 8
+// Draft rows are fetched ahead of the decision while they are few (B k V 4
+// bytes, about a microsecond of the memory's time): the draw then doesn't wait
+// for memory once more.
+constexpr long long kAheadBytes = 8 << 20;
+constexpr int kClusterFewBufs = 5;  // rows in shared memory at a time, where not all
 
-struct alignas(16) ClusterRec {  // one row of one CTA's slice (one 16-byte remote load)
+struct alignas(16) ClusterRec {  // one row of one CTA's slice
   float m;
   int arg;
   ff S;
 };
 
-struct alignas(16) ClusterDraw {  // row j's terms in one CTA's slice (two 16-byte loads)
-  ff sum_r, sum_p;
-  int last_r, last_p;
-  int pad[2];
+struct alignas(16) ClusterDraw {  // row j's terms in one CTA's slice
+  ff sum;    // their mass
+  int last;  // last index with mass (-1 if none)
+  int pad;
 };
-static_assert(sizeof(ClusterRec) == 16 && sizeof(ClusterDraw) == 32, "record sizes");
+static_assert(sizeof(ClusterRec) == 16 && sizeof(ClusterDraw) == 16, "record sizes");
+
+// Dynamic shared memory: `bufs` rows' slices, then the k draft rows'.
+static size_t cluster_smem(int k, int slice, int bufs, bool ahead) {
+  return sizeof(float) * static_cast<size_t>(slice) * (bufs + (ahead ? k : 0));
+}
+
+// Inclusive float-float prefix over the first `n` lanes (n a power of two): a
+// lane's exclusive value is the inclusive value of the lane before, bit for bit.
+__device__ __forceinline__ ff warp_scan_ff(ff v, int n, ff *excl) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    if (o >= n) break;
+    const ff t = shfl_up_ff(v, o);
+    if (lane >= o) v = ff_add(t, v);
+  }
+  *excl = shfl_up_ff(v, 1);
+  if (lane == 0) *excl = ff_of(0.f);
+  return v;
+}
+
+__device__ __forceinline__ ff shfl_ff(ff v, int lane) {
+  return ff{__shfl_sync(0xffffffffu, v.hi, lane), __shfl_sync(0xffffffffu, v.lo, lane)};
+}
+
+// The same over the block, with two barriers; returns the thread's exclusive
+// value (again the inclusive value of the thread before).
+__device__ __forceinline__ ff block_scan2(ff v, ff *s_warp, ff *total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  ff ex, wex;
+  v = warp_scan_ff(v, 32, &ex);
+  __syncthreads();  // s_warp may be in use
+  if (lane == 31) s_warp[warp] = v;
+  __syncthreads();
+  const ff w = warp_scan_ff(lane < kAccWarps ? s_warp[lane] : ff_of(0.f), kAccWarps, &wex);
+  *total = shfl_ff(w, kAccWarps - 1);
+  const ff off = shfl_ff(wex, warp);
+  const ff prev = shfl_up_ff(ff_add(off, v), 1);
+  return lane > 0 ? prev : off;
+}
 
 __global__ void __launch_bounds__(kAccThreads)
-accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice) {
-  extern __shared__ float s_terms[];  // [slice]
-  __shared__ ClusterRec s_rec[SF_MAX_DRAFT + 1];
-  __shared__ ClusterRec s_part[SF_MAX_DRAFT + 1][kAccWarps];  // per-warp partials of phase 1
-  __shared__ ClusterDraw s_draw;
-  __shared__ int s_dec_j;
-  __shared__ float s_dec_m;
-  __shared__ ff s_dec_S;
-  __shared__ ff s_d[32];
-  __shared__ ff s_scan[kAccWarps + 1];
-  __shared__ int s_acc[SF_MAX_DRAFT];
-  __shared__ float s_rm[SF_MAX_DRAFT + 1], s_rlx[SF_MAX_DRAFT + 1], s_rqx[SF_MAX_DRAFT + 1];
-  __shared__ int s_rarg[SF_MAX_DRAFT + 1], s_rhx[SF_MAX_DRAFT + 1];
+accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, int bufs, int q_ahead) {
+  extern __shared__ __align__(128) float s_rows[];  // [bufs][slice], then [k][slice] of q
+  __shared__ ClusterRec s_all[kClusterMax][SF_MAX_DRAFT + 1];  // pushed by every CTA of the cluster
+  __shared__ ClusterDraw s_draws[kClusterMax];
+  __shared__ float s_wm[SF_MAX_DRAFT + 1][kAccWarps];
+  __shared__ int s_wi[SF_MAX_DRAFT + 1][kAccWarps];
+  __shared__ ff s_part[SF_MAX_DRAFT + 1][kAccWarps];
+  __shared__ float s_rm[SF_MAX_DRAFT + 1];
+  __shared__ int s_rarg[SF_MAX_DRAFT + 1];
   __shared__ ff s_rS[SF_MAX_DRAFT + 1];
-  __shared__ int s_i0, s_i1;
-  __shared__ ff s_base, s_total;
+  __shared__ Decision s_dec;
+  __shared__ ff s_scan[kAccWarps];
+  __shared__ int s_last[kAccWarps], s_tok;
+  __shared__ uint64_t s_bars[SF_MAX_DRAFT + 2];
 
+  const int rank = blockIdx.x, b = blockIdx.y;
+  const int tid = threadIdx.x, lane = tid & 31, warp = uniform_warp_id();
+  const int k = p.k, V = p.V;
+  const int x0 = min(V, rank * slice), len = min(V, x0 + slice) - x0;
+  const uint32_t bars = smem_addr(s_bars);
+  float *s_q = s_rows + static_cast<size_t>(bufs) * slice;
+  if (tid == 0) {
+    for (int r = 0; r <= k + 1; ++r) mbar_init(bars + 8u * r, 1);
+    fence_mbar_init();
+    s_tok = INT_MAX;
+  }
+  __syncthreads();
+  cluster_arrive();        // this CTA has started
   grid_dependency_wait();  // logits, q, tokens and the outputs follow the previous kernel
   grid_launch_dependents();
-  const int rank = blockIdx.x, b = blockIdx.y;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int k = p.k, V = p.V;
-  const float tau = p.tau[b];
-  const bool greedy = !(tau > 0.0f);
-  const int x0 = min(V, rank * slice), x1 = min(V, x0 + slice);
 
-  // ---- 1. row statistics of the slice: warp w reduces the w-th eighth of
-  // the slice of every row (rows interleaved, short dependency chains), then
-  // warp r merges row r's eight partials in warp order ----
-  {
-    constexpr int kRG = 6;  // rows per pass
-    const int sub = kClusterMaxSlice / kAccWarps;  // 256 tokens per warp
-    const int w0 = x0 + warp * sub, w1 = min(x1, w0 + sub);
-    for (int g = 0; g <= k; g += kRG) {
-      float v[kRG][8];
-#pragma unroll
-      for (int i = 0; i < kRG; ++i) {
-        const int r = g + i;
-        const float *row = p.logits + ((size_t)b * (k + 1) + (r <= k ? r : k)) * V;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int e = w0 + 4 * (lane + 32 * h);
-          float4 x = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-          if (r <= k) {
-            if (p.vec4) {
-              if (e < w1) x = *reinterpret_cast<const float4 *>(row + e);
-            } else {
-              if (e < w1) x.x = row[e];
-              if (e + 1 < w1) x.y = row[e + 1];
-              if (e + 2 < w1) x.z = row[e + 2];
-              if (e + 3 < w1) x.w = row[e + 3];
-            }
-          }
-          v[i][4 * h] = x.x; v[i][4 * h + 1] = x.y; v[i][4 * h + 2] = x.z; v[i][4 * h + 3] = x.w;
+  // ---- 1. copies ----
+  const float *rows = p.logits + (size_t)b * (k + 1) * V + x0;
+  const float *qrows = p.q + (size_t)b * k * V + x0;
+  const bool bulk = p.vec4;  // rows are 16-byte aligned and their slices multiples of 16 bytes
+  // rows r0 .. r0 + n - 1 into the buffers
+  auto fetch = [&](int r0, int n) {
+    if (bulk) {
+      const uint32_t bytes = static_cast<uint32_t>(len) * 4u;
+      for (int i = warp; i < n; i += kAccWarps) {
+        if (elect_one()) {
+          mbar_arrive_expect_tx(bars + 8u * i, bytes);
+          bulk_copy_g2s(smem_addr(s_rows + static_cast<size_t>(i) * slice), rows + (size_t)(r0 + i) * V, bytes,
+                        bars + 8u * i);
         }
+        __syncwarp();
       }
+    } else {
+      for (int i = 0; i < n; ++i) {
 #pragma unroll
-      for (int i = 0; i < kRG; ++i) {
-        float bv = -INFINITY;
-        int bi = INT_MAX;
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const int e = w0 + 4 * (lane + 32 * (t / 4)) + (t % 4);
-          if (better(v[i][t], e, bv, bi)) { bv = v[i][t]; bi = e; }
+        for (int t = 0; t < kClusterPerThread; ++t) {
+          const int e = tid + kAccThreads * t;
+          if (e < len) s_rows[static_cast<size_t>(i) * slice + e] = rows[(size_t)(r0 + i) * V + e];
         }
-        warp_argmax(bv, bi);
-        ff S = ff_of(0.f);
-        if (!greedy && bv != -INFINITY) {
-          float e[8];
-#pragma unroll
-          for (int t = 0; t < 8; ++t) e[t] = v[i][t] != -INFINITY ? exp_scaled(v[i][t], bv, tau) : 0.f;
-          S = ff_add(ff_of(sum4(e[0], e[1], e[2], e[3])), ff_of(sum4(e[4], e[5], e[6], e[7])));
-          S = warp_sum_ff(S);
-        }
-        if (lane == 0 && g + i <= k) s_part[g + i][warp] = ClusterRec{bv, bi, S};
-      }
-    }
-    __syncthreads();
-    for (int r = warp; r <= k; r += kAccWarps) {
-      // lane w < 8 holds warp w's partial; merged in warp order
-      float cm = -INFINITY;
-      int ca = INT_MAX;
-      ff cS = ff_of(0.f);
-      if (lane < kAccWarps) {
-        cm = s_part[r][lane].m;
-        ca = s_part[r][lane].arg;
-        cS = s_part[r][lane].S;
-      }
-      float mv = cm;
-      int mi = ca;
-      warp_argmax(mv, mi);
-      ff Sr = ff_of(0.f);
-      if (!greedy && mv != -INFINITY) {
-        for (int w = 0; w < kAccWarps; ++w) {
-          const float wm = __shfl_sync(0xffffffffu, cm, w);
-          const ff wS = ff{__shfl_sync(0xffffffffu, cS.hi, w), __shfl_sync(0xffffffffu, cS.lo, w)};
-          if (ff_pos(wS)) Sr = ff_add(Sr, ff_mul(wS, exp_diff_accurate(wm, mv, tau)));
-        }
-      }
-      if (lane == 0) s_rec[r] = ClusterRec{mv, mi, Sr};
-    }
-  }
-  cluster_sync();
-
-  // ---- 2. CTA 0: combine the slices of every row and decide ----
-  if (rank == 0) {
-    int my_tok = -1;
-    float my_u = 0.f;
-    if (tid < k) {
-      my_tok = p.tokens[(size_t)b * k + tid];
-      my_u = p.u[(size_t)b * (k + 1) + tid];
-    }
-    for (int r = warp; r <= k; r += kAccWarps) {
-      float mv = -INFINITY, cm = -INFINITY;
-      int mi = INT_MAX;
-      ff cS = ff_of(0.f);
-      if (lane < cs) {
-        const float4 rec = ld_dsmem_f32x4(smem_addr(&s_rec[r]), lane);
-        cm = rec.x;
-        cS = ff{rec.z, rec.w};
-        mv = cm;
-        mi = __float_as_int(rec.y);
-      }
-      warp_argmax(mv, mi);
-      ff Sr = ff_of(0.f);
-      if (!greedy && mv != -INFINITY) {
-        if (lane < cs && ff_pos(cS)) Sr = ff_mul(cS, exp_diff_accurate(cm, mv, tau));
-        Sr = warp_sum_ff(Sr);
-      }
-      if (lane == 0) {
-        const int x = r < k ? p.tokens[(size_t)b * k + r] : -1;
-        const bool ok = x >= 0 && x < V;
-        s_rm[r] = mv;
-        s_rarg[r] = mi;
-        s_rS[r] = Sr;
-        s_rlx[r] = ok ? p.logits[((size_t)b * (k + 1) + r) * V + x] : 0.f;
-        s_rqx[r] = ok ? p.q[((size_t)b * k + r) * V + x] : 0.f;
-        s_rhx[r] = ok ? 1 : 0;
-      }
-    }
-    __syncthreads();
-    decide_sequence(p, b, greedy, tau, my_tok, my_u, s_rm, s_rarg, s_rS, s_rlx, s_rqx, s_rhx, s_acc);
-    // publish j and row j's (max, sum) into every CTA's shared memory
-    if (tid < cs) {
-      int j = k;
-      for (int i = 0; i < k; ++i)
-        if (!s_acc[i]) { j = i; break; }
-      st_dsmem_f32(dsmem_addr(smem_addr(&s_dec_j), tid), __int_as_float(j));
-      st_dsmem_f32(dsmem_addr(smem_addr(&s_dec_m), tid), s_rm[j]);
-      st_dsmem_f32(dsmem_addr(smem_addr(&s_dec_S), tid), s_rS[j].hi);
-      st_dsmem_f32(dsmem_addr(smem_addr(&s_dec_S) + 4, tid), s_rS[j].lo);
-    }
-  }
-  cluster_sync();
-  if (greedy) return;  // uniform over the cluster: the sequence is complete
-
-  // ---- 3. row j's residual (or bonus) terms of the slice ----
-  const int j = s_dec_j;
-  const float mj = s_dec_m;
-  const ff Sj = s_dec_S;
-  const bool residual = j < k;
-  const float invS = ff_div_to_f(1.0f, Sj);
-  const float *row = p.logits + ((size_t)b * (k + 1) + j) * V;
-  const float *qrow = residual ? p.q + ((size_t)b * k + j) * V : nullptr;
-  const int len = x1 - x0;
-  ff sp = ff_of(0.f);
-  int lr = -1, lp = -1;
-  {
-    float xv[kClusterPerThread], qv[kClusterPerThread];
-#pragma unroll
-    for (int t = 0; t < kClusterPerThread; ++t) {
-      const int e = tid + kAccThreads * t;
-      xv[t] = e < len ? row[x0 + e] : 0.f;
-      qv[t] = (residual && e < len) ? qrow[x0 + e] : 0.f;
-    }
-    float pzs[kClusterPerThread];
-#pragma unroll
-    for (int t = 0; t < kClusterPerThread; ++t) {
-      const int e = tid + kAccThreads * t;
-      pzs[t] = 0.f;
-      if (e < len) {
-        float rr;
-        draw_terms(xv[t], qv[t], residual, mj, tau, invS, rr, pzs[t]);
-        s_terms[e] = rr;
-        if (rr > 0.f) lr = x0 + e;
-        if (pzs[t] > 0.f) lp = x0 + e;
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < kClusterPerThread; t += 4)
-      sp = ff_add(sp, ff_of(sum4(pzs[t], pzs[t + 1], pzs[t + 2], pzs[t + 3])));
-  }
-  __syncthreads();
-  // thread t owns the contiguous run [a0, a1) of the slice, summed in order
-  const int per = (len + kAccThreads - 1) / kAccThreads;
-  const int a0 = min(len, tid * per), a1 = min(len, a0 + per);
-  {
-    ff mine = ff_of(0.f);
-    for (int e = a0; e < a1; ++e) mine = ff_add(mine, ff_of(s_terms[e]));
-    ff ex, tot;
-    block_inclusive_scan(mine, s_scan, &ex, &tot);
-    const ff tp = block_sum(sp, s_d);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lr = max(lr, __shfl_xor_sync(0xffffffffu, lr, o));
-      lp = max(lp, __shfl_xor_sync(0xffffffffu, lp, o));
-    }
-    if (tid == 0) { s_i0 = -1; s_i1 = -1; }
-    __syncthreads();
-    if (lane == 0) { atomicMax(&s_i0, lr); atomicMax(&s_i1, lp); }
-    __syncthreads();
-    if (tid == 0) s_draw = ClusterDraw{tot, tp, s_i0, s_i1, {0, 0}};
-  }
-  cluster_sync();
-
-  // ---- 4. the slice holding u_k * S draws the token ----
-  if (warp == 0) {
-    // lane l reads slice l's record (all in flight together); the sums run
-    // in rank order through shuffles, identically in every CTA
-    ff r_l = ff_of(0.f), p_l = ff_of(0.f);
-    int lr_l = -1, lp_l = -1;
-    if (lane < cs) {
-      const uint32_t a = smem_addr(&s_draw);
-      const float4 s0 = ld_dsmem_f32x4(a, lane), s1 = ld_dsmem_f32x4(a + 16, lane);
-      r_l = ff{s0.x, s0.y};
-      p_l = ff{s0.z, s0.w};
-      lr_l = __float_as_int(s1.x);
-      lp_l = __float_as_int(s1.y);
-    }
-    ff tr = ff_of(0.f), tp = ff_of(0.f);
-    for (int l = 0; l < cs; ++l) {
-      tr = ff_add(tr, ff{__shfl_sync(0xffffffffu, r_l.hi, l), __shfl_sync(0xffffffffu, r_l.lo, l)});
-      tp = ff_add(tp, ff{__shfl_sync(0xffffffffu, p_l.hi, l), __shfl_sync(0xffffffffu, p_l.lo, l)});
-    }
-    const bool use_p = !ff_pos(tr);  // residual with no mass (rounding only)
-    const ff total = use_p ? tp : tr;
-    const ff target = ff_mul(total, p.u[(size_t)b * (k + 1) + k]);
-    // slice l covers [cum_l, cum_l + sum_l); cum_{l+1} = ff_add(cum_l, sum_l) exactly
-    int cross = -1, last = -1;
-    ff cum = ff_of(0.f), base = ff_of(0.f);
-    for (int l = 0; l < cs; ++l) {
-      const ff mine = use_p ? p_l : r_l;
-      const ff sl = ff{__shfl_sync(0xffffffffu, mine.hi, l), __shfl_sync(0xffffffffu, mine.lo, l)};
-      const ff nxt = ff_add(cum, sl);
-      last = max(last, __shfl_sync(0xffffffffu, use_p ? lp_l : lr_l, l));
-      if (cross < 0 && ff_pos(sl) && ff_lt(target, nxt) && !ff_lt(target, cum)) {
-        cross = l;
-        base = cum;
-      }
-      cum = nxt;
-    }
-    if (lane == 0) {
-      s_i0 = cross;
-      s_i1 = use_p ? 1 : 0;
-      s_total = target;
-      s_base = base;
-      // no slice holds the target (rounding): the last token with positive mass
-      if (cross < 0 && rank == 0) p.out_tokens[(size_t)b * (k + 1) + j] = last;
-    }
-  }
-  __syncthreads();
-  if (s_i0 == rank) {
-    const bool use_p = s_i1 != 0;
-    if (use_p) {
-      for (int e = tid; e < len; e += kAccThreads) {
-        float rr, pz;
-        draw_terms(row[x0 + e], 0.f, false, mj, tau, invS, rr, pz);
-        s_terms[e] = pz;
       }
       __syncthreads();
     }
-    const ff target = s_total;
-    ff mine = ff_of(0.f);
-    for (int e = a0; e < a1; ++e) mine = ff_add(mine, ff_of(s_terms[e]));
-    ff ex, tot;
-    block_inclusive_scan(mine, s_scan, &ex, &tot);
-    ff c = ff_add(s_base, ex);
-    if (tid == 0) s_i0 = INT_MAX;
-    __syncthreads();
-    for (int e = a0; e < a1; ++e) {
-      c = ff_add(c, ff_of(s_terms[e]));
-      if (ff_lt(target, c)) { atomicMin(&s_i0, x0 + e); break; }
+  };
+  fetch(0, min(bufs, k + 1));
+  const float tau = p.tau[b];
+  const bool greedy = !(tau > 0.0f);
+  DraftEntry ent = {-1, 0.f, 0.f, 0.f};
+  if (warp == 0) ent = load_draft(p, b);
+  const float u_k = p.u[(size_t)b * (k + 1) + k];
+  const bool ahead = q_ahead && !greedy;
+  if (ahead) {
+    const uint32_t bytes = static_cast<uint32_t>(len) * 4u, qb = bars + 8u * (k + 1);
+    if (warp == kAccWarps - 1) {
+      if (elect_one()) mbar_arrive_expect_tx(qb, bytes * static_cast<uint32_t>(k));
+      __syncwarp();
+      for (int r = 0; r < k; ++r) {
+        if (elect_one())
+          bulk_copy_g2s(smem_addr(s_q + static_cast<size_t>(r) * slice), qrows + (size_t)r * V, bytes, qb);
+        __syncwarp();
+      }
+    }
+  }
+  bool landed = true;  // every copy waited for so far
+
+  // ---- 2. the slice's statistics: warp w takes tokens [256 w, 256 w + 256)
+  // of every row, lane l tokens 128 h + 4 l .. + 3 of them ----
+  auto load8 = [&](int buf, float (&v)[8]) {
+    const float *row = s_rows + static_cast<size_t>(buf) * slice;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = 256 * warp + 128 * h + 4 * lane;
+      const float4 x = e < slice ? *reinterpret_cast<const float4 *>(row + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[4 * h] = e < len ? x.x : -INFINITY;
+      v[4 * h + 1] = e + 1 < len ? x.y : -INFINITY;
+      v[4 * h + 2] = e + 2 < len ? x.z : -INFINITY;
+      v[4 * h + 3] = e + 3 < len ? x.w : -INFINITY;
+    }
+  };
+  int r0 = 0;  // the buffers hold rows r0 .. r0 + bufs - 1
+#pragma unroll 1
+  for (uint32_t lap = 0;; ++lap) {
+    const int n = min(bufs, k + 1 - r0);
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      if (bulk) landed &= mbar_wait_bounded(bars + 8u * i, lap & 1u);
+      float v[8];
+      load8(i, v);
+      float bv = -INFINITY;
+      int bi = INT_MAX;
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        const int e = x0 + 256 * warp + 128 * (t / 4) + 4 * lane + (t % 4);
+        if (better(v[t], e, bv, bi)) { bv = v[t]; bi = e; }
+      }
+      warp_argmax(bv, bi);
+      if (lane == 0) {
+        s_wm[r0 + i][warp] = bv;
+        s_wi[r0 + i][warp] = bi;
+      }
     }
     __syncthreads();
-    if (tid == 0)
-      p.out_tokens[(size_t)b * (k + 1) + j] =
-          s_i0 != INT_MAX ? s_i0 : (use_p ? s_draw.last_p : s_draw.last_r);
+    if (!greedy) {
+#pragma unroll 1
+      for (int i = 0; i < n; ++i) {
+        float m = s_wm[r0 + i][0];
+#pragma unroll
+        for (int w = 1; w < kAccWarps; ++w) m = fmaxf(m, s_wm[r0 + i][w]);
+        const float ref = m == -INFINITY ? 0.f : m;  // all masked: every term is 0
+        float v[8];
+        load8(i, v);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[t] = __fsub_rn(v[t], ref);
+        if (tau != 1.0f) {
+#pragma unroll
+          for (int t = 0; t < 8; ++t) v[t] = __fdiv_rn(v[t], tau);
+        }
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[t] = exp_fast(v[t]);
+        const ff S = warp_sum_ff(two_sum(sum4(v[0], v[1], v[2], v[3]), sum4(v[4], v[5], v[6], v[7])));
+        if (lane == 0) s_part[r0 + i][warp] = S;
+      }
+    }
+    if (r0 + bufs > k) break;
+    if (bulk) fence_proxy_async_smem();  // this thread's reads before the next copies
+    __syncthreads();
+    r0 += bufs;
+    fetch(r0, min(bufs, k + 1 - r0));
   }
-  cluster_sync();  // peers may still read this CTA's s_draw
+  __syncthreads();
+  cluster_wait();  // every peer has started
+  for (int r = warp; r <= k; r += kAccWarps) {
+    // the eight warps' records of row r, in warp order
+    float mv = lane < kAccWarps ? s_wm[r][lane] : -INFINITY;
+    int mi = lane < kAccWarps ? s_wi[r][lane] : INT_MAX;
+    warp_argmax(mv, mi);
+    ff S = lane < kAccWarps && !greedy ? s_part[r][lane] : ff_of(0.f);
+    S = shfl_ff(warp_sum_ff<kAccWarps>(S), 0);
+    if (lane < cs) {
+      const uint32_t at = dsmem_addr(smem_addr(&s_all[rank][r]), static_cast<uint32_t>(lane));
+      st_dsmem_f32x2(at, mv, __int_as_float(mi));
+      st_dsmem_f32x2(at + 8, S.hi, S.lo);
+    }
+  }
+  cluster_sync();
+
+  // ---- 3. combine the slices of every row, in rank order, and decide ----
+  for (int r = warp; r <= k; r += kAccWarps) {
+    float cm = -INFINITY;
+    int ci = INT_MAX;
+    ff cS = ff_of(0.f);
+    if (lane < cs) {
+      cm = s_all[lane][r].m;
+      ci = s_all[lane][r].arg;
+      cS = s_all[lane][r].S;
+    }
+    float mv = cm;
+    int mi = ci;
+    warp_argmax(mv, mi);
+    ff Sr = ff_of(0.f);
+    if (!greedy && mv != -INFINITY) {
+      if (lane < cs && ff_pos(cS)) Sr = ff_mul(cS, exp_diff_accurate(cm, mv, tau));
+      Sr = warp_sum_ff<kClusterMax>(Sr);
+    }
+    if (lane == 0) {
+      s_rm[r] = mv;
+      s_rarg[r] = mi;
+      s_rS[r] = Sr;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const int r = lane <= k ? lane : 0;
+    const Decision d =
+        decide_core(p, b, tau, s_rm[r], s_rarg[r], s_rS[r], ent.tok, ent.u, ent.lx, ent.qx, rank == 0);
+    if (lane == 0) s_dec = d;
+  }
+  if (!__all_sync(0xffffffffu, landed) && lane == 0) set_status(p.status, SF_DEVICE_TIMEOUT);
+  if (greedy) return;  // uniform over the cluster: the sequence is complete
+  __syncthreads();
+
+  // ---- 4. row j's residual (or bonus) terms, tokens 8 tid .. 8 tid + 7 ----
+  const Decision dec = s_dec;
+  const int j = dec.j;
+  const bool residual = j < k;
+  const float invS = ff_div_to_f(1.0f, dec.S);
+  const int e0 = 8 * tid;
+  float tr[8], tp[8];
+  {
+    float xv[8], qv[8];
+    const bool here = j >= r0;  // row j is still in its buffer
+    const float *row = s_rows + static_cast<size_t>(here ? j - r0 : 0) * slice;
+    // four tokens of a row of the slice in global memory
+    auto fetch4 = [&](const float *g, int e, float pad) -> float4 {
+      if (bulk) return __ldg(reinterpret_cast<const float4 *>(g + e));
+      return make_float4(g[e], e + 1 < len ? g[e + 1] : pad, e + 2 < len ? g[e + 2] : pad,
+                         e + 3 < len ? g[e + 3] : pad);
+    };
+    if (ahead) {  // also when all drafts were accepted: the copies must have landed before the CTA ends
+      if (!__all_sync(0xffffffffu, mbar_wait_bounded(bars + 8u * (k + 1), 0)) && lane == 0)
+        set_status(p.status, SF_DEVICE_TIMEOUT);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = e0 + 4 * h;
+      float4 x = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY), q = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (e < len) {
+        x = here ? *reinterpret_cast<const float4 *>(row + e) : fetch4(rows + (size_t)j * V, e, -INFINITY);
+        if (residual)
+          q = ahead ? *reinterpret_cast<const float4 *>(s_q + static_cast<size_t>(j) * slice + e)
+                    : fetch4(qrows + (size_t)j * V, e, 0.f);
+      }
+      xv[4 * h] = x.x; xv[4 * h + 1] = x.y; xv[4 * h + 2] = x.z; xv[4 * h + 3] = x.w;
+      qv[4 * h] = q.x; qv[4 * h + 1] = q.y; qv[4 * h + 2] = q.z; qv[4 * h + 3] = q.w;
+    }
+#pragma unroll
+    for (int t = 0; t < 8; ++t) tr[t] = tp[t] = 0.f;
+    // the temperature is tested once, not once per term (its divisions are
+    // skipped together)
+    if (tau == 1.f) {
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (e0 + t < len) draw_terms(xv[t], qv[t], residual, dec.m, 1.f, invS, tr[t], tp[t]);
+    } else {
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (e0 + t < len) draw_terms(xv[t], qv[t], residual, dec.m, tau, invS, tr[t], tp[t]);
+    }
+  }
+  auto sum8 = [](const float (&t)[8]) {
+    return ff_add(ff_add(two_sum(t[0], t[1]), two_sum(t[2], t[3])), ff_add(two_sum(t[4], t[5]), two_sum(t[6], t[7])));
+  };
+  // the slice's mass of the terms t and its last index with mass, into every
+  // CTA's s_draws; returns the thread's exclusive prefix
+  auto publish = [&](const float (&t)[8]) -> ff {
+    int last = -1;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (t[i] > 0.f) last = x0 + e0 + i;
+    last = __reduce_max_sync(0xffffffffu, last);
+    if (lane == 0) s_last[warp] = last;
+    ff tot;
+    const ff ex = block_scan2(sum8(t), s_scan, &tot);  // its barriers order s_last too
+    if (warp == 0) {
+      last = __reduce_max_sync(0xffffffffu, lane < kAccWarps ? s_last[lane] : -1);
+      if (lane < cs) {
+        const uint32_t at = dsmem_addr(smem_addr(&s_draws[rank]), static_cast<uint32_t>(lane));
+        st_dsmem_f32x2(at, tot.hi, tot.lo);
+        st_dsmem_f32(at + 8, __int_as_float(last));
+      }
+    }
+    return ex;
+  };
+  ff excl = publish(tr);
+  cluster_sync();
+
+  // ---- 5. the slice holding u_k * S draws the token ----
+  // slice l covers [ex, in) of an inclusive scan over the slices, identical in
+  // every warp of every CTA
+  const bool have = lane < cs;
+  ff in, ex, mass, total;
+  auto scan_slices = [&]() {
+    mass = have ? s_draws[lane].sum : ff_of(0.f);
+    in = warp_scan_ff(mass, kClusterMax, &ex);
+    total = shfl_ff(in, cs - 1);
+  };
+  scan_slices();
+  if (!ff_pos(total)) {
+    // a residual with no mass (rounding only): draw from the target's row
+    // instead, the cluster once more round the same steps
+#pragma unroll
+    for (int t = 0; t < 8; ++t) tr[t] = tp[t];
+    cluster_sync();  // every CTA has read its s_draws
+    excl = publish(tr);
+    cluster_sync();
+    scan_slices();
+  }
+  const ff target = ff_mul(total, u_k);
+  const unsigned hit = __ballot_sync(0xffffffffu, have && ff_pos(mass) && ff_lt(target, in) && !ff_lt(target, ex));
+  int32_t *out = p.out_tokens + (size_t)b * (k + 1) + j;
+  if (!hit) {
+    // no slice holds the target (rounding): the last token with positive mass
+    const int last = __reduce_max_sync(0xffffffffu, have ? s_draws[lane].last : -1);
+    if (rank == 0 && tid == 0) *out = last;
+    return;
+  }
+  const int cross = __ffs(hit) - 1;
+  if (cross != rank) return;
+  ff c = ff_add(shfl_ff(ex, cross), excl);
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    c = ff_add(c, ff_of(tr[t]));
+    if (tr[t] > 0.f && ff_lt(target, c)) {
+      atomicMin(&s_tok, x0 + e0 + t);
+      break;
+    }
+  }
+  __syncthreads();
+  if (tid == 0) *out = s_tok != INT_MAX ? s_tok : s_draws[rank].last;
 }
 
 // Fused path: the decisions from the projection's per-CTA row statistics
@@ -497,22 +595,17 @@ accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice) {
 // logits.  grid (B), kAccThreads threads: warp w combines rows w, w + 8, ...
 __global__ void __launch_bounds__(kAccThreads)
 accept_decide_kernel(const __grid_constant__ AccParams p, const SampStat *__restrict__ stats, int G) {
-  __shared__ int s_acc[SF_MAX_DRAFT];
-  __shared__ float s_rm[SF_MAX_DRAFT + 1], s_rlx[SF_MAX_DRAFT + 1], s_rqx[SF_MAX_DRAFT + 1];
-  __shared__ int s_rarg[SF_MAX_DRAFT + 1], s_rhx[SF_MAX_DRAFT + 1];
+  __shared__ float s_rm[SF_MAX_DRAFT + 1];
+  __shared__ int s_rarg[SF_MAX_DRAFT + 1];
   __shared__ ff s_rS[SF_MAX_DRAFT + 1];
   grid_dependency_wait();  // statistics and logits come from the projection
   grid_launch_dependents();
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int k = p.k, V = p.V;
+  const int k = p.k;
   const float tau = p.tau[b];
   const bool greedy = !(tau > 0.0f);
-  int my_tok = -1;
-  float my_u = 0.f;
-  if (tid < k) {
-    my_tok = p.tokens[(size_t)b * k + tid];
-    my_u = p.u[(size_t)b * (k + 1) + tid];
-  }
+  DraftEntry e = {-1, 0.f, 0.f, 0.f};
+  if (warp == 0) e = load_draft(p, b);  // in flight with the statistics
   for (int rr = warp; rr <= k; rr += kAccWarps) {
     const size_t row = (size_t)b * (k + 1) + rr;
     const SampStat *cr = stats + row * G;
@@ -528,19 +621,17 @@ accept_decide_kernel(const __grid_constant__ AccParams p, const SampStat *__rest
       Sr = warp_sum_ff(Sr);
     }
     if (lane == 0) {
-      const int x = rr < k ? p.tokens[(size_t)b * k + rr] : -1;
-      const bool ok = x >= 0 && x < V;
       s_rm[rr] = mv;
       s_rarg[rr] = mi;
       s_rS[rr] = Sr;
-      s_rlx[rr] = ok ? p.logits[row * V + x] : 0.f;
-      s_rqx[rr] = ok ? p.q[((size_t)b * k + rr) * V + x] : 0.f;
-      s_rhx[rr] = ok ? 1 : 0;
-      p.rows[row] = RowStat{mv, mi, Sr};
     }
   }
   __syncthreads();
-  decide_sequence(p, b, greedy, tau, my_tok, my_u, s_rm, s_rarg, s_rS, s_rlx, s_rqx, s_rhx, s_acc);
+  if (warp == 0) {
+    const int r = lane <= k ? lane : 0;
+    const Decision d = decide_core(p, b, tau, s_rm[r], s_rarg[r], s_rS[r], e.tok, e.u, e.lx, e.qx, true);
+    if (lane == 0) p.seqs[b] = SeqState{d.j, d.m, d.S};
+  }
 }
 
 // The residual (j < k) or bonus (j == k) draw of sequence b (grid (C2, B)
@@ -889,70 +980,22 @@ __device__ __forceinline__ void run_chunk(RunState &st, int lane, const float4 (
 __device__ __forceinline__ RowStat combine_runs(const AccParams &p, int row, float tau,
                                                 bool greedy);
 
-// The k accept/reject decisions of sequence b by one warp, from the final
-// row statistics (lane i < k tests draft i, exactly as decide_sequence
-// does); writes every output except, for a sampled sequence, out_tokens[j],
-// which the draw kernel writes.
+// The decisions of sequence b by one warp, from the final row statistics in
+// global memory; leaves j and row j's statistics to the draw kernel.
 __device__ void decide_warp(const AccParams &p, int b) {
-  const int lane = threadIdx.x & 31, k = p.k, V = p.V;
-  const float tau = p.tau[b];
-  const bool greedy = !(tau > 0.0f);
-  const RowStat *rows = p.rows + (size_t)b * (k + 1);
+  const int lane = threadIdx.x & 31, k = p.k;
   float rm = 0.f;
   int rarg = -1;
   ff rS = ff_of(0.f);
   if (lane <= k) {
-    const float4 v = __ldcg(reinterpret_cast<const float4 *>(rows + lane));
+    const float4 v = __ldcg(reinterpret_cast<const float4 *>(p.rows + (size_t)b * (k + 1) + lane));
     rm = v.x;
     rarg = __float_as_int(v.y);
     rS = ff{v.z, v.w};
   }
-  int tok = -1;
-  float u = 0.f, lx = 0.f, qx = 0.f;
-  bool in_range = false;
-  if (lane < k) {
-    tok = p.tokens[(size_t)b * k + lane];
-    u = p.u[(size_t)b * (k + 1) + lane];
-    in_range = tok >= 0 && tok < V;
-    if (in_range) {
-      lx = p.logits[((size_t)b * (k + 1) + lane) * V + tok];
-      qx = p.q[((size_t)b * k + lane) * V + tok];
-    }
-  }
-  int acc = 0;
-  if (lane < k) {
-    float ratio = 0.f;
-    if (!in_range) {
-      set_status(p.status, SF_DEVICE_BAD_TOKEN);  // treated as a rejection
-    } else if (greedy) {
-      acc = tok == rarg;
-      ratio = acc ? 1.f : 0.f;
-    } else {
-      // p(x) = exp((l_x - m) / tau) / S; accept iff u * q(x) < p(x), with the
-      // product u * q kept exactly as float-float
-      const float px = ff_div_to_f(exp_diff_accurate(lx, rm, tau), rS);
-      const float uq = __fmul_rn(u, qx);
-      const ff uqf = ff{uq, __fmaf_rn(u, qx, -uq)};
-      acc = ff_lt(uqf, ff_of(px)) ? 1 : 0;
-      ratio = qx > 0.f ? fminf(1.f, __fdiv_rn(px, qx)) : 1.f;
-    }
-    if (p.ratio) p.ratio[(size_t)b * k + lane] = ratio;
-  }
-  const unsigned rejected = __ballot_sync(0xffffffffu, lane < k && !acc);
-  const int j = rejected ? __ffs(rejected) - 1 : k;
-  const int arg_j = __shfl_sync(0xffffffffu, rarg, j);
-  const float m_j = __shfl_sync(0xffffffffu, rm, j);
-  const ff S_j = ff{__shfl_sync(0xffffffffu, rS.hi, j), __shfl_sync(0xffffffffu, rS.lo, j)};
-  if (lane <= k) {
-    int v = -1;
-    if (lane < j) v = tok;
-    else if (lane == j && greedy) v = arg_j;
-    if (!(lane == j && !greedy)) p.out_tokens[(size_t)b * (k + 1) + lane] = v;
-  }
-  if (lane == 0) {
-    p.num_accepted[b] = j;
-    p.seqs[b] = SeqState{j, m_j, S_j};
-  }
+  const DraftEntry e = load_draft(p, b);
+  const Decision d = decide_core(p, b, p.tau[b], rm, rarg, rS, e.tok, e.u, e.lx, e.qx, true);
+  if (lane == 0) p.seqs[b] = SeqState{d.j, d.m, d.S};
 }
 
 // A run record whose row ticket is taken: the row, its number of runs and
@@ -1232,6 +1275,11 @@ static bool cluster_plan(int V, int *cs, int *slice) {
   return true;
 }
 
+// The largest dynamic shared memory of a launch: k = 16 rows of a full slice,
+// with as many draft rows ahead as fit.
+constexpr int kClusterMostSmem = 200 * 1024;
+static_assert(kClusterMostSmem >= (SF_MAX_DRAFT + 1) * kClusterMaxSlice * 4, "the rows themselves fit");
+
 // Sets the kernel attributes once per device and reports whether a cluster
 // of cs CTAs can be resident (*ok false: use the two-kernel path).
 static int cluster_setup(int cs, bool *ok) {
@@ -1243,11 +1291,11 @@ static int cluster_setup(int cs, bool *ok) {
   if (dev.ordinal < 0 || dev.ordinal >= 64) return fail(SF_ERR_UNSUPPORTED, "device ordinal %d", dev.ordinal);
   std::lock_guard<std::mutex> lock(mu);
   if (state[dev.ordinal][cs] == 0) {
+    const int most = kClusterMostSmem;
     cudaError_t e = cudaFuncSetAttribute(accept_cluster_kernel,
                                          cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(accept_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(sizeof(float) * kClusterMaxSlice));
+      e = cudaFuncSetAttribute(accept_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess)
       return fail(SF_ERR_CUDA, "cudaFuncSetAttribute (accept cluster): %s", cudaGetErrorString(e));
     cudaLaunchAttribute attr[1];
@@ -1258,7 +1306,7 @@ static int cluster_setup(int cs, bool *ok) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs, 1);
     cfg.blockDim = dim3(kAccThreads);
-    cfg.dynamicSmemBytes = sizeof(float) * kClusterMaxSlice;
+    cfg.dynamicSmemBytes = most;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
@@ -1384,11 +1432,21 @@ int sf_accept(const float *target_logits, const float *draft_probs,
     cudaLaunchConfig_t ccfg = {};
     ccfg.gridDim = dim3(cs, B);
     ccfg.blockDim = dim3(kAccThreads);
-    ccfg.dynamicSmemBytes = sizeof(float) * slice;
+    // Every row in shared memory while the batch's clusters are all resident
+    // so (about 7 clusters of 16 per CTA that an SM holds), else kClusterFewBufs
+    // rows at a time: more clusters per SM are worth a second round of copies
+    // (B = 16, k = 8, V = 32000: 33 us with all nine rows, 26 with five).
+    const size_t sm_bytes = 228 * 1024, fixed = 9 * 1024;  // static and reserved shared memory
+    const int groups = cs > 8 ? 7 : 15 * 8 / cs;
+    const long long resident = groups * static_cast<long long>(sm_bytes / (cluster_smem(k, slice, k + 1, false) + fixed));
+    const int bufs = B <= resident || k + 1 < kClusterFewBufs ? k + 1 : kClusterFewBufs;
+    const bool ahead = prm.vec4 && bufs == k + 1 && 4LL * B * k * V <= kAheadBytes &&
+                       cluster_smem(k, slice, bufs, true) <= static_cast<size_t>(kClusterMostSmem);
+    ccfg.dynamicSmemBytes = cluster_smem(k, slice, bufs, ahead);
     ccfg.stream = stream;
     ccfg.attrs = cattr;
     ccfg.numAttrs = 2;
-    cudaError_t ce = cudaLaunchKernelEx(&ccfg, accept_cluster_kernel, prm, cs, slice);
+    cudaError_t ce = cudaLaunchKernelEx(&ccfg, accept_cluster_kernel, prm, cs, slice, bufs, ahead ? 1 : 0);
     if (ce != cudaSuccess) return fail(SF_ERR_CUDA, "accept cluster launch: %s", cudaGetErrorString(ce));
     return SF_OK;
   }

@@ -123,19 +123,22 @@ __device__ __forceinline__ ff shfl_up_ff(ff a, int o) {
   return ff{__shfl_up_sync(0xffffffffu, a.hi, o), __shfl_up_sync(0xffffffffu, a.lo, o)};
 }
 
+// Sum over the warp's lanes; with LANES < 32, over each aligned group of them.
+template <int LANES = 32>
 __device__ __forceinline__ ff warp_sum_ff(ff v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = ff_add(v, shfl_xor_ff(v, o));
+  for (int o = LANES / 2; o > 0; o >>= 1) v = ff_add(v, shfl_xor_ff(v, o));
   return v;
 }
 
+// The largest value of the warp (no NaN) and its lowest index, by two integer
+// reductions: the floats' order as unsigned integers (-0 taken as +0).
 __device__ __forceinline__ void warp_argmax(float &v, int &i) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float ov = __shfl_xor_sync(0xffffffffu, v, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, i, o);
-    if (better(ov, oi, v, i)) { v = ov; i = oi; }
-  }
+  const int s = __float_as_int(__fadd_rn(v, 0.0f));
+  const unsigned key = s < 0 ? ~static_cast<unsigned>(s) : static_cast<unsigned>(s) ^ 0x80000000u;
+  const unsigned top = __reduce_max_sync(0xffffffffu, key);
+  i = __reduce_min_sync(0xffffffffu, key == top ? i : INT_MAX);
+  v = __uint_as_float(top & 0x80000000u ? top ^ 0x80000000u : ~top);
 }
 
 // Block-wide float-float sum (fixed tree order).

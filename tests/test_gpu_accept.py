@@ -71,6 +71,22 @@ def test_vocabulary_beyond_the_single_kernel_path(oracle_mod, mode):
     _check(oracle_mod, make_accept_case(3, 4, 200003, seed=17, mode=mode))
 
 
+@pytest.mark.parametrize("B,k,V,mode,temp", [
+    (1, 1, 2, "sampling", 1.0),        # one CTA, one chunk of one lane
+    (2, 3, 2048, "alternate", 1.0),    # exactly one slice
+    (2, 3, 2049, "sampling", 0.7),     # a second CTA of one token, scalar copies
+    (1, 16, 32768, "sampling", 1.0),   # the longest rows, the most of them, no draft rows ahead
+    (3, 16, 30724, "alternate", 1.3),  # the last slice is the shortest
+    (40, 8, 32000, "sampling", 1.0),   # rows five at a time: two rounds of copies
+    (40, 15, 4100, "sampling", 0.8),   # the same with three rounds, three CTAs
+    (40, 9, 9001, "alternate", 1.0),   # the same with scalar copies
+])
+def test_cluster_path_edges(oracle_mod, B, k, V, mode, temp):
+    inp = make_accept_case(B, k, V, seed=[B, k, V], mode=mode)
+    inp.temperature *= np.float32(temp)
+    _check(oracle_mod, inp, max_excluded_frac=0.05)
+
+
 @pytest.mark.parametrize("V", [300000, 300001])
 @pytest.mark.parametrize("mode", ["sampling", "alternate"])
 def test_vocabulary_beyond_256_segments(oracle_mod, V, mode):
@@ -324,7 +340,7 @@ def test_monte_carlo_large_vocabulary_draw(V, support):
     assert chisquare(obs, law * trials).pvalue > alpha, (obs, law * trials)
 
 
-@pytest.mark.parametrize("V", [40000, 40001, 152064])
+@pytest.mark.parametrize("V", [1999, 32000, 40000, 40001, 152064])
 def test_residual_without_mass_draws_from_the_target(oracle_mod, V):
     # q = 1.001 p everywhere: the residual max(0, p - q) is exactly zero, and
     # u_0 = 0.9995 > p/q rejects the first draft (by a relative margin of
