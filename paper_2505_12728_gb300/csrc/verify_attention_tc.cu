@@ -218,7 +218,136 @@ __device__ __forceinline__ void tc_segment(const TcPartition &tp, const AttnPara
   }
 }
 
-template <int D, int STAGES, int F>
+// The same partition decided by one warp alone, for at most 32 sequences: lane
+// b holds sequence b, and nothing goes through shared memory or a block
+// barrier.  Every warp of a CTA takes it for itself, so that the producers
+// reach their first copies without waiting for the other roles.
+constexpr int kTcWarpBatch = 32;
+
+struct TcWarpPartition {
+  TilePartition part;  // the balanced partition
+  bool aligned;
+  int T, tiles, pre;   // lane b: length of sequence b, its tiles, tiles of the sequences before
+  int ns, cpre;        // aligned: CTAs of each of its segments, CTAs of the sequences before
+};
+
+__device__ __forceinline__ int warp_exclusive_sum(int v) {
+  const int lane = threadIdx.x & 31;
+  int incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  return incl - v;
+}
+
+__device__ __forceinline__ TcWarpPartition tc_warp_partition(const AttnParams &p) {
+  const int lane = threadIdx.x & 31;
+  TcWarpPartition w;
+  w.T = 0;
+  if (lane < p.B) {
+    w.T = p.seq_lens[lane];
+    if (w.T < p.n_q || w.T > p.max_tokens) {
+      set_status(p.status, SF_DEVICE_BAD_SEQLEN);
+      w.T = w.T < p.n_q ? p.n_q : p.max_tokens;
+    }
+  }
+  w.tiles = (w.T + kTileTokens - 1) / kTileTokens;
+  w.pre = warp_exclusive_sum(w.tiles);
+  const uint32_t Tot = static_cast<uint32_t>(p.H_kv) * __reduce_add_sync(0xffffffffu, static_cast<unsigned>(w.tiles));
+  const uint32_t pG = static_cast<uint32_t>(p.G), G = Tot < pG ? Tot : pG;
+  w.part = TilePartition{Tot, G, Tot / G, Tot % G};
+  w.aligned = false;
+  w.ns = w.cpre = 0;
+  const uint32_t S = static_cast<uint32_t>(p.B * p.H_kv);
+  if (pG > S) {
+    uint32_t Ta = (Tot + pG - S - 1) / (pG - S);
+    const uint32_t Tmin = (Tot + pG - 1) / pG;
+    w.aligned = Ta <= Tmin + kAlignSlackTiles;
+    if (w.aligned) {
+#pragma unroll 1
+      for (uint32_t cand = Tmin; cand <= Ta; ++cand) {
+        w.ns = static_cast<int>((static_cast<uint32_t>(w.tiles) + cand - 1) / cand);
+        const unsigned need = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(w.ns));
+        if (static_cast<unsigned long long>(need) * static_cast<unsigned>(p.H_kv) <= pG) break;  // Ta always fits
+      }
+      w.cpre = warp_exclusive_sum(p.H_kv * w.ns);
+    }
+  }
+  return w;
+}
+
+// First CTA and number of pieces of segment (b, h); called by whole warps.
+__device__ __forceinline__ void tc_warp_segment(const TcWarpPartition &w, const AttnParams &p, int b, int h,
+                                                int &c_first, int &n_pieces) {
+  if (w.aligned) {
+    n_pieces = __shfl_sync(0xffffffffu, w.ns, b);
+    c_first = __shfl_sync(0xffffffffu, w.cpre, b) + h * n_pieces;
+  } else {
+    const int tiles_b = __shfl_sync(0xffffffffu, w.tiles, b);
+    const uint32_t first = static_cast<uint32_t>(p.H_kv) * static_cast<uint32_t>(__shfl_sync(0xffffffffu, w.pre, b)) +
+                           static_cast<uint32_t>(h * tiles_b);
+    c_first = static_cast<int>(w.part.owner(first));
+    n_pieces = static_cast<int>(w.part.owner(first + tiles_b - 1)) - c_first + 1;
+  }
+}
+
+// The CTA's tile range [t_begin, t_end) and, in the aligned partition, its one
+// piece; called by whole warps.
+__device__ __forceinline__ void tc_warp_range(const TcWarpPartition &w, const AttnParams &p, uint32_t &t_begin,
+                                              uint32_t &t_end, Piece &pc) {
+  const int lane = threadIdx.x & 31, c = static_cast<int>(blockIdx.x);
+  t_begin = t_end = w.part.Tot;
+  if (w.aligned) {
+    // the last sequence whose first CTA is <= c holds it, unless c is past all
+    const unsigned below = __ballot_sync(0xffffffffu, lane < p.B && w.cpre <= c);
+    const int b = 31 - __clz(below);
+    const int tiles_b = __shfl_sync(0xffffffffu, w.tiles, b), ns = __shfl_sync(0xffffffffu, w.ns, b);
+    const int local = c - __shfl_sync(0xffffffffu, w.cpre, b);
+    const int h = local / ns, q = local - h * ns;
+    pc.T = __shfl_sync(0xffffffffu, w.T, b);
+    const int pre = __shfl_sync(0xffffffffu, w.pre, b);
+    if (h < p.H_kv) {
+      pc.b = b;
+      pc.h_kv = h;
+      pc.seg = b * p.H_kv + h;
+      pc.lt0 = q * tiles_b / ns;
+      pc.n_tiles = (q + 1) * tiles_b / ns - pc.lt0;
+      pc.c_first = c - q;
+      pc.n_pieces = ns;
+      pc.Lb = pc.T - p.n_q;
+      t_begin = static_cast<uint32_t>(p.H_kv) * static_cast<uint32_t>(pre) + static_cast<uint32_t>(h * tiles_b + pc.lt0);
+      t_end = t_begin + static_cast<uint32_t>(pc.n_tiles);
+    }
+  } else if (c < static_cast<int>(w.part.G)) {
+    t_begin = w.part.start(c);
+    t_end = w.part.start(c + 1);
+  }
+}
+
+// The piece of the balanced partition that starts at tile t; whole warps.
+__device__ __forceinline__ Piece tc_warp_piece(const TcWarpPartition &w, const AttnParams &p, uint32_t t,
+                                               uint32_t t_end) {
+  const int lane = threadIdx.x & 31;
+  Piece pc;
+  const unsigned below = __ballot_sync(
+      0xffffffffu, lane < p.B && static_cast<uint32_t>(p.H_kv) * static_cast<uint32_t>(w.pre) <= t);
+  pc.b = 31 - __clz(below);
+  const int tiles_b = __shfl_sync(0xffffffffu, w.tiles, pc.b);
+  const uint32_t in = t - static_cast<uint32_t>(p.H_kv) * static_cast<uint32_t>(__shfl_sync(0xffffffffu, w.pre, pc.b));
+  pc.h_kv = static_cast<int>(in / static_cast<uint32_t>(tiles_b));
+  pc.lt0 = static_cast<int>(in) - pc.h_kv * tiles_b;
+  const uint32_t left = t_end - t;
+  pc.n_tiles = left < static_cast<uint32_t>(tiles_b - pc.lt0) ? static_cast<int>(left) : tiles_b - pc.lt0;
+  pc.seg = pc.b * p.H_kv + pc.h_kv;
+  pc.T = __shfl_sync(0xffffffffu, w.T, pc.b);
+  pc.Lb = pc.T - p.n_q;
+  tc_warp_segment(w, p, pc.b, pc.h_kv, pc.c_first, pc.n_pieces);
+  return pc;
+}
+
+template <int D, int STAGES, int F, bool kWarpPart>
 __global__ void __maxnreg__(kTcMaxRegs)
 verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
                            const __grid_constant__ CUtensorMap tmap_v,
@@ -276,48 +405,58 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
     s_misc[3] = 0;
     s_misc[4] = 0;
   }
-  tile_prefix<kTcThreads>(p, s_prefix, s_len, s_misc + 8);
-  __syncthreads();
-
-  const TcPartition tp = tc_partition<kTcThreads>(p, s_prefix, s_cpre, s_misc + 8);
-  const TilePartition &part = tp.part;
-  const bool aligned = tp.aligned;
-  const int Ta = tp.Ta;
-  const uint32_t Tot = part.Tot;
-  const int G = static_cast<int>(part.G);
+  uint32_t t_begin, t_end;
   Piece apc{};  // the aligned partition's piece of this CTA
-  uint32_t t_begin = Tot, t_end = Tot;
-  if (aligned) {
-    const int c = static_cast<int>(blockIdx.x);
-    if (c < s_cpre[p.B]) {
-      int lo = 0, hi = p.B - 1;  // last sequence whose first CTA is <= c
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (s_cpre[mid] <= c) lo = mid; else hi = mid - 1;
+  bool aligned;
+  TcWarpPartition wp{};
+  TilePartition part{};
+  if constexpr (kWarpPart) {
+    __syncthreads();  // barrier initialisation visible to every role
+    wp = tc_warp_partition(p);
+    aligned = wp.aligned;
+    tc_warp_range(wp, p, t_begin, t_end, apc);
+  } else {
+    tile_prefix<kTcThreads>(p, s_prefix, s_len, s_misc + 8);
+    __syncthreads();
+    const TcPartition tp = tc_partition<kTcThreads>(p, s_prefix, s_cpre, s_misc + 8);
+    part = tp.part;
+    aligned = tp.aligned;
+    const int Ta = tp.Ta;
+    t_begin = t_end = part.Tot;
+    if (aligned) {
+      const int c = static_cast<int>(blockIdx.x);
+      if (c < s_cpre[p.B]) {
+        int lo = 0, hi = p.B - 1;  // last sequence whose first CTA is <= c
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (s_cpre[mid] <= c) lo = mid; else hi = mid - 1;
+        }
+        const int b = lo, tiles_b = s_prefix[b + 1] - s_prefix[b];
+        const int ns = (tiles_b + Ta - 1) / Ta, local = c - s_cpre[b];
+        const int h = local / ns, q = local % ns;
+        apc.b = b;
+        apc.h_kv = h;
+        apc.seg = b * p.H_kv + h;
+        apc.lt0 = q * tiles_b / ns;
+        apc.n_tiles = (q + 1) * tiles_b / ns - apc.lt0;
+        apc.c_first = s_cpre[b] + h * ns;
+        apc.n_pieces = ns;
+        apc.T = s_len[b];
+        apc.Lb = apc.T - p.n_q;
+        t_begin = static_cast<uint32_t>(p.H_kv) * static_cast<uint32_t>(s_prefix[b]) +
+                  static_cast<uint32_t>(h * tiles_b + apc.lt0);
+        t_end = t_begin + static_cast<uint32_t>(apc.n_tiles);
       }
-      const int b = lo, tiles_b = s_prefix[b + 1] - s_prefix[b];
-      const int ns = (tiles_b + Ta - 1) / Ta, local = c - s_cpre[b];
-      const int h = local / ns, q = local % ns;
-      apc.b = b;
-      apc.h_kv = h;
-      apc.seg = b * p.H_kv + h;
-      apc.lt0 = q * tiles_b / ns;
-      apc.n_tiles = (q + 1) * tiles_b / ns - apc.lt0;
-      apc.c_first = s_cpre[b] + h * ns;
-      apc.n_pieces = ns;
-      apc.T = s_len[b];
-      apc.Lb = apc.T - p.n_q;
-      t_begin = static_cast<uint32_t>(p.H_kv) * static_cast<uint32_t>(s_prefix[b]) +
-                static_cast<uint32_t>(h * tiles_b + apc.lt0);
-      t_end = t_begin + static_cast<uint32_t>(apc.n_tiles);
+    } else if (blockIdx.x < part.G) {
+      t_begin = part.start(blockIdx.x);
+      t_end = part.start(blockIdx.x + 1);
     }
-  } else if (static_cast<int>(blockIdx.x) < G) {
-    t_begin = part.start(blockIdx.x);
-    t_end = part.start(blockIdx.x + 1);
   }
-  // the piece starting at tile t of this CTA's range
+  // the piece starting at tile t of this CTA's range (called by whole warps)
   auto piece_at = [&](uint32_t t) -> Piece {
-    return aligned ? apc : locate_piece(t, t_end, part, s_prefix, s_len, p);
+    if (aligned) return apc;
+    if constexpr (kWarpPart) return tc_warp_piece(wp, p, t, t_end);
+    else return locate_piece(t, t_end, part, s_prefix, s_len, p);
   };
 
   if (warp == kTcKWarp || warp == kTcVWarp) {
@@ -870,7 +1009,7 @@ constexpr int kTcMergeBatch = 12;
 // 256 threads x 104 registers fit next to a split CTA (224 x 128) on one SM
 constexpr int kTcMergeMaxRegs = 104;
 
-template <int D>
+template <int D, bool kWarpPart>
 __global__ void __maxnreg__(kTcMergeMaxRegs)
 verify_tc_merge_kernel(const __grid_constant__ AttnParams p) {
   constexpr float kLn2 = 0.6931471805599453f;
@@ -881,9 +1020,15 @@ verify_tc_merge_kernel(const __grid_constant__ AttnParams p) {
   int *s_len = s_prefix + p.B + 1;   // [B]
   int *s_cpre = s_len + p.B;         // [B+1]
   grid_launch_dependents();
-  tile_prefix<kTcMergeThreads>(p, s_prefix, s_len, s_scratch + 8);
-  __syncthreads();
-  const TcPartition tp = tc_partition<kTcMergeThreads>(p, s_prefix, s_cpre, s_scratch + 8);
+  TcWarpPartition wp{};
+  TcPartition tp{};
+  if constexpr (kWarpPart) {
+    wp = tc_warp_partition(p);
+  } else {
+    tile_prefix<kTcMergeThreads>(p, s_prefix, s_len, s_scratch + 8);
+    __syncthreads();
+    tp = tc_partition<kTcMergeThreads>(p, s_prefix, s_cpre, s_scratch + 8);
+  }
   grid_dependency_wait();
   // work units of kTcMergeThreads items of one segment (32-bit indices:
   // the units of all segments number fewer than 2^31)
@@ -895,12 +1040,12 @@ verify_tc_merge_kernel(const __grid_constant__ AttnParams p) {
   for (int unit = blockIdx.x; unit < units; unit += gridDim.x) {
     const int seg = unit / units_per_seg;
     const int rem = (unit - seg * units_per_seg) * kTcMergeThreads + threadIdx.x;
-    if (rem >= per_seg) continue;
     const int c4 = rem / p.R, r = rem - c4 * p.R;
     const int b = seg / p.H_kv, h_kv = seg - b * p.H_kv;
     int c_first, n_pieces;
-    tc_segment(tp, p, s_prefix, s_cpre, b, h_kv, c_first, n_pieces);
-    if (n_pieces <= 1) continue;  // the split kernel wrote the output
+    if constexpr (kWarpPart) tc_warp_segment(wp, p, b, h_kv, c_first, n_pieces);
+    else tc_segment(tp, p, s_prefix, s_cpre, b, h_kv, c_first, n_pieces);
+    if (n_pieces <= 1 || rem >= per_seg) continue;  // one piece: the split kernel wrote the output
     const int F = p.R <= 32 ? 4 : (p.R <= 64 ? 2 : 1);  // key-split copies per piece
     const float *slot0 = p.partials + (size_t)(c_first + seg) * F * stride;
     n_pieces *= F;
@@ -954,12 +1099,17 @@ using TcKernelFn = void (*)(const CUtensorMap, const CUtensorMap, const AttnPara
 // at most 4.
 static int tc_key_split(int R) { return R <= 32 ? 4 : (R <= 64 ? 2 : 1); }
 
-template <int D>
+template <int D, bool kWarpPart>
 static TcKernelFn tc_kernel(int F) {
   constexpr int S = TcConfig<D>::kStages;
-  if (F == 4) return verify_attention_tc_kernel<D, S, 4>;
-  if (F == 2) return verify_attention_tc_kernel<D, S, 2>;
-  return verify_attention_tc_kernel<D, S, 1>;
+  if (F == 4) return verify_attention_tc_kernel<D, S, 4, kWarpPart>;
+  if (F == 2) return verify_attention_tc_kernel<D, S, 2, kWarpPart>;
+  return verify_attention_tc_kernel<D, S, 1, kWarpPart>;
+}
+
+static TcKernelFn tc_kernel(int head_dim, int F, bool warp_part) {
+  if (head_dim == 128) return warp_part ? tc_kernel<128, true>(F) : tc_kernel<128, false>(F);
+  return warp_part ? tc_kernel<64, true>(F) : tc_kernel<64, false>(F);
 }
 
 template <int D>
@@ -984,8 +1134,9 @@ int tc_setup(int head_dim, int device) {
   const int k = head_dim == 128 ? 1 : 0;
   std::lock_guard<std::mutex> lock(mu);
   if (done[device][k]) return SF_OK;
-  for (int F : {1, 2, 4}) {
-    TcKernelFn fn = head_dim == 128 ? tc_kernel<128>(F) : tc_kernel<64>(F);
+  for (int v = 0; v < 6; ++v) {
+    const int F = 1 << (v >> 1);
+    TcKernelFn fn = tc_kernel(head_dim, F, v & 1);
     const int smem = head_dim == 128 ? tc_bytes<128>(F, SF_MAX_BATCH) : tc_bytes<64>(F, SF_MAX_BATCH);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
@@ -1011,8 +1162,8 @@ int tc_launch(int head_dim, int G, int smem, const CUtensorMap &tk, const CUtens
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const int F = tc_key_split(prm.R);
-  TcKernelFn fn = head_dim == 128 ? tc_kernel<128>(F) : tc_kernel<64>(F);
-  cudaError_t e = cudaLaunchKernelEx(&cfg, fn, tk, tv, prm);
+  const bool warp_part = prm.B <= kTcWarpBatch;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, tc_kernel(head_dim, F, warp_part), tk, tv, prm);
   if (e != cudaSuccess) return fail(SF_ERR_CUDA, "verify attention (tcgen05) launch: %s", cudaGetErrorString(e));
   const long long items = (long long)prm.R * (head_dim / 4) * prm.B * prm.H_kv;
   long long ctas = (items + kTcMergeThreads - 1) / kTcMergeThreads;
@@ -1020,8 +1171,10 @@ int tc_launch(int head_dim, int G, int smem, const CUtensorMap &tk, const CUtens
   cfg.gridDim = dim3(static_cast<unsigned>(ctas));
   cfg.blockDim = dim3(kTcMergeThreads);
   cfg.dynamicSmemBytes = 4 * (3 * prm.B + 2);
-  e = head_dim == 64 ? cudaLaunchKernelEx(&cfg, verify_tc_merge_kernel<64>, prm)
-                     : cudaLaunchKernelEx(&cfg, verify_tc_merge_kernel<128>, prm);
+  void (*merge)(const AttnParams) =
+      head_dim == 64 ? (warp_part ? verify_tc_merge_kernel<64, true> : verify_tc_merge_kernel<64, false>)
+                     : (warp_part ? verify_tc_merge_kernel<128, true> : verify_tc_merge_kernel<128, false>);
+  e = cudaLaunchKernelEx(&cfg, merge, prm);
   if (e != cudaSuccess) return fail(SF_ERR_CUDA, "verify merge launch: %s", cudaGetErrorString(e));
   return SF_OK;
 }
