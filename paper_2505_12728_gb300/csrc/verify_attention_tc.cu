@@ -126,6 +126,13 @@ struct TcSmem {
   static int bytes(int B) { return 1024 + kPrefixOffset + 4 * (3 * B + 3); }
 };
 
+// max of three in one instruction (a NaN is ignored, as by fmaxf).
+__device__ __forceinline__ float fmax3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // tcgen05.ld / st of N consecutive 32-bit columns of the thread's lane.
 template <int N>
 __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&v)[N]) {
@@ -392,7 +399,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
     }
     for (int x = 0; x < kNumS; ++x) {
       mbar_init(bar(SFULL + x), 1);
-      mbar_init(bar(PFULL + x), kTcSoftmaxThreads);
+      mbar_init(bar(PFULL + x), kTcSoftmaxThreads / 32);
       mbar_init(bar(ODONE + x), 1);
     }
     mbar_init(bar(QFULL), kTcSoftmaxThreads);
@@ -538,7 +545,10 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
     // (P V of tile m - NS issued: the MMAs run in issue order, so that P V
     // reads its P before Q K^T overwrites it) and, for the first tile of a
     // piece, the piece's Q (q_full); P V of tile m needs its P (p_full).
-    // The two streams are issued as soon as their conditions hold.
+    // The two streams are issued as soon as their conditions hold.  The
+    // descriptors of a tile's MMAs are one base and compile-time offsets, and
+    // an idle round is one look at each barrier: the clock and the abort word
+    // are read every 16th (both measured in the softmax comment below).
     // ------------------------------------------------------------------
     grid_dependency_wait();
     tmem_alloc(smem_addr(s_misc), kTmemCols);
@@ -561,6 +571,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
       total += pc.n_tiles;
     }
     unsigned long long t0 = 0;
+    uint32_t idle = 0;
     bool ok = true;
     while (pv < total && ok) {
       bool progress = false;
@@ -588,13 +599,13 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
         if (__all_sync(0xffffffffu, ready)) {
           tc_fence_after_sync();
           if (lane == 0) s_misc[3] = static_cast<int>(qk + 1);
-          const uint32_t kb = ring + slot * L::kStageBytes;
+          const uint64_t b0 = smem_desc_sw128(ring + slot * L::kStageBytes, 16, kKSbo);
           const uint32_t d = tmem + kTmemS + (qk % NS) * 64u;
           if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
               // K step kk: columns 16kk .. 16kk+15 = 32-byte column kk%4 of half kk/4
-              const uint64_t b = smem_desc_sw128(kb + (kk >> 2) * 1024 + (kk & 3) * 32, 16, kKSbo);
+              const uint64_t b = b0 + (((kk >> 2) * 1024 + (kk & 3) * 32) >> 4);
               tc_mma_ts(d, tmem + kTmemQ + kk * 8, b, kIdescQK, kk > 0 ? 1u : 0u);
             }
             tc_commit(bar(SFULL + qk % NS));
@@ -609,7 +620,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
         if (__all_sync(0xffffffffu, ready)) {
           tc_fence_after_sync();
           const uint32_t slot = pv % STAGES;
-          const uint32_t vb = ring + slot * L::kStageBytes + L::kTileBytes;
+          const uint64_t b0 = smem_desc_sw128(ring + slot * L::kStageBytes + L::kTileBytes, kPageHalfBytes, 1024);
           const bool first = pv == pv_piece_start;
           const bool seq_first = first && pv_lt0 == 0;  // the sequence's first tile: P_hi + P_lo
           if (elect_one()) {
@@ -617,7 +628,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
             for (int j = 0; j < kTileTokens / 16; ++j) {
               // V page j = keys 16j..16j+15 (K): 8-key groups 1024 B apart;
               // the 64-column halves of N are kPageHalfBytes apart
-              const uint64_t b = smem_desc_sw128(vb + j * kPageBytes, kPageHalfBytes, 1024);
+              const uint64_t b = b0 + (j * kPageBytes >> 4);
               const uint32_t pb = tmem + kTmemS + (pv % NS) * 64u + j * 8u;
               tc_mma_ts(tmem + kTmemO, pb, b, kIdescPV, (first && j == 0) ? 0u : 1u);
               if (seq_first) tc_mma_ts(tmem + kTmemO, pb + 32u, b, kIdescPV, 1u);
@@ -634,6 +645,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
         t0 = 0;
       } else {
         // nothing ready: bounded wait (the abort word stops it early)
+        if ((++idle & 15u) != 0u) continue;
         if (t0 == 0) t0 = global_timer_ns();
         if (*s_abort) ok = false;
         else if (global_timer_ns() - t0 > kWaitBudgetNs) {
@@ -653,8 +665,28 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
     // tid / RPK (keys kap*KPL .. kap*KPL+KPL-1 of every tile) of query row
     // r = tid % RPK (rows >= R are padding).  Each lane keeps its own
     // reference, sum and O over its keys.
+    //
+    // This loop paces the kernel: K/V tiles are never waited for, and a
+    // 64-key tile takes one pass of it (about 1,150 cycles, of which the
+    // 32 exponentials of two copies are 250 at the MUFU's rate).  So
+    //  * padding rows never take the mask path, which their warp's real rows
+    //    would sit through at every tile;
+    //  * P goes to TMEM by the lane's own columns and zeros for the other
+    //    copies (the copy is warp-uniform), not by 32 selects, and one lane
+    //    of a warp arrives;
+    //  * the maximum is taken in threes, the rescale (rare) stands before
+    //    the exponentials, where fewer registers are live, and the row sum
+    //    is added up while the stores to TMEM are in flight.
+    // With the MMA warp's two changes, per layer: 4 sequences of 4.9k
+    // tokens, 56 rows, 15.1 -> 14.1 us; 8 sequences of 1.2-3.6k, 42 rows, 15.3 ->
+    // 14.5; 70 rows (one copy) 19.3 -> 17.6; 16 sequences of 8-32k, 56 rows,
+    // 113.3 -> 111.5.  Not kept: a second group of softmax warps taking every
+    // other tile (14.2-16.1: the tiles beyond the ring are then waited for,
+    // and two groups' states have to be folded), reading the next tile's
+    // scores while the stores complete (+0.4: more registers), spinning on
+    // the barriers without the try_wait suspension (+0.1).
     // ------------------------------------------------------------------
-    const int kap = tid / RPK, r = tid % RPK;
+    const int kap = warp * 32 / RPK, r = tid % RPK;  // kap: warp-uniform (RPK is a multiple of 32)
     const bool valid = r < p.R;
     const int qi = valid ? r / p.group : 0, qj = valid ? r % p.group : 0;
     float2 *s_ml = reinterpret_cast<float2 *>(smem + L::kMlOffset);
@@ -728,7 +760,8 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
       }
 
       // last visible key position of this row (draft row i sees L_b + i)
-      const int lim = valid ? pc.Lb + min(qi, p.n_q - 1) : -1;
+      // (padding rows see every key: Q is 0 there, and nothing is written)
+      const int lim = valid ? pc.Lb + min(qi, p.n_q - 1) : 0x7fffffc0;
       float ref = -INFINITY, l_run = 0.f;
       for (int it = 0; it < pc.n_tiles && ok; ++it, ++n) {
         const uint32_t sb = tl + kTmemS + (n % NS) * 64u;  // this tile's S buffer
@@ -756,19 +789,22 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
         }
         // this lane's keys kap*KPL .. kap*KPL + KPL-1 (raw scores; the
         // scale, > 0, is applied to the maximum and folded into the exponent)
-        // tile maximum as a tree (a chain of KPL dependent max operations
-        // is ~5 cycles each on the softmax's critical path)
+        // tile maximum in four chains (one chain of KPL dependent max
+        // operations is ~5 cycles each on the softmax's critical path)
         float mx;
         {
-          float t[KPL / 2];
+          float a0 = __uint_as_float(sv[0]), a1 = __uint_as_float(sv[1]), a2 = __uint_as_float(sv[2]),
+                a3 = __uint_as_float(sv[3]);
 #pragma unroll
-          for (int c = 0; c < KPL / 2; ++c) t[c] = fmaxf(__uint_as_float(sv[2 * c]), __uint_as_float(sv[2 * c + 1]));
-#pragma unroll
-          for (int w = KPL / 4; w >= 1; w >>= 1) {
-#pragma unroll
-            for (int c = 0; c < w; ++c) t[c] = fmaxf(t[c], t[c + w]);
+          for (int c = 4; c < KPL; c += 8) {
+            a0 = fmax3(a0, __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
+            a1 = fmax3(a1, __uint_as_float(sv[c + 2]), __uint_as_float(sv[c + 3]));
+            if (c + 4 < KPL) {
+              a2 = fmax3(a2, __uint_as_float(sv[c + 4]), __uint_as_float(sv[c + 5]));
+              a3 = fmax3(a3, __uint_as_float(sv[c + 6]), __uint_as_float(sv[c + 7]));
+            }
           }
-          mx = t[0];
+          mx = fmaxf(fmax3(a0, a1, a2), a3);
         }
         const int key0 = tile_pos + kap * KPL;
         if (key0 + KPL - 1 > lim) {
@@ -787,24 +823,6 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
           if (ref != -INFINITY) alpha = exp2f(ref - mx);
           ref = mx;
         }
-        const float mu = ref == -INFINITY ? 0.f : ref;
-        uint32_t mine[KPL / 2], mine_lo[KPL / 2];
-        float ps[KPL / 2];  // pair sums, added as a tree below
-#pragma unroll
-        for (int c2 = 0; c2 < KPL / 2; ++c2) {
-          const float p0 = fast_exp2(fmaf(__uint_as_float(sv[2 * c2]), p.scale_log2, -mu));
-          const float p1 = fast_exp2(fmaf(__uint_as_float(sv[2 * c2 + 1]), p.scale_log2, -mu));
-          ps[c2] = p0 + p1;
-          if (split_p) split_bf16x2(p0, p1, mine[c2], mine_lo[c2]);
-          else mine[c2] = pack_bf16x2(p0, p1);
-        }
-#pragma unroll
-        for (int w = KPL / 4; w >= 1; w >>= 1) {
-#pragma unroll
-          for (int c = 0; c < w; ++c) ps[c] += ps[c + w];
-        }
-        const float rs = ps[0];
-        l_run = l_run * alpha + rs;
         if (__any_sync(0xffffffffu, alpha != 1.f)) {
           // O *= alpha after the P V of tile n-1 (it > 0 here: the first
           // tile of a piece starts with ref = -inf, so alpha = 1)
@@ -813,31 +831,62 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
             break;
           }
           tc_fence_after_sync();
+          constexpr int kOCols = F == 1 ? 16 : 32;
 #pragma unroll 1
-          for (int ch = 0; ch < D / 32; ++ch) {
-            uint32_t ov[32];
-            tmem_ld_32x32b_x32(tl + kTmemO + ch * 32, ov);
+          for (int ch = 0; ch < D / kOCols; ++ch) {
+            uint32_t ov[kOCols];
+            tmem_ld_cols<kOCols>(tl + kTmemO + ch * kOCols, ov);
 #pragma unroll
-            for (int c = 0; c < 32; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * alpha);
-            tmem_st_32x32b_x32(tl + kTmemO + ch * 32, ov);
+            for (int c = 0; c < kOCols; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * alpha);
+            tmem_st_cols<kOCols>(tl + kTmemO + ch * kOCols, ov);
           }
+        }
+        const float mu = ref == -INFINITY ? 0.f : ref;
+        uint32_t mine[KPL / 2];
+#pragma unroll
+        for (int c2 = 0; c2 < KPL / 2; ++c2) {
+          const float p0 = fast_exp2(fmaf(__uint_as_float(sv[2 * c2]), p.scale_log2, -mu));
+          const float p1 = fast_exp2(fmaf(__uint_as_float(sv[2 * c2 + 1]), p.scale_log2, -mu));
+          mine[c2] = pack_bf16x2(p0, p1);
+          sv[2 * c2] = __float_as_uint(p0);
+          sv[2 * c2 + 1] = __float_as_uint(p1);
         }
         // P over the scores: this lane's keys, zeros for the other copies'
         // keys (the A operand of P V covers the whole tile)
         {
-          uint32_t pk[32];
+          uint32_t zero[KPL / 2];
 #pragma unroll
-          for (int c = 0; c < 32; ++c) pk[c] = (c / (KPL / 2) == kap) ? mine[c % (KPL / 2)] : 0u;
-          tmem_st_32x32b_x32(sb, pk);
+          for (int c = 0; c < KPL / 2; ++c) zero[c] = 0u;
+#pragma unroll
+          for (int k = 1; k < F; ++k)
+            tmem_st_cols<KPL / 2>(sb + static_cast<uint32_t>((kap + k) % F) * (KPL / 2), zero);
+          tmem_st_cols<KPL / 2>(sb + kap * (KPL / 2), mine);
           if (split_p) {  // the sequence's first tile: P_lo too (warp-uniform)
 #pragma unroll
-            for (int c = 0; c < 32; ++c) pk[c] = (c / (KPL / 2) == kap) ? mine_lo[c % (KPL / 2)] : 0u;
-            tmem_st_32x32b_x32(sb + 32, pk);
+            for (int c2 = 0; c2 < KPL / 2; ++c2) {
+              uint32_t hi;
+              split_bf16x2(__uint_as_float(sv[2 * c2]), __uint_as_float(sv[2 * c2 + 1]), hi, mine[c2]);
+            }
+#pragma unroll
+            for (int k = 1; k < F; ++k)
+              tmem_st_cols<KPL / 2>(sb + 32 + static_cast<uint32_t>((kap + k) % F) * (KPL / 2), zero);
+            tmem_st_cols<KPL / 2>(sb + 32 + kap * (KPL / 2), mine);
           }
         }
+        // the sum, as a tree, while the stores are in flight
+        float ps[KPL / 2];
+#pragma unroll
+        for (int c = 0; c < KPL / 2; ++c) ps[c] = __uint_as_float(sv[2 * c]) + __uint_as_float(sv[2 * c + 1]);
+#pragma unroll
+        for (int w = KPL / 4; w >= 1; w >>= 1) {
+#pragma unroll
+          for (int c = 0; c < w; ++c) ps[c] += ps[c + w];
+        }
+        l_run = l_run * alpha + ps[0];
         tmem_wait_st();
         tc_fence_before_sync();
-        mbar_arrive(bar(PFULL + n % NS));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(PFULL + n % NS));
       }
 
       // ---- the next piece's Q (every Q K^T of this piece has completed:

@@ -271,6 +271,36 @@ def test_tcgen05_many_piece_merges_match_oracle(oracle_mod, B, n_q, H_q, H_kv, d
 
 
 @pytest.mark.parametrize("n_q,H_q,H_kv,d", [
+    (3, 12, 2, 64),     # 18 rows per KV head: four key-split copies, 14 padding lanes each
+    (11, 6, 2, 128),    # 33 rows: two copies, 31 padding lanes each
+    (16, 16, 4, 128),   # 64 rows: two copies, no padding
+    (13, 10, 2, 64),    # 65 rows: one copy, 63 padding lanes
+    (16, 8, 1, 128),    # 128 rows: one copy, no padding
+])
+@pytest.mark.parametrize("B", [1, 31, 32, 33])
+@pytest.mark.parametrize("ragged", [False, True])
+def test_tcgen05_partition_and_row_copies_at_their_edges(oracle_mod, n_q, H_q, H_kv, d, B, ragged):
+    # Up to 32 sequences each warp takes the work partition for itself, above
+    # that the block does.  Equal lengths take the segment-aligned partition,
+    # very different ones the balanced one.  The last page's unused slots hold
+    # NaN and infinity: padding lanes multiply them by a zero Q row, and
+    # nothing of that may reach a real row.
+    rng = np.random.default_rng(B + n_q)
+    prefixes = [int(x) for x in rng.choice([0, 3, 70, 500, 2100], size=B)] if ragged else [333] * B
+    case = make_attention_case(B, n_q, H_q, H_kv, d, prefixes, seed=5000 + B + n_q)
+    ref_out, ref_lse = oracle_attention(oracle_mod, case)
+    nan, inf = f32_to_bf16_bits(np.array([np.nan, np.inf], np.float32))
+    for b in range(B):
+        T = int(case.seq_lens[b])
+        if T % 16:
+            last = case.block_table[0, b, (T - 1) // 16]
+            case.k_cache[0, last, :, T % 16:, :] = inf
+            case.v_cache[0, last, :, T % 16:, :] = nan
+    out, lse = run_attention(case, num_splits=0)
+    assert_attention_close(out, lse, ref_out, ref_lse)
+
+
+@pytest.mark.parametrize("n_q,H_q,H_kv,d", [
     (4, 8, 8, 64),      # mma.sync kernel: 8192 segments of one or two tiles
     (8, 28, 4, 128),    # tcgen05 kernel: 56 rows per KV head, 4096 segments
 ])
