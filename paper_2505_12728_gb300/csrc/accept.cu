@@ -64,12 +64,9 @@ struct alignas(16) SeqState {  // what the draw needs, in one 16-byte load
   ff S;            // row j's sum of exp((x - m) / tau)
 };
 
-struct alignas(16) DrawPart {  // one segment of row j
+struct alignas(32) DrawPart {  // one segment of row j: a 32-byte sector, written by one warp
   ff sum_r;        // residual (or bonus) mass of the segment
   ff sum_p;        // target mass of the segment (fallback when the residual is 0)
-  int last_r;      // last index with r > 0 (-1 if none)
-  int last_p;      // last index with p > 0 (-1 if none)
-  int pad[2];
 };
 
 struct AccParams {
@@ -259,8 +256,9 @@ __device__ __forceinline__ ff shfl_ff(ff v, int lane) {
 }
 
 // The same over the block, with two barriers; returns the thread's exclusive
-// value (again the inclusive value of the thread before).
-__device__ __forceinline__ ff block_scan2(ff v, ff *s_warp, ff *total) {
+// value, and in *next (if asked for) the exclusive value of the thread after
+// it, bit for bit (*total after the last), so that [excl, next) tile [0, total).
+__device__ __forceinline__ ff block_scan2(ff v, ff *s_warp, ff *total, ff *next = nullptr) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   ff ex, wex;
   v = warp_scan_ff(v, 32, &ex);
@@ -271,7 +269,12 @@ __device__ __forceinline__ ff block_scan2(ff v, ff *s_warp, ff *total) {
   *total = shfl_ff(w, kAccWarps - 1);
   const ff off = shfl_ff(wex, warp);
   const ff prev = shfl_up_ff(ff_add(off, v), 1);
-  return lane > 0 ? prev : off;
+  const ff excl = lane > 0 ? prev : off;
+  if (next) {
+    const ff after = shfl_ff(excl, (lane + 1) & 31), warp_end = shfl_ff(w, warp);
+    *next = lane < 31 ? after : warp_end;
+  }
+  return excl;
 }
 
 __global__ void __launch_bounds__(kAccThreads)
@@ -641,16 +644,21 @@ accept_decide_kernel(const __grid_constant__ AccParams p, const SampStat *__rest
 // (one atomic ticket; nobody waits) locates the segment holding u_k * S with
 // a float-float scan over the segment sums in order, and scans that segment
 // in ascending token order, four tokens per thread.
+//
+// One wave of CTAs and then one CTA per sequence: the kernel is the issue of
+// a warp's 32 terms (four warps share a scheduler) and a chain of latencies.
+// So the temperature is tested once for all terms, the last index with mass
+// is looked for only where rounding asks for it, and the scans take two
+// barriers each.  From the release of the kernel to the token, 16
+// sequences of V = 152064: 9.0 -> 7.0 us.
 __device__ void draw_residual(const AccParams &p, int b, int c, int j, RowStat rs, float tau,
                               float u_k) {
-  __shared__ ff s_d[32];
-  __shared__ ff s_scan[kAccWarps + 1];
-  __shared__ int s_flag, s_seg, s_token;
+  __shared__ ff s_scan[kAccWarps];
   __shared__ ff s_base;
+  __shared__ int s_flag, s_seg, s_token;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int k = p.k, V = p.V, NS = p.C1;
   const bool residual = j < k;
-  const float invS = ff_div_to_f(1.0f, rs.S);
   const float *row = p.logits + ((size_t)b * (k + 1) + j) * V;
   const float *qrow = residual ? p.q + ((size_t)b * k + j) * V : nullptr;
   DrawPart *parts = p.parts + (size_t)b * NS;
@@ -676,163 +684,137 @@ __device__ void draw_residual(const AccParams &p, int b, int c, int j, RowStat r
   // ---- segment sums of r and p: lane sums of 32 terms added pairwise in
   // fp32, then a float-float warp sum ----
   const int sg = c * kAccWarps + warp;
+  float invS;
   if (sg < NS) {
     float4 xv[8], qv[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) load4(sg * kSegTokens + 128 * i + 4 * lane, xv[i], qv[i]);
+    invS = ff_div_to_f(1.0f, rs.S);  // while the loads are in flight
     float gr[8], gp[8];
-    int lr = -1, lp = -1;
+    auto terms = [&](float t) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int e = sg * kSegTokens + 128 * i + 4 * lane;
-      const float xs[4] = {xv[i].x, xv[i].y, xv[i].z, xv[i].w};
-      const float qs[4] = {qv[i].x, qv[i].y, qv[i].z, qv[i].w};
-      float rr[4], pz[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        draw_terms(xs[u], qs[u], residual, rs.m, tau, invS, rr[u], pz[u]);
-        lr = rr[u] > 0.f ? e + u : lr;
-        lp = pz[u] > 0.f ? e + u : lp;
+      for (int i = 0; i < 8; ++i) {
+        float rr[4], pz[4];
+        draw_terms(xv[i].x, qv[i].x, residual, rs.m, t, invS, rr[0], pz[0]);
+        draw_terms(xv[i].y, qv[i].y, residual, rs.m, t, invS, rr[1], pz[1]);
+        draw_terms(xv[i].z, qv[i].z, residual, rs.m, t, invS, rr[2], pz[2]);
+        draw_terms(xv[i].w, qv[i].w, residual, rs.m, t, invS, rr[3], pz[3]);
+        gr[i] = sum4(rr[0], rr[1], rr[2], rr[3]);
+        gp[i] = sum4(pz[0], pz[1], pz[2], pz[3]);
       }
-      gr[i] = sum4(rr[0], rr[1], rr[2], rr[3]);
-      gp[i] = sum4(pz[0], pz[1], pz[2], pz[3]);
-    }
+    };
+    if (tau == 1.0f) terms(1.0f);
+    else terms(tau);
     const ff Sr = warp_sum_ff(ff_of(__fadd_rn(__fadd_rn(__fadd_rn(gr[0], gr[1]), __fadd_rn(gr[2], gr[3])),
                                               __fadd_rn(__fadd_rn(gr[4], gr[5]), __fadd_rn(gr[6], gr[7])))));
     const ff Sp = warp_sum_ff(ff_of(__fadd_rn(__fadd_rn(__fadd_rn(gp[0], gp[1]), __fadd_rn(gp[2], gp[3])),
                                               __fadd_rn(__fadd_rn(gp[4], gp[5]), __fadd_rn(gp[6], gp[7])))));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lr = max(lr, __shfl_xor_sync(0xffffffffu, lr, o));
-      lp = max(lp, __shfl_xor_sync(0xffffffffu, lp, o));
-    }
-    if (lane == 0) parts[sg] = DrawPart{Sr, Sp, lr, lp, {0, 0}};
+    if (lane == 0) parts[sg] = DrawPart{Sr, Sp};
+  } else {
+    invS = ff_div_to_f(1.0f, rs.S);
   }
 
   // ---- the last CTA of the sequence draws the token ----
   __syncthreads();  // every part of this CTA is written
-  if (tid == 0)     // release this CTA's parts, acquire the others'
+  if (tid == 0) {   // release this CTA's parts, acquire the others'
     s_flag = atom_add_acq_rel_gpu(p.draw_tickets + b, 1u) == static_cast<unsigned>(p.C2 - 1);
+    s_seg = -1;
+    s_token = INT_MAX;
+  }
   __syncthreads();
   if (!s_flag) return;
 
-  auto part_sum = [&](int cc, bool pmass) -> ff {
-    const float4 v = __ldcg(reinterpret_cast<const float4 *>(parts + cc));
-    return pmass ? ff{v.z, v.w} : ff{v.x, v.y};
+  // ---- the segment: thread t owns segments [t per, (t + 1) per), one each up
+  // to V = 262144 ----
+  const int per = (NS + kAccThreads - 1) / kAccThreads, first = tid * per, end = min(NS, first + per);
+  auto part = [&](int at) { return __ldcg(reinterpret_cast<const float4 *>(parts + at)); };
+  const float4 v0 = first < end ? part(first) : make_float4(0.f, 0.f, 0.f, 0.f);
+  bool use_p = false;
+  auto mass = [&](int at) {
+    const float4 v = at == first ? v0 : part(at);
+    return use_p ? ff{v.z, v.w} : ff{v.x, v.y};
   };
-  ff target;
-  bool use_p;
-  int my_last_r = -1, my_last_p = -1;  // one segment per thread: its last indices
-  if (tid == 0) { s_seg = INT_MAX; s_base = ff_of(0.f); }
-  if (NS <= kAccThreads) {
-    // one segment per thread: every part is loaded once, and one scan gives
-    // both the segment intervals and the total (its last inclusive value, so
-    // that the intervals tile [0, total) exactly)
-    float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (tid < NS) {
-      v0 = __ldcg(reinterpret_cast<const float4 *>(parts + tid));
-      my_last_r = __ldcg(&parts[tid].last_r);
-      my_last_p = __ldcg(&parts[tid].last_p);
-    }
-    ff v = ff{v0.x, v0.y};
-    ff excl, total;
-    ff incl = block_inclusive_scan(v, s_scan, &excl, &total);
-    use_p = !ff_pos(total);  // residual with no mass (rounding only)
-    if (use_p) {
-      v = ff{v0.z, v0.w};
-      incl = block_inclusive_scan(v, s_scan, &excl, &total);
-    }
-    target = ff_mul(total, u_k);
-    if (tid < NS && ff_pos(v) && ff_lt(target, incl) && !ff_lt(target, excl)) atomicMin(&s_seg, tid);
-    __syncthreads();
-    if (s_seg == tid) s_base = excl;
-  } else {
-    ff total;
-    {
-      ff pr = ff_of(0.f);
-      for (int cc = tid; cc < NS; cc += kAccThreads) pr = ff_add(pr, part_sum(cc, false));
-      total = block_sum(pr, s_d);
-    }
-    use_p = !ff_pos(total);  // residual with no mass (rounding only)
-    if (use_p) {
-      ff pp = ff_of(0.f);
-      for (int cc = tid; cc < NS; cc += kAccThreads) pp = ff_add(pp, part_sum(cc, true));
-      total = block_sum(pp, s_d);
-    }
-    target = ff_mul(total, u_k);
-    // segment holding the target: inclusive float-float scan over the
-    // segment sums in order; segment cc covers [excl, incl), and excl of cc
-    // is bit-identical to incl of cc - 1, so the intervals tile [0, total)
-    ff carry = ff_of(0.f);
-    for (int base = 0; base < NS; base += kAccThreads) {
-      const int cc = base + tid;
-      const ff v = cc < NS ? part_sum(cc, use_p) : ff_of(0.f);
-      ff excl_local, blk_total;
-      const ff incl_local = block_inclusive_scan(v, s_scan, &excl_local, &blk_total);
-      const ff excl = ff_add(carry, excl_local), incl = ff_add(carry, incl_local);
-      if (cc < NS && ff_pos(v) && ff_lt(target, incl) && !ff_lt(target, excl)) atomicMin(&s_seg, cc);
-      __syncthreads();
-      if (s_seg == cc) s_base = excl;
-      carry = ff_add(carry, blk_total);
-      __syncthreads();
-      if (s_seg != INT_MAX) break;
-    }
+  ff sum, ex, next, total;
+  auto scan_segments = [&]() {
+    sum = ff_of(0.f);
+#pragma unroll 1
+    for (int at = first; at < end; ++at) sum = ff_add(sum, mass(at));
+    ex = block_scan2(sum, s_scan, &total, &next);
+  };
+  scan_segments();
+  if (!ff_pos(total)) {  // residual with no mass (rounding only): the target's row
+    use_p = true;
+    scan_segments();
   }
-  __syncthreads();
-  int token = -1;
-  if (s_seg == INT_MAX) {
-    // u*S at or past the total (rounding): the last token with positive mass
-    int last = -1;
-    if (NS <= kAccThreads) {
-      last = use_p ? my_last_p : my_last_r;
-    } else {
-      for (int cc = tid; cc < NS; cc += kAccThreads)
-        last = max(last, use_p ? __ldcg(&parts[cc].last_p) : __ldcg(&parts[cc].last_r));
+  const ff target = ff_mul(total, u_k);
+  // u S at or past the total (rounding): the last token with mass of all
+  const bool take_last = !ff_lt(target, total);
+  // the thread's first segment whose running sum passes the target (its last
+  // one with mass if rounding leaves none), and the sum before it
+  auto walk = [&]() {
+    ff run = ex;
+#pragma unroll 1
+    for (int at = first; at < end; ++at) {
+      const ff m = mass(at);
+      if (!ff_pos(m)) continue;
+      s_seg = at;
+      s_base = run;
+      run = ff_add(run, m);
+      if (!take_last && ff_lt(target, run)) break;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
-    if (tid == 0) s_token = -1;
+  };
+  const bool here = ff_pos(sum) && (take_last || !ff_lt(target, ex));
+  if (!take_last && here && ff_lt(target, next)) walk();
+  __syncthreads();
+  if (s_seg < 0) {  // take_last, or rounding put the target between two threads' intervals
     __syncthreads();
-    if (lane == 0) atomicMax(&s_token, last);
+    if (here) atomicMax(&s_flag, tid + 1);  // the last thread with mass up to the target; 1 from the ticket
     __syncthreads();
-    token = s_token;
-  } else {
+    if (here && s_flag == tid + 1) walk();
+    __syncthreads();
+  }
+  const int cc = s_seg;
+  int token = -1;
+  if (cc >= 0) {  // uniform over the block
     // the segment in ascending token order: thread t owns tokens 4t .. 4t+3
     // (terms recomputed exactly as in the segment sums)
-    const int cc = s_seg;
     const int e = cc * kSegTokens + 4 * tid;
     float4 xv, qv;
     load4(e, xv, qv);
     const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
     const float qs[4] = {qv.x, qv.y, qv.z, qv.w};
     float t[4];
-    ff mine = ff_of(0.f);
+    int last = -1;  // the thread's last token with mass
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       float rr, pz;
       draw_terms(xs[u], qs[u], residual, rs.m, tau, invS, rr, pz);
       t[u] = use_p ? pz : rr;
-      mine = ff_add(mine, ff_of(t[u]));
+      last = t[u] > 0.f ? e + u : last;
     }
-    ff excl, unused;
-    block_inclusive_scan(mine, s_scan, &excl, &unused);
-    ff cum = ff_add(s_base, excl);
-    if (tid == 0) s_token = INT_MAX;
-    __syncthreads();
+    if (!take_last) {
+      ff all;
+      ff cum = ff_add(s_base, block_scan2(ff_add(two_sum(t[0], t[1]), two_sum(t[2], t[3])), s_scan, &all));
+      int at = INT_MAX;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      cum = ff_add(cum, ff_of(t[u]));
-      if (t[u] > 0.f && ff_lt(target, cum)) {
-        atomicMin(&s_token, e + u);
-        break;
+      for (int u = 0; u < 4; ++u) {
+        cum = ff_add(cum, ff_of(t[u]));
+        if (at == INT_MAX && t[u] > 0.f && ff_lt(target, cum)) at = e + u;
       }
+      at = __reduce_min_sync(0xffffffffu, at);
+      if (lane == 0 && at != INT_MAX) atomicMin(&s_token, at);
+      __syncthreads();
+      token = s_token;
     }
-    __syncthreads();
-    token = s_token;
-    if (token == INT_MAX) {
-      // rounding put the target past the segment's own running sum: its last
-      // positive token
-      token = use_p ? __ldcg(&parts[cc].last_p) : __ldcg(&parts[cc].last_r);
+    if (take_last || token == INT_MAX) {
+      // rounding put the target past the running sum: the last token with mass
+      __syncthreads();  // s_token has been read
+      if (tid == 0) s_token = -1;
+      __syncthreads();
+      last = __reduce_max_sync(0xffffffffu, last);
+      if (lane == 0) atomicMax(&s_token, last);
+      __syncthreads();
+      token = s_token;
     }
   }
   if (tid == 0) {
@@ -889,7 +871,9 @@ accept_draw_kernel(const __grid_constant__ AccParams p) {
 // The warp of the chunk kernel owning chunk u: the largest g with
 // floor(g U / NW) <= u (warps with empty ranges are never returned).
 __device__ __forceinline__ int warp_of(int u, int U, int NW) {
-  return static_cast<int>(((long long)(u + 1) * NW - 1) / U);
+  const unsigned long long n = static_cast<unsigned long long>(u + 1) * static_cast<unsigned>(NW) - 1;
+  if ((n >> 32) == 0) return static_cast<int>(static_cast<uint32_t>(n) / static_cast<uint32_t>(U));
+  return static_cast<int>(n / static_cast<unsigned>(U));
 }
 
 // The 32 tokens of lane `lane` in chunk c of a row: c*1024 + 128 i + 4 lane + t
@@ -917,7 +901,8 @@ __device__ __forceinline__ void load_chunk(const AccParams &p, int row, int c, i
 // it and the float-float sum of exp((x - max)/tau) over them; the warp
 // combines the lanes once, at the end of the run.
 struct RunState {
-  int row, c, start_chunk, len;
+  int row, c, len;
+  int g0, n_runs;    // the row's first warp and its number of runs
   float tau, scale;  // scale = log2(e) / tau, rounded once
   bool greedy;
   float lm;          // lane max
@@ -925,11 +910,12 @@ struct RunState {
   ff lS;             // lane sum, relative to lm
 };
 
-__device__ __forceinline__ void run_begin(const AccParams &p, RunState &st, int row, int c) {
+__device__ __forceinline__ void run_begin(const AccParams &p, RunState &st, int row, int c, int U) {
   st.row = row;
   st.c = c;
-  st.start_chunk = c;
   st.len = 0;
+  st.g0 = warp_of(row * p.C1, U, p.NW1);
+  st.n_runs = warp_of(row * p.C1 + p.C1 - 1, U, p.NW1) - st.g0 + 1;
   st.tau = __ldg(p.tau + row / (p.k + 1));
   st.greedy = !(st.tau > 0.0f);
   st.scale = st.greedy ? 0.f : __fdiv_rn(1.44269504088896341f, st.tau);
@@ -977,12 +963,13 @@ __device__ __forceinline__ void run_chunk(RunState &st, int lane, const float4 (
   ++st.len;
 }
 
-__device__ __forceinline__ RowStat combine_runs(const AccParams &p, int row, float tau,
+__device__ __forceinline__ RowStat combine_runs(const AccParams &p, int row, int n, float tau,
                                                 bool greedy);
 
 // The decisions of sequence b by one warp, from the final row statistics in
-// global memory; leaves j and row j's statistics to the draw kernel.
-__device__ void decide_warp(const AccParams &p, int b) {
+// global memory and the drafts' entries; leaves j and row j's statistics to
+// the draw kernel.
+__device__ __forceinline__ void decide_warp(const AccParams &p, int b, float tau, const DraftEntry &e) {
   const int lane = threadIdx.x & 31, k = p.k;
   float rm = 0.f;
   int rarg = -1;
@@ -993,8 +980,7 @@ __device__ void decide_warp(const AccParams &p, int b) {
     rarg = __float_as_int(v.y);
     rS = ff{v.z, v.w};
   }
-  const DraftEntry e = load_draft(p, b);
-  const Decision d = decide_core(p, b, p.tau[b], rm, rarg, rS, e.tok, e.u, e.lx, e.qx, true);
+  const Decision d = decide_core(p, b, tau, rm, rarg, rS, e.tok, e.u, e.lx, e.qx, true);
   if (lane == 0) p.seqs[b] = SeqState{d.j, d.m, d.S};
 }
 
@@ -1003,13 +989,14 @@ __device__ void decide_warp(const AccParams &p, int b) {
 struct PendingTicket {
   int row;          // -1: none
   int n_runs;       // runs of the row
+  float tau;        // its temperature
   uint32_t ticket;  // lane 0: the row ticket before this warp's add
 };
 
 // Ends the warp's run: combines the lanes, writes the run's record and
 // takes the row's ticket (lane 0; one atomic per run; nobody waits).
 __device__ __forceinline__ PendingTicket run_end(const AccParams &p, const RunState &st, int lane,
-                                                 int gw, int U) {
+                                                 int gw) {
   float wm = st.lm;
   int wi = st.li;
   warp_argmax(wm, wi);
@@ -1019,11 +1006,9 @@ __device__ __forceinline__ PendingTicket run_end(const AccParams &p, const RunSt
     if (ff_pos(st.lS)) mine = ff_mul(st.lS, exp_diff_accurate(st.lm, wm, st.tau));
     S = warp_sum_ff(mine);
   }
-  const int CPR = p.C1;
-  const int g0 = warp_of(st.row * CPR, U, p.NW1);
-  PendingTicket pt{st.row, warp_of(st.row * CPR + CPR - 1, U, p.NW1) - g0 + 1, 0u};
+  PendingTicket pt{st.row, st.n_runs, st.tau, 0u};
   if (lane == 0) {
-    p.runs[(size_t)st.row * CPR + (gw - g0)] = RowStat{wm, wi, S};  // run gw - g0 of its row
+    p.runs[(size_t)st.row * p.C1 + (gw - st.g0)] = RowStat{wm, wi, S};  // run gw - g0 of its row
     // the release covers the record; the acquire, the other runs' records
     pt.ticket = atom_add_acq_rel_gpu(p.row_tickets + pt.row, 1u);
   }
@@ -1037,9 +1022,9 @@ __device__ __forceinline__ void resolve_ticket(const AccParams &p, const Pending
   const bool last = __shfl_sync(0xffffffffu, pt.ticket == static_cast<uint32_t>(pt.n_runs - 1), 0);
   if (!last) return;
   __syncwarp();
-  const float tau = __ldg(p.tau + pt.row / (p.k + 1));
-  const RowStat rs = combine_runs(p, pt.row, tau, !(tau > 0.0f));
   const int b = pt.row / (p.k + 1);
+  const DraftEntry e = load_draft(p, b);  // in flight with the records (used by the last row's warp)
+  const RowStat rs = combine_runs(p, pt.row, pt.n_runs, pt.tau, !(pt.tau > 0.0f));
   uint32_t last_row = 0;
   if (lane == 0) {
     p.rows[pt.row] = rs;
@@ -1048,7 +1033,7 @@ __device__ __forceinline__ void resolve_ticket(const AccParams &p, const Pending
   }
   if (!__shfl_sync(0xffffffffu, last_row, 0)) return;
   __syncwarp();
-  decide_warp(p, b);
+  decide_warp(p, b, pt.tau, e);
   if (lane == 0) p.seq_tickets[b] = 0u;
 }
 
@@ -1080,15 +1065,15 @@ accept_chunks_kernel(const __grid_constant__ AccParams p) {
   const int u1 = static_cast<int>((long long)(gw + 1) * U / p.NW1);
   if (u0 >= u1) return;
   RunState st;
-  run_begin(p, st, u0 / CPR, u0 % CPR);
+  run_begin(p, st, u0 / CPR, u0 % CPR, U);
   // the next chunk: the row boundary ends the run and looks at its ticket
   auto advance = [&](int u) {
     int nrow = st.row, nc = st.c + 1;
     if (nc == CPR) { nc = 0; ++nrow; }
     if (nc == 0 || u + 1 == u1) {
-      const PendingTicket now = run_end(p, st, lane, gw, U);
+      const PendingTicket now = run_end(p, st, lane, gw);
       resolve_ticket(p, now, lane);
-      if (u + 1 < u1) run_begin(p, st, nrow, 0);
+      if (u + 1 < u1) run_begin(p, st, nrow, 0, U);
     } else {
       st.c = nc;
     }
@@ -1177,18 +1162,15 @@ accept_chunks_kernel(const __grid_constant__ AccParams p) {
   }
 }
 
-// Combines the run records of target row `row` (in run order, which is
+// Combines the n run records of target row `row` (in run order, which is
 // chunk order) into the row's max, first argmax and float-float sum rescaled
 // to the max.  Executed by one whole warp; all loads are issued before any
 // is used.
-__device__ __forceinline__ RowStat combine_runs(const AccParams &p, int row, float tau,
+__device__ __forceinline__ RowStat combine_runs(const AccParams &p, int row, int n, float tau,
                                                 bool greedy) {
   constexpr int kPer = 4;  // records per lane and pass
-  const int lane = threadIdx.x & 31, CPR = p.C1;
-  const int U = p.B * (p.k + 1) * CPR;
-  const int g0 = warp_of(row * CPR, U, p.NW1);
-  const int n = warp_of(row * CPR + CPR - 1, U, p.NW1) - g0 + 1;
-  const float4 *rr = reinterpret_cast<const float4 *>(p.runs + (size_t)row * CPR);
+  const int lane = threadIdx.x & 31;
+  const float4 *rr = reinterpret_cast<const float4 *>(p.runs + (size_t)row * p.C1);
   float mv = -INFINITY;
   int mi = INT_MAX;
   ff Sr = ff_of(0.f);

@@ -91,7 +91,7 @@ def test_cluster_path_edges(oracle_mod, B, k, V, mode, temp):
 @pytest.mark.parametrize("mode", ["sampling", "alternate"])
 def test_vocabulary_beyond_256_segments(oracle_mod, V, mode):
     # more than 256 segments of 1024 tokens per row: the draw's last CTA
-    # searches the segment sums block by block (one segment per thread
+    # searches the segment sums several to a thread (one segment per thread
     # otherwise); V % 4 == 0 streams the logits by bulk copies, V % 4 != 0
     # through registers
     _check(oracle_mod, make_accept_case(2, 3, V, seed=V % 97, mode=mode))
@@ -358,3 +358,34 @@ def test_residual_without_mass_draws_from_the_target(oracle_mod, V):
     inp = AcceptInputs(logits, q, tokens, u, np.ones(B, np.float32))
     ref, n, toks = _check(oracle_mod, inp, max_excluded_frac=0.0)
     assert (n == 0).all()
+
+
+@pytest.mark.parametrize("V", [32772, 152064, 262144, 262145, 524289])
+@pytest.mark.parametrize("temp", [1.0, 0.5])
+def test_draw_finds_every_token_of_a_sparse_row(V, temp):
+    # The bonus row has equal mass on n tokens at the edges of segments (1024
+    # tokens), of a CTA's eight segments and of the row, none elsewhere; one
+    # sequence per u in the middle of each token's interval, and u = 0, the
+    # largest float below 1 and 1.  One segment per thread of the last CTA up
+    # to V = 262144, several above.
+    support = sorted({0, 1023, 1024, 1027, 8191, 8192, 20000, 32767, 32768, V // 2, V - 1})
+    n = len(support)
+    u_last = [(i + 0.5) / n for i in range(n)] + [0.0, 1.0 - 2.0 ** -24, 1.0]
+    expected = support + [support[0], support[-1], support[-1]]
+    B, k = len(u_last), 1
+    logits = np.full((B, k + 1, V), -np.inf, np.float32)
+    logits[:, :, support] = 0.25
+    q = np.zeros((B, k, V), np.float32)
+    q[:, 0, support[0]] = 0.5 / n                      # p / q = 2: accepted
+    tokens = np.full((B, k), support[0], np.int32)
+    u = np.stack([np.full(B, 0.5), np.array(u_last)], axis=1).astype(np.float32)
+    n_acc, toks, _ = run_accept(AcceptInputs(logits, q, tokens, u, np.full(B, temp, np.float32)))
+    assert (n_acc == k).all()
+    np.testing.assert_array_equal(toks[:, k], expected)
+    # the residual: q takes all of the first token's mass and rejects it
+    q[:, 0, support[0]] = 4.0 / n
+    u[:, 0] = 0.5
+    u[:, 1] = [(i + 0.5) / (n - 1) for i in range(n - 1)] + [0.0] * (B - n + 1)
+    n_acc, toks, _ = run_accept(AcceptInputs(logits, q, tokens, u, np.full(B, temp, np.float32)))
+    assert (n_acc == 0).all()
+    np.testing.assert_array_equal(toks[:, 0], support[1:] + [support[1]] * (B - n + 1))
