@@ -181,6 +181,20 @@ def test_sample_many_rows_and_unaligned_vocabulary(oracle_mod):
     assert excluded <= 3
 
 
+@pytest.mark.parametrize("V", [131068, 131072, 131073])
+def test_sample_on_both_sides_of_the_streaming_size(oracle_mod, V):
+    # 64 rows: 8 R V bytes is just below, at and above 2^26, from where the
+    # probabilities are stored as streaming data; the last with scalar accesses
+    rng = np.random.default_rng(V)
+    R = 64
+    logits = (2.0 * rng.standard_normal((R, V))).astype(np.float32)
+    tau = np.where(np.arange(R) % 3 == 1, 0.0, np.where(np.arange(R) % 3 == 2, 0.6, 1.0)).astype(np.float32)
+    u = rng.random(R, dtype=np.float32)
+    probs, tokens = run_sample(logits, u, tau)
+    some = np.array([0, 1, 2, 31, 62, 63])
+    check_sampler(oracle_mod, logits[some], u[some], tau[some], probs[some], tokens[some])
+
+
 def test_sample_masked_tokens_and_ties(oracle_mod):
     R, V = 6, 7000
     logits, u, temp = make_sample_case(R, V, seed=5)
