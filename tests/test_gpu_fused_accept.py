@@ -100,6 +100,19 @@ def test_fused_invalid_arguments():
     assert lib.sf_verify_lm_head_accept_workspace_size(1, 5, 32000) > 0
 
 
+@pytest.mark.parametrize("B,k,V", [
+    (1, 1, 128),       # two rows, one record each
+    (3, 15, 4000),     # 16 rows, 32 records: one per lane
+    (2, 16, 4200),     # 17 rows, the most; 33 records
+    (15, 16, 20000),   # 255 rows, a record of every SM
+])
+def test_decisions_with_a_warp_for_each_row(oracle_mod, B, k, V):
+    hidden, weight, inp, ref_logits = make_case(oracle_mod, B, k, V, 64, seed=[B, k, V], mode="alternate")
+    logits, n, toks, ratio = run_fused(hidden, weight, inp)
+    assert np.array_equal(logits.astype(np.float64), ref_logits)
+    assert compare_accept(oracle_accept(oracle_mod, inp), n, toks, ratio) <= max(1, B // 8)
+
+
 @pytest.mark.parametrize("V,d", [(152064, 3584), (32000, 4096)])
 def test_lm_head_then_accept_on_one_stream(oracle_mod, V, d):
     # The target logits written by sf_lm_head are read by sf_accept launched
