@@ -236,47 +236,6 @@ static size_t cluster_smem(int k, int slice, int bufs, bool ahead) {
   return sizeof(float) * static_cast<size_t>(slice) * (bufs + (ahead ? k : 0));
 }
 
-// Inclusive float-float prefix over the first `n` lanes (n a power of two): a
-// lane's exclusive value is the inclusive value of the lane before, bit for bit.
-__device__ __forceinline__ ff warp_scan_ff(ff v, int n, ff *excl) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    if (o >= n) break;
-    const ff t = shfl_up_ff(v, o);
-    if (lane >= o) v = ff_add(t, v);
-  }
-  *excl = shfl_up_ff(v, 1);
-  if (lane == 0) *excl = ff_of(0.f);
-  return v;
-}
-
-__device__ __forceinline__ ff shfl_ff(ff v, int lane) {
-  return ff{__shfl_sync(0xffffffffu, v.hi, lane), __shfl_sync(0xffffffffu, v.lo, lane)};
-}
-
-// The same over the block, with two barriers; returns the thread's exclusive
-// value, and in *next (if asked for) the exclusive value of the thread after
-// it, bit for bit (*total after the last), so that [excl, next) tile [0, total).
-__device__ __forceinline__ ff block_scan2(ff v, ff *s_warp, ff *total, ff *next = nullptr) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  ff ex, wex;
-  v = warp_scan_ff(v, 32, &ex);
-  __syncthreads();  // s_warp may be in use
-  if (lane == 31) s_warp[warp] = v;
-  __syncthreads();
-  const ff w = warp_scan_ff(lane < kAccWarps ? s_warp[lane] : ff_of(0.f), kAccWarps, &wex);
-  *total = shfl_ff(w, kAccWarps - 1);
-  const ff off = shfl_ff(wex, warp);
-  const ff prev = shfl_up_ff(ff_add(off, v), 1);
-  const ff excl = lane > 0 ? prev : off;
-  if (next) {
-    const ff after = shfl_ff(excl, (lane + 1) & 31), warp_end = shfl_ff(w, warp);
-    *next = lane < 31 ? after : warp_end;
-  }
-  return excl;
-}
-
 __global__ void __launch_bounds__(kAccThreads)
 accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, int bufs, int q_ahead) {
   extern __shared__ __align__(128) float s_rows[];  // [bufs][slice], then [k][slice] of q

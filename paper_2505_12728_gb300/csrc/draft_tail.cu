@@ -562,23 +562,30 @@ __global__ void __launch_bounds__(kFfThreads) sample_stats_kernel(const __grid_c
 // token, draws T'.  grid (ceil(V / span), R); dynamic shared memory
 // holds the row's Cn statistics.
 //
-// Warp 0 of every CTA combines the statistics alone, with shuffles instead of
-// block barriers (all lanes' loads in one round trip, one barrier in all),
-// while the other warps' first logits are in flight: with a block-wide
-// combine of ten barriers a wave of CTAs spent 10 us before its first store.
-template <bool kStream>
-__global__ void __launch_bounds__(kFfThreads, kFinishCtasPerSm)
+// Nothing is written before the combination, while the first logits are in
+// flight.  With many CTAs per SM (the other CTAs' work hides it) or few chunks,
+// warp 0 combines alone, with shuffles and one barrier in all (a block-wide
+// combine of ten barriers: 10 us in a wave of CTAs before its first store).
+// With kBlock a thread takes each chunk, with one barrier for the maximum, two
+// for the scan and one for the crossing chunk: with one or two CTAs per SM and
+// the projection's 152 chunks 2.4 us instead of 5.5 (five chunks to a lane, in
+// code that runs cold).
+template <bool kStream, bool kBlock>
+__global__ void __launch_bounds__(kFfThreads, kBlock ? 4 : kFinishCtasPerSm)
 sample_finish_kernel(const __grid_constant__ SampleParams p) {
   extern __shared__ SampStat s_st[];
-  __shared__ ff s_scan[kFfWarps + 1];
-  __shared__ float s_m, s_inv;
-  __shared__ int s_arg, s_cross, s_crossed, s_tok, s_last;
+  __shared__ ff s_scan[kFfWarps];
+  __shared__ float s_m, s_inv, s_wm[kFfWarps];
+  __shared__ int s_arg, s_cross, s_crossed, s_tok, s_last, s_wi[kFfWarps];
   __shared__ ff s_base, s_target;
   constexpr int kBatch = 4;
   constexpr unsigned kAll = 0xffffffffu;
   grid_dependency_wait();  // the statistics and logits come from the previous kernels
   grid_launch_dependents();
-  const int r = blockIdx.y, tid = threadIdx.x;
+  const int r = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float4 rec = kBlock && tid < p.Cn  // this thread's chunk
+                         ? __ldcg(reinterpret_cast<const float4 *>(p.stats + static_cast<size_t>(r) * p.Cn) + tid)
+                         : make_float4(-INFINITY, __int_as_float(INT_MAX), 0.f, 0.f);
   const float *row = p.logits + static_cast<size_t>(r) * p.V;
   float *prow = p.probs + static_cast<size_t>(r) * p.V;
   const float tau = p.tau[r];
@@ -597,90 +604,144 @@ sample_finish_kernel(const __grid_constant__ SampleParams p) {
       if (x < x1) f[j] = load4(x);
     }
   }
-  if (tid < 32) {
-    const int lane = tid;
-    const SampStat *st = p.stats + static_cast<size_t>(r) * p.Cn;
-#pragma unroll 4
-    for (int c = lane; c < p.Cn; c += 32) s_st[c] = st[c];
-    __syncwarp();
-    // lane l owns chunks [c_lo, c_hi), in order
-    const int c_lo = lane * p.Cn / 32, c_hi = (lane + 1) * p.Cn / 32;
+  float m, invS = 0.f;
+  int arg, cs = -1;
+  ff target;
+  bool crossed = false;
+  if constexpr (kBlock) {
+    const float u = p.u[r];
     // row maximum and its first index
-    float m = -INFINITY;
-    int arg = INT_MAX;
-    for (int c = c_lo; c < c_hi; ++c)
-      if (better(s_st[c].m, s_st[c].arg, m, arg)) {
-        m = s_st[c].m;
-        arg = s_st[c].arg;
-      }
+    m = rec.x;
+    arg = __float_as_int(rec.y);
     warp_argmax(m, arg);
-    if (!greedy) {
-      // chunk masses relative to m, and their prefix over the lanes: excl of a
-      // lane is, bit for bit, incl of the lane before
-      ff incl = ff_of(0.f);
-      for (int c = c_lo; c < c_hi; ++c) {
-        const ff w = s_st[c].m == -INFINITY ? ff_of(0.f) : ff_mul(s_st[c].S, term_of(s_st[c].m, m, tau));
-        s_st[c].S = w;
-        incl = ff_add(incl, w);
-      }
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const ff n = shfl_up_ff(incl, o);
-        if (lane >= o) incl = ff_add(n, incl);
-      }
-      const ff prev = shfl_up_ff(incl, 1);
-      const ff total = ff{__shfl_sync(kAll, incl.hi, 31), __shfl_sync(kAll, incl.lo, 31)};
-      const ff target = ff_mul(total, p.u[r]);
-      // the first chunk whose inclusive prefix exceeds the target
-      ff cum = lane > 0 ? prev : ff_of(0.f);
-      ff base = cum;
-      int cand = INT_MAX, lastpos = -1;
-      for (int c = c_lo; c < c_hi; ++c) {
-        const ff w = s_st[c].S;
-        const ff nxt = ff_add(cum, w);
-        if (ff_pos(w)) lastpos = c;
-        if (cand == INT_MAX && ff_lt(target, nxt)) {
-          cand = c;
-          base = cum;
-        }
-        cum = nxt;
-      }
-      const unsigned any = __ballot_sync(kAll, cand != INT_MAX);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) lastpos = max(lastpos, __shfl_xor_sync(kAll, lastpos, o));
-      if (lane == (any ? __ffs(any) - 1 : 0)) {
-        s_crossed = any != 0u;
-        s_cross = any ? cand : lastpos;  // no crossing (u >= 1 or NaN): last positive chunk
-        s_base = base;
-        s_target = target;
-        s_inv = ff_div_to_f(1.f, total);
-      }
-    }
     if (lane == 0) {
-      s_m = m;
-      s_arg = arg;
+      s_wm[warp] = m;
+      s_wi[warp] = arg;
+    }
+    if (tid == 0) {
+      s_cross = -1;
       s_tok = INT_MAX;
       s_last = -1;
     }
+    __syncthreads();
+    m = lane < kFfWarps ? s_wm[lane] : -INFINITY;
+    arg = lane < kFfWarps ? s_wi[lane] : INT_MAX;
+    warp_argmax(m, arg);
+    if (!greedy) {
+      // chunk masses relative to m, and their prefix over the threads
+      const ff mass = rec.x == -INFINITY ? ff_of(0.f) : ff_mul(ff{rec.z, rec.w}, term_of(rec.x, m, tau));
+      ff total, next;
+      const ff ex = block_scan2(mass, s_scan, &total, &next);
+      invS = ff_div_to_f(1.f, total);
+      target = ff_mul(total, u);
+      crossed = ff_lt(target, total);  // not for u >= 1 or NaN: then the last chunk with mass
+      const bool here = ff_pos(mass) && (!crossed || tid == 0 || !ff_lt(target, ex));
+      if (crossed && here && ff_lt(target, next)) {
+        s_cross = tid;
+        s_base = ex;
+      }
+      __syncthreads();
+      if (s_cross < 0) {  // nothing crossed, or rounding put the target between two chunks' intervals
+        if (here) atomicMax(&s_last, tid);
+        __syncthreads();
+        const int owner = s_last;
+        __syncthreads();
+        if (tid == owner) {
+          s_cross = tid;
+          s_base = ex;
+        }
+        if (tid == 0) s_last = -1;
+        __syncthreads();
+      }
+      cs = s_cross;
+    }
+  } else {
+    if (tid < 32) {
+      const SampStat *st = p.stats + static_cast<size_t>(r) * p.Cn;
+#pragma unroll 4
+      for (int c = lane; c < p.Cn; c += 32) s_st[c] = st[c];
+      __syncwarp();
+      // lane l owns chunks [c_lo, c_hi), in order
+      const int c_lo = lane * p.Cn / 32, c_hi = (lane + 1) * p.Cn / 32;
+      // row maximum and its first index
+      m = -INFINITY;
+      arg = INT_MAX;
+      for (int c = c_lo; c < c_hi; ++c)
+        if (better(s_st[c].m, s_st[c].arg, m, arg)) {
+          m = s_st[c].m;
+          arg = s_st[c].arg;
+        }
+      warp_argmax(m, arg);
+      if (!greedy) {
+        // chunk masses relative to m, and their prefix over the lanes: excl of a
+        // lane is, bit for bit, incl of the lane before
+        ff incl = ff_of(0.f);
+        for (int c = c_lo; c < c_hi; ++c) {
+          const ff w = s_st[c].m == -INFINITY ? ff_of(0.f) : ff_mul(s_st[c].S, term_of(s_st[c].m, m, tau));
+          s_st[c].S = w;
+          incl = ff_add(incl, w);
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const ff n = shfl_up_ff(incl, o);
+          if (lane >= o) incl = ff_add(n, incl);
+        }
+        const ff prev = shfl_up_ff(incl, 1);
+        const ff total = ff{__shfl_sync(kAll, incl.hi, 31), __shfl_sync(kAll, incl.lo, 31)};
+        target = ff_mul(total, p.u[r]);
+        // the first chunk whose inclusive prefix exceeds the target
+        ff cum = lane > 0 ? prev : ff_of(0.f);
+        ff base = cum;
+        int cand = INT_MAX, lastpos = -1;
+        for (int c = c_lo; c < c_hi; ++c) {
+          const ff w = s_st[c].S;
+          const ff nxt = ff_add(cum, w);
+          if (ff_pos(w)) lastpos = c;
+          if (cand == INT_MAX && ff_lt(target, nxt)) {
+            cand = c;
+            base = cum;
+          }
+          cum = nxt;
+        }
+        const unsigned any = __ballot_sync(kAll, cand != INT_MAX);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) lastpos = max(lastpos, __shfl_xor_sync(kAll, lastpos, o));
+        if (lane == (any ? __ffs(any) - 1 : 0)) {
+          s_crossed = any != 0u;
+          s_cross = any ? cand : lastpos;  // no crossing (u >= 1 or NaN): last positive chunk
+          s_base = base;
+          s_target = target;
+          s_inv = ff_div_to_f(1.f, total);
+        }
+      }
+      if (lane == 0) {
+        s_m = m;
+        s_arg = arg;
+        s_tok = INT_MAX;
+        s_last = -1;
+      }
+    }
+    __syncthreads();
+    m = s_m;
+    arg = s_arg;
+    if (!greedy) {
+      target = s_target;
+      crossed = s_crossed != 0;
+      cs = s_cross;
+      invS = s_inv;
+    }
   }
-  __syncthreads();
   if (greedy) {
     // one-hot P', T' = the first argmax
-    const int arg = s_arg;
     for (int x = x0 + tid; x < x1; x += kFfThreads) prow[x] = x == arg ? 1.f : 0.f;
     if (tid == 0 && arg >= x0 && arg < x1) p.tokens[r] = arg;
     return;
   }
-  const float m = s_m;
-  const ff target = s_target;
-  const bool crossed = s_crossed != 0;
-  const int cs = s_cross;
 
   // P' for this CTA's span.  Rows are 16-byte aligned and the span a
   // multiple of 4 in the vector path, so a float4 is either wholly inside
   // the span or wholly outside; each thread issues the next kBatch loads
   // before the arithmetic and stores of the current ones.
-  const float invS = s_inv;
   if (p.vec4) {
     constexpr int kStep = 4 * kFfThreads * kBatch;
     for (int base = x0 + 4 * tid; base < x1; base += kStep) {
@@ -726,34 +787,37 @@ sample_finish_kernel(const __grid_constant__ SampleParams p) {
   int lastpos = -1;
   for (int s0 = e0; s0 < e1; s0 += 4 * kFfThreads) {
     float t[4];
-    ff tsum = ff_of(0.f);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int x = s0 + 4 * tid + j;
       t[j] = x < e1 ? term_of(row[x], m, tau) : 0.f;
       if (t[j] > 0.f) lastpos = x;
-      tsum = ff_add(tsum, ff_of(t[j]));
     }
-    ff ex, tot;
-    block_inclusive_scan(tsum, s_scan, &ex, &tot);
+    ff tot;
+    const ff ex = block_scan2(ff_add(two_sum(t[0], t[1]), two_sum(t[2], t[3])), s_scan, &tot);
     if (crossed) {
       ff cum = ff_add(base, ex);
+      int at = INT_MAX;  // the thread's first token past the target
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         cum = ff_add(cum, ff_of(t[j]));
-        if (ff_lt(target, cum)) {
-          atomicMin(&s_tok, s0 + 4 * tid + j);
-          break;
-        }
+        if (at == INT_MAX && ff_lt(target, cum)) at = s0 + 4 * tid + j;
       }
+      at = __reduce_min_sync(kAll, at);
+      if (at != INT_MAX && (tid & 31) == 0) atomicMin(&s_tok, at);
     }
     __syncthreads();
-    if (s_tok != INT_MAX) break;
+    if (s_tok != INT_MAX) {
+      if (tid == 0) p.tokens[r] = s_tok;
+      return;
+    }
     base = ff_add(base, tot);
   }
-  if (lastpos >= 0) atomicMax(&s_last, lastpos);
+  // nothing crossed (rounding, u >= 1 or NaN): the chunk's last token with mass
+  lastpos = __reduce_max_sync(kAll, lastpos);
+  if (lastpos >= 0 && (tid & 31) == 0) atomicMax(&s_last, lastpos);
   __syncthreads();
-  if (tid == 0) p.tokens[r] = s_tok != INT_MAX ? s_tok : s_last;
+  if (tid == 0) p.tokens[r] = s_last;
 }
 
 // ---------------------------------------------------------------------------
@@ -778,10 +842,10 @@ static int lm_setup(const DeviceInfo &dev) {
   cudaError_t e = cudaFuncSetAttribute(lm_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        dev.max_smem_optin);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(sample_finish_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(sample_finish_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kMaxStatChunks * static_cast<int>(sizeof(SampStat)));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(sample_finish_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(sample_finish_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kMaxStatChunks * static_cast<int>(sizeof(SampStat)));
   if (e != cudaSuccess) return fail(SF_ERR_CUDA, "cudaFuncSetAttribute (draft tail): %s", cudaGetErrorString(e));
   done[dev.ordinal] = true;
@@ -948,9 +1012,18 @@ static int launch_finish(SampleParams prm, cudaStream_t stream) {
   if (st != SF_OK) return st;
   prm.span = finish_span(prm.R, prm.V, dev.sm_count);
   const int spans = (prm.V + prm.span - 1) / prm.span;
+  // Projection and sampling of 5 rows, 32000 x 4096 (160 CTAs, 152 chunks) 51.8 ->
+  // 49.3 us, 9 rows, 32000 x 2048 (288 CTAs) 32.4 -> 29.6; beyond two CTAs per SM the
+  // block-wide combination is even or behind (128 rows 73.3 -> 73.6 us), and up to
+  // 32 chunks it has nothing to share out (sampling alone, 5 x 32000: 8.8 -> 9.3).
+  const bool block = prm.Cn > 32 && prm.Cn <= kFfThreads &&
+                     static_cast<long long>(spans) * prm.R <= 2LL * dev.sm_count;
   cudaLaunchConfig_t cfg = pdl_config(dim3(spans, prm.R), dim3(kFfThreads),
-                                      static_cast<size_t>(prm.Cn) * sizeof(SampStat), stream, attr);
-  auto *kernel = 8LL * prm.R * prm.V >= kStreamBytes ? sample_finish_kernel<true> : sample_finish_kernel<false>;
+                                      block ? 0 : static_cast<size_t>(prm.Cn) * sizeof(SampStat), stream, attr);
+  const bool streaming = 8LL * prm.R * prm.V >= kStreamBytes;
+  auto *kernel = block       ? (streaming ? sample_finish_kernel<true, true> : sample_finish_kernel<false, true>)
+                 : streaming ? sample_finish_kernel<true, false>
+                             : sample_finish_kernel<false, false>;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, prm);
   if (e != cudaSuccess) return fail(SF_ERR_CUDA, "sampling launch: %s", cudaGetErrorString(e));
   return SF_OK;

@@ -174,39 +174,45 @@ __device__ inline void block_argmax(float &v, int &i, float *s_v, int *s_i) {
   i = s_i[0];
 }
 
-// Inclusive float-float prefix sum over the block (fixed order).  Returns
-// the thread's inclusive value; *excl receives its exclusive value (the
-// previous thread's inclusive value, bit for bit) and *total the block total
-// (the last thread's inclusive value).  s_buf holds kFfWarps + 1 values.
-__device__ inline ff block_inclusive_scan(ff v, ff *s_buf, ff *excl, ff *total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Inclusive float-float prefix over the first `n` lanes (n a power of two): a
+// lane's exclusive value is the inclusive value of the lane before, bit for bit.
+__device__ __forceinline__ ff warp_scan_ff(ff v, int n, ff *excl) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const ff n = shfl_up_ff(v, o);
-    if (lane >= o) v = ff_add(n, v);
+    if (o >= n) break;
+    const ff t = shfl_up_ff(v, o);
+    if (lane >= o) v = ff_add(t, v);
   }
+  *excl = shfl_up_ff(v, 1);
+  if (lane == 0) *excl = ff_of(0.f);
+  return v;
+}
+
+__device__ __forceinline__ ff shfl_ff(ff v, int lane) {
+  return ff{__shfl_sync(0xffffffffu, v.hi, lane), __shfl_sync(0xffffffffu, v.lo, lane)};
+}
+
+// The same over the block, with two barriers; returns the thread's exclusive
+// value, and in *next (if asked for) the exclusive value of the thread after
+// it, bit for bit (*total after the last), so that [excl, next) tile [0, total).
+__device__ __forceinline__ ff block_scan2(ff v, ff *s_warp, ff *total, ff *next = nullptr) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  ff ex, wex;
+  v = warp_scan_ff(v, 32, &ex);
+  __syncthreads();  // s_warp may be in use
+  if (lane == 31) s_warp[warp] = v;
   __syncthreads();
-  if (lane == 31) s_buf[warp] = v;  // warp totals
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    // warp offsets in sequence: off(w) = ff_add(off(w-1), t(w-1)) is, bit for
-    // bit, the inclusive value of the last thread of warp w-1
-    ff off = ff_of(0.f);
-    for (int w = 0; w < kFfWarps; ++w) {
-      const ff t = s_buf[w];
-      s_buf[w] = off;
-      off = ff_add(off, t);
-    }
-    s_buf[kFfWarps] = off;
+  const ff w = warp_scan_ff(lane < kFfWarps ? s_warp[lane] : ff_of(0.f), kFfWarps, &wex);
+  *total = shfl_ff(w, kFfWarps - 1);
+  const ff off = shfl_ff(wex, warp);
+  const ff prev = shfl_up_ff(ff_add(off, v), 1);
+  const ff excl = lane > 0 ? prev : off;
+  if (next) {
+    const ff after = shfl_ff(excl, (lane + 1) & 31), warp_end = shfl_ff(w, warp);
+    *next = lane < 31 ? after : warp_end;
   }
-  __syncthreads();
-  const ff off = s_buf[warp];
-  const ff incl = ff_add(off, v);
-  const ff prev = shfl_up_ff(incl, 1);
-  *excl = lane > 0 ? prev : off;
-  *total = s_buf[kFfWarps];
-  __syncthreads();  // s_buf is reused by the next call
-  return incl;
+  return excl;
 }
 
 }  // namespace sf

@@ -195,6 +195,34 @@ def test_sample_on_both_sides_of_the_streaming_size(oracle_mod, V):
     check_sampler(oracle_mod, logits[some], u[some], tau[some], probs[some], tokens[some])
 
 
+@pytest.mark.parametrize("R,V", [
+    (1, 65536),    # 32 chunks: one warp combines them
+    (1, 65537),    # 33: a thread for each, scalar accesses
+    (4, 70000),    # the same with several rows
+    (2, 155648),   # 304 CTAs: two per SM
+    (2, 155652),   # 306: one warp again
+    (1, 311296),   # the most chunks that the block combines (152)
+])
+def test_sample_combination_by_a_warp_or_the_block(oracle_mod, R, V):
+    rng = np.random.default_rng(V + R)
+    for u_set in ([0.0, 1.0 - 2.0 ** -24, 0.25, 0.999], list(rng.random(4))):
+        logits = (2.0 * rng.standard_normal((R, V))).astype(np.float32)
+        logits[0, : 5 * 2048] = -np.inf          # chunks without mass, at both ends
+        logits[0, V - 2 * 2048:] = -np.inf
+        tau = np.array([1.0, 0.6, 0.0, 2.0], np.float32)[:R]
+        u = np.array(u_set[:R], np.float32)
+        probs, tokens = run_sample(logits, u, tau)
+        check_sampler(oracle_mod, logits, u, tau, probs, tokens)
+
+
+def test_uniform_of_one_draws_the_last_token_with_mass():
+    for V in (32000, 152064):                    # a warp's combination, the block's
+        logits = np.zeros((2, V), np.float32)
+        logits[:, V - 3000:] = -np.inf
+        _, tokens = run_sample(logits, np.ones(2, np.float32), np.ones(2, np.float32))
+        assert (tokens == V - 3001).all()
+
+
 def test_sample_masked_tokens_and_ties(oracle_mod):
     R, V = 6, 7000
     logits, u, temp = make_sample_case(R, V, seed=5)
