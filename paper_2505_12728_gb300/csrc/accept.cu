@@ -22,7 +22,8 @@
 //    accept_draw_kernel (the residual draw in C2 CTAs per sequence over row
 //    j, the last CTA of a sequence scanning for u_k * S);
 //  * behind the fused LM head, whose projection already left per-CTA row
-//    statistics: accept_decide_kernel then accept_draw_kernel.
+//    statistics: accept_decide_kernel then accept_draw_kernel (small batches
+//    of V <= 16 x 2048: the cluster kernel on the projection's logits).
 // Every launch uses programmatic stream serialisation: a kernel is resident
 // while the previous one drains and waits for it (griddepcontrol.wait)
 // before reading its results.
@@ -1261,6 +1262,22 @@ static int chunks_setup(int device) {
   return SF_OK;
 }
 
+// How the rows of a launch of clusters of cs CTAs lie in shared memory: *bufs of
+// them at a time, and whether the draft rows follow (fetched ahead of the
+// decisions).
+static bool cluster_rows(int B, int k, int V, int cs, int slice, bool vec4, int *bufs) {
+  // Every row in shared memory while the batch's clusters are all resident
+  // so (about 7 clusters of 16 per CTA that an SM holds), else kClusterFewBufs
+  // rows at a time: more clusters per SM are worth a second round of copies
+  // (B = 16, k = 8, V = 32000: 33 us with all nine rows, 26 with five).
+  const size_t sm_bytes = 228 * 1024, fixed = 9 * 1024;  // static and reserved shared memory
+  const int groups = cs > 8 ? 7 : 15 * 8 / cs;
+  const long long resident = groups * static_cast<long long>(sm_bytes / (cluster_smem(k, slice, k + 1, false) + fixed));
+  *bufs = B <= resident || k + 1 < kClusterFewBufs ? k + 1 : kClusterFewBufs;
+  return vec4 && *bufs == k + 1 && 4LL * B * k * V <= kAheadBytes &&
+         cluster_smem(k, slice, *bufs, true) <= static_cast<size_t>(kClusterMostSmem);
+}
+
 static int check_accept_shapes(int B, int k, int V) {
   if (B < 1 || B > SF_MAX_BATCH) return fail(SF_ERR_INVALID_ARG, "B=%d outside [1, %d]", B, SF_MAX_BATCH);
   if (k < 1 || k > SF_MAX_DRAFT) return fail(SF_ERR_INVALID_ARG, "k=%d outside [1, %d]", k, SF_MAX_DRAFT);
@@ -1358,16 +1375,8 @@ int sf_accept(const float *target_logits, const float *draft_probs,
     cudaLaunchConfig_t ccfg = {};
     ccfg.gridDim = dim3(cs, B);
     ccfg.blockDim = dim3(kAccThreads);
-    // Every row in shared memory while the batch's clusters are all resident
-    // so (about 7 clusters of 16 per CTA that an SM holds), else kClusterFewBufs
-    // rows at a time: more clusters per SM are worth a second round of copies
-    // (B = 16, k = 8, V = 32000: 33 us with all nine rows, 26 with five).
-    const size_t sm_bytes = 228 * 1024, fixed = 9 * 1024;  // static and reserved shared memory
-    const int groups = cs > 8 ? 7 : 15 * 8 / cs;
-    const long long resident = groups * static_cast<long long>(sm_bytes / (cluster_smem(k, slice, k + 1, false) + fixed));
-    const int bufs = B <= resident || k + 1 < kClusterFewBufs ? k + 1 : kClusterFewBufs;
-    const bool ahead = prm.vec4 && bufs == k + 1 && 4LL * B * k * V <= kAheadBytes &&
-                       cluster_smem(k, slice, bufs, true) <= static_cast<size_t>(kClusterMostSmem);
+    int bufs = 0;
+    const bool ahead = cluster_rows(B, k, V, cs, slice, prm.vec4 != 0, &bufs);
     ccfg.dynamicSmemBytes = cluster_smem(k, slice, bufs, ahead);
     ccfg.stream = stream;
     ccfg.attrs = cattr;
@@ -1458,8 +1467,27 @@ int sf_verify_lm_head_accept(const void *hidden, const void *weight, const float
     return fail(SF_ERR_WORKSPACE, "workspace has %zu bytes, needs %zu", workspace_bytes, need);
 
   uint8_t *ws = static_cast<uint8_t *>(workspace);
-  SampStat *stats = reinterpret_cast<SampStat *>(ws + lay.total);
+  const bool vec4 = (V % 4 == 0) && aligned(logits, 16) && aligned(draft_probs, 16);
   int Gl = 0;
+  // Where sf_accept is one cluster launch with the draft rows fetched ahead, it
+  // is shorter than the statistics epilogue, the decisions and the draw: the
+  // projection then writes the logits alone.  B = 1, k = 5, V = 32000 54.9 -> 51.3 us,
+  // B = 8, k = 5 58.6 -> 55.4, B = 16, k = 8, V = 8000 34.7 -> 27.8, B = 1, k = 2, V = 2000
+  // 19.0 -> 13.4; not fetched ahead it is longer (B = 2, k = 16, V = 32000 58.1, 61.0 so).
+  int cs = 0, slice = 0, bufs = 0;
+  bool cluster_ok = false;
+  if (cluster_plan(V, &cs, &slice) && cluster_rows(B, k, V, cs, slice, vec4, &bufs)) {
+    st = cluster_setup(cs, &cluster_ok);
+    if (st != SF_OK) return st;
+  }
+  if (cluster_ok) {
+    st = launch_projection_stats(hidden, weight, R, d, V, logits, temperature, k + 1, nullptr,
+                                 reinterpret_cast<uint32_t *>(ws), &Gl, stream);
+    if (st != SF_OK) return st;
+    return sf_accept(logits, draft_probs, draft_tokens, uniforms, temperature, B, k, V, num_accepted, out_tokens,
+                     accept_ratio, workspace, workspace_bytes, stream);
+  }
+  SampStat *stats = reinterpret_cast<SampStat *>(ws + lay.total);
   // target logits and their per-CTA row statistics; row b*(k+1)+i uses tau_b
   st = launch_projection_stats(hidden, weight, R, d, V, logits, temperature, k + 1, stats,
                                reinterpret_cast<uint32_t *>(ws), &Gl, stream);
@@ -1488,7 +1516,7 @@ int sf_verify_lm_head_accept(const void *hidden, const void *weight, const float
   prm.C1 = plan.C1;
   prm.C2 = plan.C2;
   prm.NW1 = 0;
-  prm.vec4 = (V % 4 == 0) && aligned(logits, 16) && aligned(draft_probs, 16);
+  prm.vec4 = vec4;
 
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -113,6 +113,24 @@ def test_decisions_with_a_warp_for_each_row(oracle_mod, B, k, V):
     assert compare_accept(oracle_accept(oracle_mod, inp), n, toks, ratio) <= max(1, B // 8)
 
 
+@pytest.mark.parametrize("B,k,V", [
+    (13, 5, 32000),    # draft rows of 8.32 MB: one cluster launch after the projection
+    (14, 5, 32000),    # 8.96 MB: statistics, decisions and draw
+    (1, 8, 32768),     # the longest rows of a cluster
+    (1, 8, 32772),     # one step beyond
+    (2, 16, 32000),    # rows and draft rows don't fit shared memory together
+    (3, 4, 5001),      # not 16-byte aligned
+    (5, 1, 16),
+])
+def test_routes_behind_the_projection_agree(oracle_mod, B, k, V):
+    hidden, weight, inp, ref_logits = make_case(oracle_mod, B, k, V, 64, seed=[B, k, V, 1], mode="alternate")
+    ref = oracle_accept(oracle_mod, inp)
+    for _ in range(2):
+        logits, n, toks, ratio = run_fused(hidden, weight, inp)
+        assert np.array_equal(logits.astype(np.float64), ref_logits)
+        assert compare_accept(ref, n, toks, ratio) <= max(1, B // 8)
+
+
 @pytest.mark.parametrize("V,d", [(152064, 3584), (32000, 4096)])
 def test_lm_head_then_accept_on_one_stream(oracle_mod, V, d):
     # The target logits written by sf_lm_head are read by sf_accept launched
