@@ -240,24 +240,6 @@ __device__ __forceinline__ void st_dsmem_f32x2(uint32_t remote, float a, float b
                : "memory");
 }
 
-__device__ __forceinline__ void st_dsmem_u32(uint32_t remote, uint32_t v) {
-  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
-}
-
-// Arrival on an mbarrier of another CTA of the cluster (an address obtained
-// with dsmem_addr), releasing this thread's earlier writes, and those ordered
-// before it by a CTA barrier, at cluster scope; mbar_wait_or_abort_cluster
-// acquires them.
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t remote) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
-}
-
-// Orders this thread's generic accesses to shared memory, of any CTA of the
-// cluster, with later accesses through the async proxy (tcgen05, TMA).
-__device__ __forceinline__ void fence_proxy_async() {
-  asm volatile("fence.proxy.async;" ::: "memory");
-}
-
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -273,36 +255,6 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint32_t bar, uint32_t parity
 #pragma unroll 1
     for (int i = 0; i < 64; ++i)
       if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_word) return false;
-    if (global_timer_ns() - t0 > kWaitBudgetNs) {
-      *abort_word = 1;
-      return false;
-    }
-  }
-}
-
-// The same with cluster-scope acquire, for barriers that other CTAs of the
-// cluster arrive on.
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-__device__ __forceinline__ bool mbar_wait_or_abort_cluster(uint32_t bar, uint32_t parity,
-                                                           volatile int *abort_word) {
-  if (mbar_try_wait_cluster(bar, parity)) return true;
-  const unsigned long long t0 = global_timer_ns();
-  while (true) {
-#pragma unroll 1
-    for (int i = 0; i < 64; ++i)
-      if (mbar_try_wait_cluster(bar, parity)) return true;
     if (*abort_word) return false;
     if (global_timer_ns() - t0 > kWaitBudgetNs) {
       *abort_word = 1;
