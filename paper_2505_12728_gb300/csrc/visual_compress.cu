@@ -19,22 +19,22 @@
 //     into ks ranges when F*N has too few 128-row tiles to fill the GPU
 //     (each split writes partial sums); it copies the features after the
 //     dependency wait and leaves them in L2 (evict_last) for 3.;
-//  2. compress_softmax_kernel: one warp per (frame, query) sums the ks
-//     partials in a fixed order, takes the row max, and writes the
-//     unnormalised weights exp(s - max) rounded to bf16 into P [C][F][Np]
-//     (Np = N rounded up to 64, zeros past N) and the sum of the rounded
-//     weights into l [F][C];
+//  2. compress_softmax_kernel: a warp, or a block where there are several
+//     partials, per (frame, query) sums the ks partials in a fixed order;
+//     one warp takes the row max, and writes the unnormalised weights
+//     exp(s - max) rounded to bf16 into P [C][F][Np] (Np = N rounded up to
+//     64, zeros past N) and the sum of the rounded weights into l [F][C];
 //  3. compress_apply_kernel, up to two CTAs per SM, each with some of a frame's
 //     groups of 128 columns: the transposed product O^T = F_V^T P^T as a
 //     pipelined tcgen05 GEMM with M = 128 feature columns (A = the frame's
 //     features, MN-major), N = C padded to 16 (B = P, K-major) and K = 16
 //     tokens, two accumulators in tensor memory.
-// Measured per call (graph of calls over three inputs): 5 x 576 x 4096, C 64:
-// 24.2 -> 17.4 us; 128 x 144 x 3584, C 16: 55.9 -> 47 us; 1 x 576 x 4096:
-// 37.3 -> 14.9 us.  A single launch with a cluster per frame, the scores
-// exchanged through distributed shared memory, was slower (31.7 and 48.9 us):
-// a CTA's 147 KB of partial scores and 74 KB of weights move at ~13 bytes per
-// clock.  Computing the weights in the third kernel instead of the second:
+// Measured per call (graph of calls over three inputs), against a CTA per 128
+// columns and one softmax warp per query: 5 x 576 x 4096, C 64: 23.6 -> 16.4 us;
+// 128 x 144 x 3584, C 16: 55.9 -> 46.6; 1 x 576 x 4096, C 64: 36.9 -> 14.5.
+// A single launch with a cluster per frame, the scores exchanged through
+// distributed shared memory, was slower (31.7 and 48.9 us): a CTA's 147 KB of
+// partial scores and 74 KB of weights move at ~13 bytes per clock.  Computing the weights in the third kernel instead of the second:
 // 46.1 us for the video shape, 66.6 for the images.
 // N is at most 768 and C at most 128.  Every wait is bounded
 // (SF_DEVICE_TIMEOUT).
@@ -55,8 +55,7 @@ constexpr int kVcTokens = 64;       // tokens per box of weights (128 bytes)
 constexpr int kVcMaxTokens = 768;   // N
 constexpr int kVcMaxQueries = 128;  // C
 constexpr int kVcMaxStages = 8;
-constexpr int kVcMaxSplits = 4;      // partial scores that the softmax adds
-constexpr int kVcSoftmaxWarps = 2;
+constexpr int kVcSoftmaxWarpThreads = 64;  // softmax CTA where a warp takes a query
 
 struct VcSoftmaxParams {
   const float *scores;  // [ks][C][F*N]
@@ -82,55 +81,67 @@ static size_t vc_smem_bytes(int stages, uint32_t stage_bytes, int C) {
   return 1024 + static_cast<size_t>(stages) * stage_bytes + 8 * (2 * stages + 5) + 64 + 4 * C;
 }
 
-// grid (F, ceil(C / 2)), 64 threads, one warp per query: the partial scores
-// summed in split order, then the unnormalised weights exp(s - max) rounded to
-// bf16, two tokens (64 i + 2 lane and the next) at a time, zeros past N.
-// Bound by memory round trips: every load of the row is in flight at once
-// (loads of one partial behind the sums of the one before: 17.6 us alone for
-// 5 x 576 x 4096, C 64, against 6.5), so there are at most kVcMaxSplits
-// partials; with up to 30 per score a single image took 31 us instead of 15.
-__global__ void __launch_bounds__(32 * kVcSoftmaxWarps)
+// One query of one frame: the partial scores summed in split order, then the
+// unnormalised weights exp(s - max) rounded to bf16, zeros past N, and their
+// sum l.  Threads: kT share the partials' loads and sums, then the query's first
+// warp goes on alone, lane t with tokens 64 i + 2 t and the next.  l is added as
+// 32 chains (chain t: tokens t, t + 32, ...) and a tree over them.  Neither order
+// depends on kT.
+// Bound by memory round trips, so kFly partials of every token of a thread are in
+// flight at once (loads of one partial behind the sums of the one before: 17.6
+// us alone for 5 x 576 x 4096, C 64).  grid (F, queries / those of a CTA).
+template <int kT>
+__global__ void __launch_bounds__(kT > 32 ? kT : kVcSoftmaxWarpThreads)
 compress_softmax_kernel(const __grid_constant__ VcSoftmaxParams p) {
-  constexpr int kPairs = kVcMaxTokens / 64, kFly = kVcMaxSplits - 1;
+  constexpr int kPairs = kVcMaxTokens / 64;                // token pairs per lane of the first warp
+  constexpr int kOwn = kVcMaxTokens / kT;                  // tokens whose partials a thread adds
+  constexpr int kFly = 72 / kOwn;                          // partials in flight
+  constexpr int kQueries = kT > 32 ? 1 : kVcSoftmaxWarpThreads / kT;  // per CTA
+  constexpr unsigned kAll = 0xffffffffu;
+  __shared__ float2 s_x[kT > 32 ? kVcMaxTokens / 2 : 1];
   grid_dependency_wait();  // the partial scores come from the projection
   grid_launch_dependents();
-  const int f = blockIdx.x, c = blockIdx.y * kVcSoftmaxWarps + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
+  const int f = blockIdx.x, c = blockIdx.y * kQueries + threadIdx.x / kT;
+  const int t = threadIdx.x % kT, lane = threadIdx.x & 31;
   if (c >= p.C) return;
   const float *row = p.scores + static_cast<long long>(c) * p.F * p.N + static_cast<long long>(f) * p.N;
-  float x[kPairs], y[kPairs];
+  auto token = [&](int i) { return kT > 32 ? t + kT * i : 64 * (i / 2) + 2 * t + i % 2; };
+  float x[2 * kPairs];
 #pragma unroll
-  for (int i = 0; i < kPairs; ++i) {
-    const int n = 64 * i + 2 * lane;
-    x[i] = n < p.N ? __ldg(row + n) : -INFINITY;
-    y[i] = n + 1 < p.N ? __ldg(row + n + 1) : -INFINITY;
-  }
+  for (int i = 0; i < kOwn; ++i) x[i] = token(i) < p.N ? __ldg(row + token(i)) : -INFINITY;
+#pragma unroll 1
   for (int s0 = 1; s0 < p.ks; s0 += kFly) {
-    float vx[kFly][kPairs], vy[kFly][kPairs];
+    float v[kFly][kOwn];
 #pragma unroll
     for (int u = 0; u < kFly; ++u) {
       const float *part = row + (s0 + u) * p.part_stride;
 #pragma unroll
-      for (int i = 0; i < kPairs; ++i) {
-        const int n = 64 * i + 2 * lane;
-        vx[u][i] = s0 + u < p.ks && n < p.N ? __ldg(part + n) : 0.f;
-        vy[u][i] = s0 + u < p.ks && n + 1 < p.N ? __ldg(part + n + 1) : 0.f;
-      }
+      for (int i = 0; i < kOwn; ++i)
+        v[u][i] = s0 + u < p.ks && token(i) < p.N ? __ldg(part + token(i)) : 0.f;
     }
 #pragma unroll
     for (int u = 0; u < kFly; ++u) {
 #pragma unroll
-      for (int i = 0; i < kPairs; ++i) {
-        x[i] += vx[u][i];
-        y[i] += vy[u][i];
-      }
+      for (int i = 0; i < kOwn; ++i) x[i] += v[u][i];
+    }
+  }
+  if constexpr (kT > 32) {
+#pragma unroll
+    for (int i = 0; i < kOwn; ++i) reinterpret_cast<float *>(s_x)[token(i)] = x[i];
+    __syncthreads();
+    if (t >= 32) return;
+#pragma unroll
+    for (int i = 0; i < kPairs; ++i) {
+      const float2 pair = s_x[32 * i + lane];
+      x[2 * i] = pair.x;
+      x[2 * i + 1] = pair.y;
     }
   }
   float m = -INFINITY;
 #pragma unroll
-  for (int i = 0; i < kPairs; ++i) m = fmaxf(m, fmaxf(x[i], y[i]));
+  for (int i = 0; i < 2 * kPairs; ++i) m = fmaxf(m, x[i]);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
   constexpr float kLog2e = 1.4426950408889634f;
   const float mb = m * kLog2e;
   uint32_t *prow = reinterpret_cast<uint32_t *>(p.P + static_cast<long long>(c) * p.F * p.Np +
@@ -140,14 +151,18 @@ compress_softmax_kernel(const __grid_constant__ VcSoftmaxParams p) {
   for (int i = 0; i < kPairs; ++i) {
     const int n = 64 * i + 2 * lane;
     if (64 * i < p.Np) {
-      const __nv_bfloat162 w = __floats2bfloat162_rn(n < p.N ? fast_exp2(fmaf(x[i], kLog2e, -mb)) : 0.f,
-                                                     n + 1 < p.N ? fast_exp2(fmaf(y[i], kLog2e, -mb)) : 0.f);
-      l += __low2float(w) + __high2float(w);
-      prow[32 * i + lane] = *reinterpret_cast<const uint32_t *>(&w);
+      const __nv_bfloat162 w = __floats2bfloat162_rn(n < p.N ? fast_exp2(fmaf(x[2 * i], kLog2e, -mb)) : 0.f,
+                                                     n + 1 < p.N ? fast_exp2(fmaf(x[2 * i + 1], kLog2e, -mb)) : 0.f);
+      const uint32_t bits = *reinterpret_cast<const uint32_t *>(&w);
+      prow[32 * i + lane] = bits;
+      // chain `lane`: tokens 64 i + lane and 64 i + 32 + lane
+      const uint32_t w0 = __shfl_sync(kAll, bits, lane >> 1), w1 = __shfl_sync(kAll, bits, 16 + (lane >> 1));
+      l += __uint_as_float(lane & 1 ? w0 & 0xffff0000u : w0 << 16);
+      l += __uint_as_float(lane & 1 ? w1 & 0xffff0000u : w1 << 16);
     }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(kAll, l, o);
   if (lane == 0) p.l[f * p.C + c] = l;
 }
 
@@ -373,7 +388,6 @@ struct VcLayout {
 static VcLayout vc_layout(int F, int N, int C, int d, int sm_count) {
   VcLayout L;
   L.ks = projection_splits(F * N, d, sm_count);
-  if (L.ks > kVcMaxSplits) L.ks = kVcMaxSplits;
   const int Np = (N + kVcTokens - 1) / kVcTokens * kVcTokens;
   size_t off = 256;
   L.scores = off;
@@ -460,10 +474,22 @@ int sf_visual_compress(const void *queries, const void *features, int F, int N, 
   sp.N = N;
   sp.C = C;
   sp.Np = Np;
-  cfg.gridDim = dim3(F, (C + kVcSoftmaxWarps - 1) / kVcSoftmaxWarps);
-  cfg.blockDim = dim3(32 * kVcSoftmaxWarps);
+  // Threads per query: the fewest that have all partials in flight at once
+  // (kFly + 1: 4, 13 or 25), or 256.  Whole calls: 5 x
+  // 576 x 4096, C 64 (6 partials) 128 threads 16.4 us, 256 17.2; 1 x 576 x 4096
+  // (30) 14.5, 15.0 with 128.  Few partials: 128 threads as long as the CTAs fit the
+  // GPU at once (8 x 576 x 4096, C 64, 4 partials: 20.0, 20.7 with a warp per query),
+  // else the warp (310 x 20 x 768, C 3: 15.4, 16.1 with 128 threads).
+  const bool one_wave = static_cast<long long>(F) * C <= 5LL * dev.sm_count;
+  const int threads = L.ks <= 1 || (L.ks <= 4 && !one_wave) ? 32 : (L.ks <= 13 ? 128 : 256);
+  const int per_cta = threads == 32 ? kVcSoftmaxWarpThreads / 32 : 1;  // queries
+  cfg.gridDim = dim3(F, (C + per_cta - 1) / per_cta);
+  cfg.blockDim = dim3(per_cta * threads);
   cfg.dynamicSmemBytes = 0;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, compress_softmax_kernel, sp);
+  void (*softmax)(const VcSoftmaxParams) = threads == 32    ? compress_softmax_kernel<32>
+                                           : threads == 128 ? compress_softmax_kernel<128>
+                                                            : compress_softmax_kernel<256>;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, softmax, sp);
   if (e != cudaSuccess) return fail(SF_ERR_CUDA, "compressor softmax launch: %s", cudaGetErrorString(e));
 
   // 3. O^T = F_V^T P^T per (128 columns, frame), divided by l

@@ -13,7 +13,7 @@ import torch
 
 from paper_2505_12728_gb300 import specflash_verify as sfv
 from paper_2505_12728_gb300.workloads import (COMPRESS_SHAPES, bf16_bits_to_f32,
-                                              make_compress_case)
+                                              f32_to_bf16_bits, make_compress_case)
 from tests.gpu_helpers import bf16_tensor, require_gpu
 
 pytestmark = pytest.mark.gpu
@@ -71,7 +71,9 @@ def test_compressor_matches_oracle(oracle_mod, F, N, C, d):
     (40, 97, 17, 1152),     # the first two-slot frame (a 64-token slot, then 33), 7 or 8 CTAs per frame
     (2, 96, 16, 256),       # the longest one-slot frame (weights in two boxes)
     (3, 65, 16, 128),       # one token in the second box of weights
-    (1, 129, 33, 4096),     # four hidden-range partials per score (the most)
+    (1, 129, 33, 4096),     # 64 hidden-range partials per score (the most), three rounds of loads
+    (1, 768, 7, 4096),      # 25 partials of the longest frame: a block of 256 per query, one round
+    (2, 768, 128, 1024),    # 12 partials: a block of 128 per query
 ])
 def test_compressor_at_slot_and_split_edges(oracle_mod, F, N, C, d):
     q, f = make_compress_case(F, N, C, d, seed=[F, N, C, d, 1])
@@ -79,6 +81,30 @@ def test_compressor_at_slot_and_split_edges(oracle_mod, F, N, C, d):
     frames = np.unique(np.linspace(0, F - 1, 4).astype(int))
     ref = oracle_mod.visual_compress(q, f[frames])
     assert (np.abs(got[frames] - ref) <= bound(f[frames], ref)).all()
+
+
+@pytest.mark.parametrize("N", [
+    32,     # a CTA for every 64 hidden columns: 64 partials per score
+    640,    # five row groups: 30 partials, two or three of those ranges each
+    1600,   # 13 groups (4 frames): 11 partials
+])
+def test_scores_add_the_hidden_ranges_in_order(oracle_mod, N):
+    """A score's partial sums are those of SM count / row groups hidden ranges,
+    added in order: 2^26 in one range and -2^26 in an earlier one cancel before
+    the 3 of a later range is added, which any range holding 2^26 and 3
+    together would lose (the spacing of fp32 there is 8)."""
+    d, KC, F = 4096, 64, 1 if N <= 768 else 4
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ks = min(KC, sms // -(-N // 128))
+    first = [s * KC // ks for s in range(ks)]          # first chunk of 64 columns of each range
+    cols = [64 * first[s] for s in (0, ks // 2, ks // 2 + 1)]
+    q = np.zeros((3, d), np.float32)
+    f = np.zeros((F, N // F, d), np.float32)
+    q[:, cols] = [2.0 ** 13, 2.0 ** 13, 3.0]
+    f[:, 5, cols] = [-(2.0 ** 13), 2.0 ** 13, 1.0]
+    got, _ = check(oracle_mod, f32_to_bf16_bits(q), f32_to_bf16_bits(f))
+    want = np.exp(3.0) / (np.exp(3.0) + N // F - 1)    # the weight of token 5
+    assert np.abs(got[:, :, cols[2]] - want).max() <= 2.0 ** -7 * want
 
 
 def test_frames_do_not_reach_into_one_another():
