@@ -40,6 +40,7 @@
 #include <cmath>
 #include <mutex>
 
+#include "chunk_split.h"
 #include "ff_math.cuh"
 #include "sf_device.cuh"
 #include "sf_host.h"
@@ -853,7 +854,7 @@ accept_draw_kernel(const __grid_constant__ AccParams p) {
 // running state (max, first index, float-float sum of exp((x - max)/tau)).
 // At the end of each run of chunks of one row the warp combines its lanes
 // and writes one run record; the runs of row R are stored in warp order, so
-// that run t of the row is the one of warp warp_of(R C1) + t.
+// that run t of the row is the one of warp chunk_owner(R C1) + t.
 //
 // The warp that writes a row's last run record (a ticket per row) combines
 // the row's runs in run order into its final statistics; the warp that
@@ -861,14 +862,6 @@ accept_draw_kernel(const __grid_constant__ AccParams p) {
 // decisions.  accept_draw_kernel, grid (C2, B), then draws the token of row
 // j for the sampled sequences.
 // --------------------------------------------------------------------------
-
-// The warp of the chunk kernel owning chunk u: the largest g with
-// floor(g U / NW) <= u (warps with empty ranges are never returned).
-__device__ __forceinline__ int warp_of(int u, int U, int NW) {
-  const unsigned long long n = static_cast<unsigned long long>(u + 1) * static_cast<unsigned>(NW) - 1;
-  if ((n >> 32) == 0) return static_cast<int>(static_cast<uint32_t>(n) / static_cast<uint32_t>(U));
-  return static_cast<int>(n / static_cast<unsigned>(U));
-}
 
 // The 32 tokens of lane `lane` in chunk c of a row: c*1024 + 128 i + 4 lane + t
 // (tokens at or past V read as -inf).
@@ -908,8 +901,8 @@ __device__ __forceinline__ void run_begin(const AccParams &p, RunState &st, int 
   st.row = row;
   st.c = c;
   st.len = 0;
-  st.g0 = warp_of(row * p.C1, U, p.NW1);
-  st.n_runs = warp_of(row * p.C1 + p.C1 - 1, U, p.NW1) - st.g0 + 1;
+  st.g0 = chunk_owner(row * p.C1, U, p.NW1);
+  st.n_runs = chunk_owner(row * p.C1 + p.C1 - 1, U, p.NW1) - st.g0 + 1;
   st.tau = __ldg(p.tau + row / (p.k + 1));
   st.greedy = !(st.tau > 0.0f);
   st.scale = st.greedy ? 0.f : __fdiv_rn(1.44269504088896341f, st.tau);
@@ -1053,9 +1046,9 @@ accept_chunks_kernel(const __grid_constant__ AccParams p) {
   const int gw = blockIdx.x * kAccWarps + warp;
   const int CPR = p.C1;
   const int U = p.B * (p.k + 1) * CPR;  // < 2^31: the host checks V * (k + 1) and B
-  const int u0 = static_cast<int>((long long)gw * U / p.NW1);
-  const int u1 = static_cast<int>((long long)(gw + 1) * U / p.NW1);
-  if (u0 >= u1) return;
+  const ChunkRange range = chunk_range(gw, U, p.NW1);
+  const int u0 = range.u0, u1 = range.u1;
+  if (u0 >= u1) return;  // a warp that fills up the last CTA
   RunState st;
   run_begin(p, st, u0 / CPR, u0 % CPR, U);
   // the next chunk: the row boundary ends the run and looks at its ticket
@@ -1395,13 +1388,9 @@ int sf_accept(const float *target_logits, const float *draft_probs,
   DeviceInfo dev;
   st = current_device(&dev);
   if (st != SF_OK) return st;
-  // at most one warp per chunk, so that every warp owns at least one chunk
-  // (a row's runs are then exactly the warps between its first and last
-  // chunk's owners), and at most two CTAs per SM
-  const long long units = (long long)B * (k + 1) * plan.C1;
-  long long nw = units < 2LL * dev.sm_count * kAccWarps ? units : 2LL * dev.sm_count * kAccWarps;
-  const long long ctas = (nw + kAccWarps - 1) / kAccWarps;
-  prm.NW1 = static_cast<int>(nw);
+  // at most two CTAs per SM
+  prm.NW1 = chunk_warps((long long)B * (k + 1) * plan.C1, 2LL * dev.sm_count * kAccWarps);
+  const int ctas = (prm.NW1 + kAccWarps - 1) / kAccWarps;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(ctas));
   cfg.blockDim = dim3(kAccThreads);

@@ -389,3 +389,41 @@ def test_draw_finds_every_token_of_a_sparse_row(V, temp):
     n_acc, toks, _ = run_accept(AcceptInputs(logits, q, tokens, u, np.full(B, temp, np.float32)))
     assert (n_acc == 0).all()
     np.testing.assert_array_equal(toks[:, 0], support[1:] + [support[1]] * (B - n + 1))
+
+
+@pytest.mark.parametrize("B,k,V", [
+    (1, 4, 152064),   # 745 chunks: the last CTA has one warp with a chunk, seven without
+    (1, 1, 33001),    # 66 chunks, scalar loads
+    (2, 2, 50000),    # 294 chunks
+])
+def test_part_filled_last_cta_stays_inside_its_buffers(oracle_mod, B, k, V):
+    # Fewer chunks than the GPU has warps, and not a multiple of a CTA's eight.
+    # Inputs and outputs are slices of larger tensors, with values beside them
+    # that would show (a NaN that is read, a canary that is written), over enough
+    # calls on one workspace for stray tickets to complete a row that isn't there.
+    inp = make_accept_case(B, k, V, seed=[B, k, V], mode="sampling")
+    dev = accept_to_device(inp)
+    pad = 64
+
+    def inner(t, fill):
+        buf = torch.full((t.numel() + 2 * pad,), fill, dtype=t.dtype, device="cuda")
+        buf[pad:-pad] = t.flatten()
+        return buf, buf[pad:-pad].view(t.shape)
+
+    dev = {name: inner(t, float("nan") if t.is_floating_point() else 1 << 30)[1] for name, t in dev.items()}
+    outs = {"num_accepted": torch.zeros(B, dtype=torch.int32), "out_tokens": torch.zeros(B, k + 1, dtype=torch.int32),
+            "accept_ratio": torch.zeros(B, k)}
+    bufs = {name: inner(t.cuda(), -7) for name, t in outs.items()}
+    ws = sfv.new_workspace(sfv.accept_workspace_size(B, k, V))
+    for _ in range(300):
+        sfv.accept(**dev, **{name: view for name, (_, view) in bufs.items()}, workspace=ws)
+    torch.cuda.synchronize()
+    ref = oracle_accept(oracle_mod, inp)
+    n, toks, ratio = (bufs[name][1].cpu().numpy() for name in ("num_accepted", "out_tokens", "accept_ratio"))
+    assert compare_accept(ref, n, toks, ratio) == 0
+    for buf, _ in bufs.values():
+        assert (buf[:pad] == -7).all() and (buf[-pad:] == -7).all()
+    assert sfv.read_device_status(ws) == 0
+    # the tickets, per sequence, per row and per sequence, each rounded up to 256 bytes, are all zero again
+    tickets = 256 * (2 * -(-4 * B // 256) + -(-4 * B * (k + 1) // 256))
+    assert not ws[256:256 + tickets].any()
