@@ -818,20 +818,21 @@ __device__ void draw_residual(const AccParams &p, int b, int c, int j, RowStat r
   }
 }
 
-
 __global__ void __launch_bounds__(kAccThreads, 3)
 accept_draw_kernel(const __grid_constant__ AccParams p) {
   // The previous kernel (the decision kernel of this call) lets this grid
   // start only after it has itself waited for the kernel before the call, so
   // the call's inputs (temperature, uniforms) are in place already; j and
-  // the row statistics are waited for.
+  // the row statistics are waited for.  Every CTA waits, those of greedy
+  // sequences too: the kernel after this one waits for this grid alone, and may
+  // use the call's buffers only once the decisions are complete.
   grid_launch_dependents();
   const int c = blockIdx.x, b = blockIdx.y;
   const int k = p.k;
   const float tau = p.tau[b];
-  if (!(tau > 0.0f)) return;  // greedy sequences are complete
   const float u_k = p.u[(size_t)b * (k + 1) + k];
-  grid_dependency_wait();     // j and row j's statistics come from the previous kernel
+  grid_dependency_wait();
+  if (!(tau > 0.0f)) return;  // greedy sequences are complete
   const int4 sq = __ldcg(reinterpret_cast<const int4 *>(p.seqs + b));
   const int j = sq.x;
   if (j < 0 || j > k) {       // no decision was written (a timed-out statistics pass)

@@ -427,3 +427,37 @@ def test_part_filled_last_cta_stays_inside_its_buffers(oracle_mod, B, k, V):
     # the tickets, per sequence, per row and per sequence, each rounded up to 256 bytes, are all zero again
     tickets = 256 * (2 * -(-4 * B // 256) + -(-4 * B * (k + 1) // 256))
     assert not ws[256:256 + tickets].any()
+
+
+@pytest.mark.parametrize("V", [40000, 40001])
+@pytest.mark.parametrize("graph", [False, True])
+def test_greedy_calls_back_to_back_on_one_workspace(oracle_mod, V, graph):
+    # No sequence draws, so the draw kernel has nothing to do; it must still not
+    # let the next call at the workspace before the decisions are complete.
+    cases = [make_accept_case(2, 3, V, seed=[V, i], mode="greedy") for i in range(12)]
+    devs = [accept_to_device(c) for c in cases]
+    outs = [dict(num_accepted=torch.empty(2, dtype=torch.int32, device="cuda"),
+                 out_tokens=torch.empty((2, 4), dtype=torch.int32, device="cuda"),
+                 accept_ratio=torch.empty((2, 3), device="cuda")) for _ in cases]
+    ws = sfv.new_workspace(sfv.accept_workspace_size(2, 3, V))
+
+    def calls():
+        for d, o in zip(devs, outs):
+            sfv.accept(**d, **o, workspace=ws)
+
+    calls()
+    torch.cuda.synchronize()
+    if graph:
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            calls()
+    for _ in range(30):
+        for o in outs:
+            for t in o.values():
+                t.fill_(-9)
+        g.replay() if graph else calls()
+    torch.cuda.synchronize()
+    for c, o in zip(cases, outs):
+        n, toks, ratio = (t.cpu().numpy() for t in o.values())
+        assert compare_accept(oracle_accept(oracle_mod, c), n, toks, ratio) == 0
+    assert sfv.read_device_status(ws) == 0

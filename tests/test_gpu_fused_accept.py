@@ -158,3 +158,20 @@ def test_lm_head_then_accept_on_one_stream(oracle_mod, V, d):
         assert np.array_equal(logits.cpu().numpy().reshape(B, k1, V).astype(np.float64), ref_logits)
         assert sfv.read_device_status(ws_acc) == 0
         compare_accept(ref, n.cpu().numpy(), toks.cpu().numpy(), ratio.cpu().numpy())
+
+
+def test_greedy_calls_back_to_back_on_one_workspace(oracle_mod):
+    # the next call's projection overwrites the logits and statistics that the
+    # decisions of this one read
+    B, k, V, d = 2, 3, 40000, 64
+    cases = [make_case(oracle_mod, B, k, V, d, seed=[V, i], mode="greedy") for i in range(6)]
+    devs = [(bf16_tensor(h), bf16_tensor(w), *(torch.from_numpy(a).cuda() for a in (
+        inp.draft_probs, inp.draft_tokens, inp.uniforms, inp.temperature))) for h, w, inp, _ in cases]
+    ws = sfv.new_workspace(sfv.verify_lm_head_accept_workspace_size(B, k, V))
+    logits = torch.empty((B, k + 1, V), device="cuda")  # shared, as the workspace
+    for _ in range(20):
+        outs = [sfv.verify_lm_head_accept(*dev, logits=logits, workspace=ws)[1:] for dev in devs]
+    torch.cuda.synchronize()
+    assert sfv.read_device_status(ws) == 0
+    for (_, _, inp, _), out in zip(cases, outs):
+        assert compare_accept(oracle_accept(oracle_mod, inp), *(t.cpu().numpy() for t in out)) == 0
