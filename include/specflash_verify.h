@@ -244,7 +244,9 @@ int sf_accept(const float *target_logits, const float *draft_probs,
 /* fp32 accumulate), then exactly the rule of sf_accept, with the rows'     */
 /* max, argmax and softmax sums reduced in the projection's epilogue        */
 /* instead of a second pass over the logits, except at small sizes, where   */
-/* sf_accept's single launch after the projection is shorter.               */
+/* sf_accept's single launch after the projection is shorter; the softmax   */
+/* sums have the same precision there (terms of expf on a float-float       */
+/* difference, added in float-float).                                       */
 /*                                                                           */
 /* hidden        bf16 [B][k+1][d], 16-byte aligned.                          */
 /* weight        bf16 [V][d] (the target's LM head), 16-byte aligned.        */

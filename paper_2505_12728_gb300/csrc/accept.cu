@@ -238,6 +238,14 @@ static size_t cluster_smem(int k, int slice, int bufs, bool ahead) {
   return sizeof(float) * static_cast<size_t>(slice) * (bufs + (ahead ? k : 0));
 }
 
+// kExact (behind the fused LM head): the row sums have the precision of the
+// projection's statistics, which other sizes use there: terms of expf on a
+// float-float difference, each added in float-float.  A slice's sum is scaled to
+// the row's maximum by a float-float factor, since at most 16 factors, and not
+// 152, average their errors.  Acceptance ratios against 64 bits, 40594 of nine
+// sizes and three temperatures (rms / largest error): the statistics 5.7e-8 /
+// 2.3e-7, this 5.7e-8 / 2.3e-7; the sums of sf_accept 7.4e-8 / 2.5e-7.
+template <bool kExact>
 __global__ void __launch_bounds__(kAccThreads)
 accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, int bufs, int q_ahead) {
   extern __shared__ __align__(128) float s_rows[];  // [bufs][slice], then [k][slice] of q
@@ -317,6 +325,9 @@ accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, in
     }
   }
   bool landed = true;  // every copy waited for so far
+  auto sum8 = [](const float (&t)[8]) {
+    return ff_add(ff_add(two_sum(t[0], t[1]), two_sum(t[2], t[3])), ff_add(two_sum(t[4], t[5]), two_sum(t[6], t[7])));
+  };
 
   // ---- 2. the slice's statistics: warp w takes tokens [256 w, 256 w + 256)
   // of every row, lane l tokens 128 h + 4 l .. + 3 of them ----
@@ -364,15 +375,28 @@ accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, in
         const float ref = m == -INFINITY ? 0.f : m;  // all masked: every term is 0
         float v[8];
         load8(i, v);
+        ff S;
+        if constexpr (kExact) {
+          if (tau == 1.0f) {  // one branch for all: the divisions are skipped together
 #pragma unroll
-        for (int t = 0; t < 8; ++t) v[t] = __fsub_rn(v[t], ref);
-        if (tau != 1.0f) {
+            for (int t = 0; t < 8; ++t) v[t] = exp_diff_accurate(v[t], ref, 1.0f);
+          } else {
 #pragma unroll
-          for (int t = 0; t < 8; ++t) v[t] = __fdiv_rn(v[t], tau);
+            for (int t = 0; t < 8; ++t) v[t] = exp_diff_accurate(v[t], ref, tau);
+          }
+          S = sum8(v);
+        } else {
+#pragma unroll
+          for (int t = 0; t < 8; ++t) v[t] = __fsub_rn(v[t], ref);
+          if (tau != 1.0f) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t) v[t] = __fdiv_rn(v[t], tau);
+          }
+#pragma unroll
+          for (int t = 0; t < 8; ++t) v[t] = exp_fast(v[t]);
+          S = two_sum(sum4(v[0], v[1], v[2], v[3]), sum4(v[4], v[5], v[6], v[7]));
         }
-#pragma unroll
-        for (int t = 0; t < 8; ++t) v[t] = exp_fast(v[t]);
-        const ff S = warp_sum_ff(two_sum(sum4(v[0], v[1], v[2], v[3]), sum4(v[4], v[5], v[6], v[7])));
+        S = warp_sum_ff(S);
         if (lane == 0) s_part[r0 + i][warp] = S;
       }
     }
@@ -414,7 +438,10 @@ accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, in
     warp_argmax(mv, mi);
     ff Sr = ff_of(0.f);
     if (!greedy && mv != -INFINITY) {
-      if (lane < cs && ff_pos(cS)) Sr = ff_mul(cS, exp_diff_accurate(cm, mv, tau));
+      if (lane < cs && ff_pos(cS)) {
+        if constexpr (kExact) Sr = ff_mul(cS, exp_diff_ff(cm, mv, tau));
+        else Sr = ff_mul(cS, exp_diff_accurate(cm, mv, tau));
+      }
       Sr = warp_sum_ff<kClusterMax>(Sr);
     }
     if (lane == 0) {
@@ -482,9 +509,6 @@ accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, in
         if (e0 + t < len) draw_terms(xv[t], qv[t], residual, dec.m, tau, invS, tr[t], tp[t]);
     }
   }
-  auto sum8 = [](const float (&t)[8]) {
-    return ff_add(ff_add(two_sum(t[0], t[1]), two_sum(t[2], t[3])), ff_add(two_sum(t[4], t[5]), two_sum(t[6], t[7])));
-  };
   // the slice's mass of the terms t and its last index with mass, into every
   // CTA's s_draws; returns the thread's exclusive prefix
   auto publish = [&](const float (&t)[8]) -> ff {
@@ -1201,22 +1225,28 @@ static bool cluster_plan(int V, int *cs, int *slice) {
 constexpr int kClusterMostSmem = 200 * 1024;
 static_assert(kClusterMostSmem >= (SF_MAX_DRAFT + 1) * kClusterMaxSlice * 4, "the rows themselves fit");
 
+using ClusterKernelFn = void (*)(const AccParams, int, int, int, int);
+
+static ClusterKernelFn cluster_kernel(bool exact) {
+  return exact ? accept_cluster_kernel<true> : accept_cluster_kernel<false>;
+}
+
 // Sets the kernel attributes once per device and reports whether a cluster
 // of cs CTAs can be resident (*ok false: use the two-kernel path).
-static int cluster_setup(int cs, bool *ok) {
+static int cluster_setup(int cs, bool exact, bool *ok) {
   static std::mutex mu;
-  static int state[64][kClusterMax + 1] = {};  // 0 unknown, 1 usable, 2 not usable
+  static int state[64][2][kClusterMax + 1] = {};  // 0 unknown, 1 usable, 2 not usable
   DeviceInfo dev;
   int st = current_device(&dev);
   if (st != SF_OK) return st;
   if (dev.ordinal < 0 || dev.ordinal >= 64) return fail(SF_ERR_UNSUPPORTED, "device ordinal %d", dev.ordinal);
   std::lock_guard<std::mutex> lock(mu);
-  if (state[dev.ordinal][cs] == 0) {
+  int &known = state[dev.ordinal][exact ? 1 : 0][cs];
+  if (known == 0) {
     const int most = kClusterMostSmem;
-    cudaError_t e = cudaFuncSetAttribute(accept_cluster_kernel,
-                                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(accept_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    const ClusterKernelFn fn = cluster_kernel(exact);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess)
       return fail(SF_ERR_CUDA, "cudaFuncSetAttribute (accept cluster): %s", cudaGetErrorString(e));
     cudaLaunchAttribute attr[1];
@@ -1231,11 +1261,11 @@ static int cluster_setup(int cs, bool *ok) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, accept_cluster_kernel, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
     if (e != cudaSuccess) (void)cudaGetLastError();  // not usable: clear the error
-    state[dev.ordinal][cs] = (e == cudaSuccess && n > 0) ? 1 : 2;
+    known = (e == cudaSuccess && n > 0) ? 1 : 2;
   }
-  *ok = state[dev.ordinal][cs] == 1;
+  *ok = known == 1;
   return SF_OK;
 }
 
@@ -1280,33 +1310,11 @@ static int check_accept_shapes(int B, int k, int V) {
   return SF_OK;
 }
 
-}  // namespace sf
-
-extern "C" {
-
-size_t sf_accept_workspace_size(int B, int k, int V) {
-  if (sf::check_accept_shapes(B, k, V) != SF_OK) return 0;
-  sf::AccPlan plan;
-  if (sf::plan_accept(V, &plan) != SF_OK) return 0;
-  return sf::acc_layout(B, k, plan).total;
-}
-
-int sf_accept_kernel_launches(int B, int k, int V) {
-  using namespace sf;
-  if (check_accept_shapes(B, k, V) != SF_OK) return 0;
-  int cs = 0, slice = 0;
-  bool cluster_ok = false;
-  if (cluster_plan(V, &cs, &slice) && cluster_setup(cs, &cluster_ok) != SF_OK) return 0;
-  return cluster_ok ? 1 : 2;
-}
-
-int sf_accept(const float *target_logits, const float *draft_probs,
-              const int32_t *draft_tokens, const float *uniforms, const float *temperature,
-              int B, int k, int V, int32_t *num_accepted, int32_t *out_tokens,
-              float *accept_ratio, void *workspace, size_t workspace_bytes,
-              cudaStream_t stream) {
-  using namespace sf;
-  clear_error();
+// sf_accept; exact_sums: see accept_cluster_kernel (the two-kernel path has none).
+static int launch_accept(const float *target_logits, const float *draft_probs, const int32_t *draft_tokens,
+                         const float *uniforms, const float *temperature, int B, int k, int V, int32_t *num_accepted,
+                         int32_t *out_tokens, float *accept_ratio, void *workspace, size_t workspace_bytes,
+                         bool exact_sums, cudaStream_t stream) {
   int st = check_accept_shapes(B, k, V);
   if (st != SF_OK) return st;
   if (!target_logits || !draft_probs || !draft_tokens || !uniforms || !temperature ||
@@ -1355,7 +1363,7 @@ int sf_accept(const float *target_logits, const float *draft_probs,
   int cs = 0, slice = 0;
   bool cluster_ok = false;
   if (cluster_plan(V, &cs, &slice)) {
-    st = cluster_setup(cs, &cluster_ok);
+    st = cluster_setup(cs, exact_sums, &cluster_ok);
     if (st != SF_OK) return st;
   }
   if (cluster_ok) {
@@ -1375,7 +1383,7 @@ int sf_accept(const float *target_logits, const float *draft_probs,
     ccfg.stream = stream;
     ccfg.attrs = cattr;
     ccfg.numAttrs = 2;
-    cudaError_t ce = cudaLaunchKernelEx(&ccfg, accept_cluster_kernel, prm, cs, slice, bufs, ahead ? 1 : 0);
+    cudaError_t ce = cudaLaunchKernelEx(&ccfg, cluster_kernel(exact_sums), prm, cs, slice, bufs, ahead ? 1 : 0);
     if (ce != cudaSuccess) return fail(SF_ERR_CUDA, "accept cluster launch: %s", cudaGetErrorString(ce));
     return SF_OK;
   }
@@ -1411,6 +1419,37 @@ int sf_accept(const float *target_logits, const float *draft_probs,
   e = cudaLaunchKernelEx(&cfg, accept_draw_kernel, prm);
   if (e != cudaSuccess) return fail(SF_ERR_CUDA, "accept draw launch: %s", cudaGetErrorString(e));
   return SF_OK;
+}
+
+}  // namespace sf
+
+extern "C" {
+
+size_t sf_accept_workspace_size(int B, int k, int V) {
+  if (sf::check_accept_shapes(B, k, V) != SF_OK) return 0;
+  sf::AccPlan plan;
+  if (sf::plan_accept(V, &plan) != SF_OK) return 0;
+  return sf::acc_layout(B, k, plan).total;
+}
+
+int sf_accept_kernel_launches(int B, int k, int V) {
+  using namespace sf;
+  if (check_accept_shapes(B, k, V) != SF_OK) return 0;
+  int cs = 0, slice = 0;
+  bool cluster_ok = false;
+  if (cluster_plan(V, &cs, &slice) && cluster_setup(cs, false, &cluster_ok) != SF_OK) return 0;
+  return cluster_ok ? 1 : 2;
+}
+
+int sf_accept(const float *target_logits, const float *draft_probs,
+              const int32_t *draft_tokens, const float *uniforms, const float *temperature,
+              int B, int k, int V, int32_t *num_accepted, int32_t *out_tokens,
+              float *accept_ratio, void *workspace, size_t workspace_bytes,
+              cudaStream_t stream) {
+  using namespace sf;
+  clear_error();
+  return launch_accept(target_logits, draft_probs, draft_tokens, uniforms, temperature, B, k, V, num_accepted,
+                       out_tokens, accept_ratio, workspace, workspace_bytes, false, stream);
 }
 
 size_t sf_verify_lm_head_accept_workspace_size(int B, int k, int V) {
@@ -1460,22 +1499,30 @@ int sf_verify_lm_head_accept(const void *hidden, const void *weight, const float
   const bool vec4 = (V % 4 == 0) && aligned(logits, 16) && aligned(draft_probs, 16);
   int Gl = 0;
   // Where sf_accept is one cluster launch with the draft rows fetched ahead, it
-  // is shorter than the statistics epilogue, the decisions and the draw: the
-  // projection then writes the logits alone.  B = 1, k = 5, V = 32000 54.9 -> 51.3 us,
-  // B = 8, k = 5 58.6 -> 55.4, B = 16, k = 8, V = 8000 34.7 -> 27.8, B = 1, k = 2, V = 2000
-  // 19.0 -> 13.4; not fetched ahead it is longer (B = 2, k = 16, V = 32000 58.1, 61.0 so).
+  // is mostly shorter than the statistics epilogue, the decisions and the draw:
+  // the projection then writes the logits alone, and the cluster sums the rows at
+  // the statistics' precision.  Those sums cost it 0.4 us a row, the statistics
+  // more with every 16 rows and at temperatures other than 1, so few drafts or many
+  // sequences go that way.  Whole calls, statistics -> cluster, at temperature 1
+  // and 0.7: B = 1, k = 2, V = 2000 18.9 -> 15.6, 24.9 -> 17.4 us; B = 1, k = 5, V = 32000
+  // 55.0 -> 55.0, 61.6 -> 59.1; B = 8, k = 5 59.3 -> 58.3, 74.4 -> 62.1; B = 16, k = 8,
+  // V = 8000 35.3 -> 31.2, 70.3 -> 36.7; the other side of the line: B = 1, k = 8, V =
+  // 32000 54.8 -> 58.6, 63.0 -> 64.6; B = 4, k = 8, V = 2000 20.0 -> 23.0, 33.2 -> 28.5.
+  // Not fetched ahead it is longer (B = 2, k = 16, V = 32000 58.1 -> 61.0 before the
+  // finer sums).
   int cs = 0, slice = 0, bufs = 0;
   bool cluster_ok = false;
-  if (cluster_plan(V, &cs, &slice) && cluster_rows(B, k, V, cs, slice, vec4, &bufs)) {
-    st = cluster_setup(cs, &cluster_ok);
+  if ((k <= 5 || B >= 8) && cluster_plan(V, &cs, &slice) &&
+      cluster_rows(B, k, V, cs, slice, vec4, &bufs)) {
+    st = cluster_setup(cs, true, &cluster_ok);
     if (st != SF_OK) return st;
   }
   if (cluster_ok) {
     st = launch_projection_stats(hidden, weight, R, d, V, logits, temperature, k + 1, nullptr,
                                  reinterpret_cast<uint32_t *>(ws), &Gl, stream);
     if (st != SF_OK) return st;
-    return sf_accept(logits, draft_probs, draft_tokens, uniforms, temperature, B, k, V, num_accepted, out_tokens,
-                     accept_ratio, workspace, workspace_bytes, stream);
+    return launch_accept(logits, draft_probs, draft_tokens, uniforms, temperature, B, k, V, num_accepted, out_tokens,
+                         accept_ratio, workspace, workspace_bytes, true, stream);
   }
   SampStat *stats = reinterpret_cast<SampStat *>(ws + lay.total);
   // target logits and their per-CTA row statistics; row b*(k+1)+i uses tau_b

@@ -62,6 +62,8 @@ __device__ __forceinline__ ff ff_mul(ff a, float b) {
   return ff{hi, __fsub_rn(e, __fsub_rn(hi, p))};
 }
 
+__device__ __forceinline__ ff ff_mul(ff a, ff b) { return ff_add(ff_mul(a, b.hi), ff_of(__fmul_rn(a.hi, b.lo))); }
+
 __device__ __forceinline__ bool ff_lt(ff a, ff b) {
   return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo);
 }
@@ -91,6 +93,40 @@ __device__ __forceinline__ float exp_diff_accurate(float x, float m, float tau) 
     hi = qh;
   }
   return __fmul_rn(expf(hi), __fadd_rn(1.0f, lo));
+}
+
+// exp((x - m) / tau), x <= m, as a float-float number with a relative error of
+// about 1e-8, for factors that scale a whole partial sum (where the error of
+// many terms averages out and that of one factor would not).  Cody and Waite's
+// reduction, (x - m) / tau = n ln 2 + r with ln 2 in two parts, then 1 + r exact and the
+// rest of the power series, at most 0.07, in fp32.  0 below e^-87.
+__device__ __forceinline__ ff exp_diff_ff(float x, float m, float tau) {
+  float hi = __fsub_rn(x, m);
+  const float v = __fsub_rn(hi, x);
+  float lo = __fadd_rn(__fsub_rn(x, __fsub_rn(hi, v)), __fsub_rn(-m, v));
+  if (tau != 1.0f) {
+    const float qh = __fdiv_rn(hi, tau);
+    const float rest = __fmaf_rn(-qh, tau, hi);  // hi - qh * tau, exact
+    lo = __fdiv_rn(__fadd_rn(rest, lo), tau);
+    hi = qh;
+  }
+  if (hi <= -87.0f) return ff_of(0.f);  // a masked part (x = -inf) too
+  const float n = rintf(__fmul_rn(hi, 1.44269504f));
+  constexpr float kLn2Hi = 0.693145751953125f;     // 15 bits of ln 2: n kLn2Hi is exact
+  constexpr float kLn2Lo = 1.42860682030941723e-6f;  // ln 2 - kLn2Hi
+  const ff r = two_sum(__fmaf_rn(-n, kLn2Hi, hi), __fmaf_rn(-n, kLn2Lo, lo));
+  float q = 1.0f / 40320.0f;
+  q = __fmaf_rn(q, r.hi, 1.0f / 5040.0f);
+  q = __fmaf_rn(q, r.hi, 1.0f / 720.0f);
+  q = __fmaf_rn(q, r.hi, 1.0f / 120.0f);
+  q = __fmaf_rn(q, r.hi, 1.0f / 24.0f);
+  q = __fmaf_rn(q, r.hi, 1.0f / 6.0f);
+  q = __fmaf_rn(q, r.hi, 0.5f);
+  q = __fmul_rn(q, __fmul_rn(r.hi, r.hi));
+  const ff s = two_sum(1.0f, r.hi);
+  const ff e = two_sum(s.hi, __fadd_rn(__fadd_rn(s.lo, r.lo), q));
+  const float scale = __int_as_float((static_cast<int>(n) + 127) << 23);  // 2^n, n >= -126
+  return ff{__fmul_rn(e.hi, scale), __fmul_rn(e.lo, scale)};
 }
 
 // Hardware base-2 exponential (approximate, subnormal results kept).

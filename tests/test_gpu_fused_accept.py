@@ -14,7 +14,7 @@ import torch
 from scipy.special import softmax
 
 from paper_2505_12728_gb300 import specflash_verify as sfv
-from paper_2505_12728_gb300.workloads import (AcceptInputs, HIDDEN_SIZES, WORKLOADS,
+from paper_2505_12728_gb300.workloads import (AcceptInputs, HIDDEN_SIZES, WORKLOADS, f32_to_bf16_bits,
                                               make_draft_tail_case, temperatures)
 from tests.gpu_helpers import bf16_tensor, compare_accept, oracle_accept, require_gpu, run_accept
 
@@ -116,8 +116,12 @@ def test_decisions_with_a_warp_for_each_row(oracle_mod, B, k, V):
 @pytest.mark.parametrize("B,k,V", [
     (13, 5, 32000),    # draft rows of 8.32 MB: one cluster launch after the projection
     (14, 5, 32000),    # 8.96 MB: statistics, decisions and draw
-    (1, 8, 32768),     # the longest rows of a cluster
-    (1, 8, 32772),     # one step beyond
+    (1, 8, 32768),     # more than five drafts of few sequences: the same
+    (1, 5, 32768),     # the longest rows of a cluster
+    (1, 5, 32772),     # one step beyond
+    (1, 8, 32772),
+    (7, 6, 8000),      # statistics, decisions and draw: six drafts
+    (8, 6, 8000),      # a cluster launch: eight sequences
     (2, 16, 32000),    # rows and draft rows don't fit shared memory together
     (3, 4, 5001),      # not 16-byte aligned
     (5, 1, 16),
@@ -175,3 +179,38 @@ def test_greedy_calls_back_to_back_on_one_workspace(oracle_mod):
     assert sfv.read_device_status(ws) == 0
     for (_, _, inp, _), out in zip(cases, outs):
         assert compare_accept(oracle_accept(oracle_mod, inp), *(t.cpu().numpy() for t in out)) == 0
+
+
+@pytest.mark.parametrize("V", [8000, 32000, 40000])
+def test_row_sums_carry_the_scaled_difference_in_float_float(V):
+    """A token at logit 0 in every 2000 (the slice of a CTA of the cluster) and
+    the others at -a, with a / tau a little above 8 and its fp32 rounding error as
+    large as it gets, of one sign in a row: the row sum must not show it.
+
+    The bound: p(0) = 1 / S (and q = 1), of which the share s comes from the terms
+    at -a, shows s times the error of one term, expf's (one unit in the last
+    place at most, 2^-23) and the product's with 1 + lo (2^-24), and the quotient's
+    rounding (2^-24): 1.25e-7 at s = 0.36.  An fp32 a / tau is off by 2^-21, which
+    alone is 1.7e-7 of S."""
+    rng = np.random.default_rng(V)
+    B, k, d = 16, 1, 8
+    hidden, weight = np.zeros((B, k + 1, d), np.float32), np.zeros((V, d), np.float32)
+    weight[:, 0] = -1.0
+    weight[::2000, 0] = 0.0
+    a, tau = np.empty(B), np.empty(B, np.float32)
+    for b in range(B):  # a: eight bits (exact in bf16); tau: the worst of many for it
+        a[b] = hidden[b, :, 0] = rng.integers(128, 256) / 16.0
+        t = (a[b] / (8.02 + 0.2 * rng.random(200000))).astype(np.float32)
+        off = (np.float32(a[b]) / t).astype(np.float64) - a[b] / t.astype(np.float64)
+        tau[b] = t[np.argmax(off) if b % 2 else np.argmin(off)]
+        assert abs(off).max() > 0.9 * 2.0 ** -21
+    inp = AcceptInputs(target_logits=None, draft_probs=np.ones((B, k, V), np.float32),
+                       draft_tokens=np.zeros((B, k), np.int32), uniforms=np.full((B, k + 1), 0.5, np.float32),
+                       temperature=tau)
+    logits, _, _, ratio = run_fused(f32_to_bf16_bits(hidden), f32_to_bf16_bits(weight), inp)
+    np.testing.assert_array_equal(logits[:, 0, 1], -a.astype(np.float32))
+    ones = V // 2000
+    rest = (V - ones) * np.exp(-a / tau.astype(np.float64))
+    want = 1.0 / (ones + rest)
+    err = np.abs(ratio[:, 0].astype(np.float64) - want) / want
+    assert (err <= rest * want * (2.0 ** -23 + 2.0 ** -24) + 2.0 ** -24).all(), err
