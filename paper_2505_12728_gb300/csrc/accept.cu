@@ -38,7 +38,9 @@
 // float-float gives the accuracy the decisions need.
 #include <climits>
 #include <cmath>
+#include <map>
 #include <mutex>
+#include <tuple>
 
 #include "chunk_split.h"
 #include "ff_math.cuh"
@@ -1231,42 +1233,58 @@ static ClusterKernelFn cluster_kernel(bool exact) {
   return exact ? accept_cluster_kernel<true> : accept_cluster_kernel<false>;
 }
 
-// Sets the kernel attributes once per device and reports whether a cluster
-// of cs CTAs can be resident (*ok false: use the two-kernel path).
-static int cluster_setup(int cs, bool exact, bool *ok) {
+// How many clusters of cs CTAs with `smem` bytes of dynamic shared memory each
+// are resident at once on the current device (*resident; 0: none can be).  Asked
+// of the runtime once per device, size and KB; the kernel's attributes are set
+// before the first answer.
+static int cluster_resident(int cs, size_t smem, bool exact, int *resident) {
   static std::mutex mu;
-  static int state[64][2][kClusterMax + 1] = {};  // 0 unknown, 1 usable, 2 not usable
+  static std::map<std::tuple<int, bool, int, int>, int> known;  // at most 16 x 201 per device and variant
   DeviceInfo dev;
   int st = current_device(&dev);
   if (st != SF_OK) return st;
-  if (dev.ordinal < 0 || dev.ordinal >= 64) return fail(SF_ERR_UNSUPPORTED, "device ordinal %d", dev.ordinal);
+  const int kb = static_cast<int>((smem + 1023) / 1024);
   std::lock_guard<std::mutex> lock(mu);
-  int &known = state[dev.ordinal][exact ? 1 : 0][cs];
-  if (known == 0) {
-    const int most = kClusterMostSmem;
-    const ClusterKernelFn fn = cluster_kernel(exact);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    if (e != cudaSuccess)
-      return fail(SF_ERR_CUDA, "cudaFuncSetAttribute (accept cluster): %s", cudaGetErrorString(e));
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cs, 1);
-    cfg.blockDim = dim3(kAccThreads);
-    cfg.dynamicSmemBytes = most;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
-    if (e != cudaSuccess) (void)cudaGetLastError();  // not usable: clear the error
-    known = (e == cudaSuccess && n > 0) ? 1 : 2;
+  const auto key = std::make_tuple(dev.ordinal, exact, cs, kb);
+  const auto it = known.find(key);
+  if (it != known.end()) {
+    *resident = it->second;
+    return SF_OK;
   }
-  *ok = known == 1;
+  const ClusterKernelFn fn = cluster_kernel(exact);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kClusterMostSmem);
+  if (e != cudaSuccess)
+    return fail(SF_ERR_CUDA, "cudaFuncSetAttribute (accept cluster): %s", cudaGetErrorString(e));
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cs;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cs, 1);
+  cfg.blockDim = dim3(kAccThreads);
+  cfg.dynamicSmemBytes = static_cast<size_t>(kb) * 1024;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
+  if (e != cudaSuccess) {  // not usable: clear the error
+    (void)cudaGetLastError();
+    n = 0;
+  }
+  known[key] = n;
+  *resident = n;
   return SF_OK;
+}
+
+// Whether a cluster of cs CTAs can be resident with the most shared memory that a
+// launch asks for (*ok false: use the two-kernel path).
+static int cluster_setup(int cs, bool exact, bool *ok) {
+  int n = 0;
+  const int st = cluster_resident(cs, kClusterMostSmem, exact, &n);
+  *ok = st == SF_OK && n > 0;
+  return st;
 }
 
 // Raises the bulk-copy chunk kernel's dynamic shared memory limit once per
@@ -1287,19 +1305,24 @@ static int chunks_setup(int device) {
 }
 
 // How the rows of a launch of clusters of cs CTAs lie in shared memory: *bufs of
-// them at a time, and whether the draft rows follow (fetched ahead of the
+// them at a time, and whether the draft rows follow (*ahead: fetched ahead of the
 // decisions).
-static bool cluster_rows(int B, int k, int V, int cs, int slice, bool vec4, int *bufs) {
-  // Every row in shared memory while the batch's clusters are all resident
-  // so (about 7 clusters of 16 per CTA that an SM holds), else kClusterFewBufs
-  // rows at a time: more clusters per SM are worth a second round of copies
-  // (B = 16, k = 8, V = 32000: 33 us with all nine rows, 26 with five).
-  const size_t sm_bytes = 228 * 1024, fixed = 9 * 1024;  // static and reserved shared memory
-  const int groups = cs > 8 ? 7 : 15 * 8 / cs;
-  const long long resident = groups * static_cast<long long>(sm_bytes / (cluster_smem(k, slice, k + 1, false) + fixed));
-  *bufs = B <= resident || k + 1 < kClusterFewBufs ? k + 1 : kClusterFewBufs;
-  return vec4 && *bufs == k + 1 && 4LL * B * k * V <= kAheadBytes &&
-         cluster_smem(k, slice, *bufs, true) <= static_cast<size_t>(kClusterMostSmem);
+// Every row, and then the draft rows, as long as the batch's clusters are all
+// resident so; else kClusterFewBufs rows at a time: more clusters per SM are worth
+// a second round of copies (B = 16, k = 8, V = 32000: 33 us with all nine rows, 26
+// with five; draft rows ahead in two waves of clusters: B = 8, k = 8, V = 32000
+// 27.2 us, without them 18.3).
+static int cluster_rows(int B, int k, int V, int cs, int slice, bool vec4, bool exact, int *bufs, bool *ahead) {
+  int n = 0;
+  int st = cluster_resident(cs, cluster_smem(k, slice, k + 1, false), exact, &n);
+  if (st != SF_OK) return st;
+  *bufs = B <= n || k + 1 < kClusterFewBufs ? k + 1 : kClusterFewBufs;
+  const size_t both = cluster_smem(k, slice, k + 1, true);
+  *ahead = vec4 && *bufs == k + 1 && 4LL * B * k * V <= kAheadBytes && both <= static_cast<size_t>(kClusterMostSmem);
+  if (!*ahead) return SF_OK;
+  st = cluster_resident(cs, both, exact, &n);
+  *ahead = B <= n;
+  return st;
 }
 
 static int check_accept_shapes(int B, int k, int V) {
@@ -1378,7 +1401,9 @@ static int launch_accept(const float *target_logits, const float *draft_probs, c
     ccfg.gridDim = dim3(cs, B);
     ccfg.blockDim = dim3(kAccThreads);
     int bufs = 0;
-    const bool ahead = cluster_rows(B, k, V, cs, slice, prm.vec4 != 0, &bufs);
+    bool ahead = false;
+    st = cluster_rows(B, k, V, cs, slice, prm.vec4 != 0, exact_sums, &bufs, &ahead);
+    if (st != SF_OK) return st;
     ccfg.dynamicSmemBytes = cluster_smem(k, slice, bufs, ahead);
     ccfg.stream = stream;
     ccfg.attrs = cattr;
@@ -1511,13 +1536,13 @@ int sf_verify_lm_head_accept(const void *hidden, const void *weight, const float
   // Not fetched ahead it is longer (B = 2, k = 16, V = 32000 58.1 -> 61.0 before the
   // finer sums).
   int cs = 0, slice = 0, bufs = 0;
-  bool cluster_ok = false;
-  if ((k <= 5 || B >= 8) && cluster_plan(V, &cs, &slice) &&
-      cluster_rows(B, k, V, cs, slice, vec4, &bufs)) {
+  bool cluster_ok = false, ahead = false;
+  if ((k <= 5 || B >= 8) && cluster_plan(V, &cs, &slice)) {
     st = cluster_setup(cs, true, &cluster_ok);
+    if (st == SF_OK && cluster_ok) st = cluster_rows(B, k, V, cs, slice, vec4, true, &bufs, &ahead);
     if (st != SF_OK) return st;
   }
-  if (cluster_ok) {
+  if (cluster_ok && ahead) {
     st = launch_projection_stats(hidden, weight, R, d, V, logits, temperature, k + 1, nullptr,
                                  reinterpret_cast<uint32_t *>(ws), &Gl, stream);
     if (st != SF_OK) return st;

@@ -77,6 +77,8 @@ def test_vocabulary_beyond_the_single_kernel_path(oracle_mod, mode):
     (2, 3, 2049, "sampling", 0.7),     # a second CTA of one token, scalar copies
     (1, 16, 32768, "sampling", 1.0),   # the longest rows, the most of them, no draft rows ahead
     (3, 16, 30724, "alternate", 1.3),  # the last slice is the shortest
+    (7, 8, 32000, "alternate", 1.0),   # the most clusters that are resident with draft rows ahead
+    (8, 8, 32000, "alternate", 1.0),   # one more: none ahead
     (40, 8, 32000, "sampling", 1.0),   # rows five at a time: two rounds of copies
     (40, 15, 4100, "sampling", 0.8),   # the same with three rounds, three CTAs
     (40, 9, 9001, "alternate", 1.0),   # the same with scalar copies

@@ -122,6 +122,7 @@ def test_decisions_with_a_warp_for_each_row(oracle_mod, B, k, V):
     (1, 8, 32772),
     (7, 6, 8000),      # statistics, decisions and draw: six drafts
     (8, 6, 8000),      # a cluster launch: eight sequences
+    (8, 8, 32000),     # statistics: eight clusters aren't resident with draft rows ahead
     (2, 16, 32000),    # rows and draft rows don't fit shared memory together
     (3, 4, 5001),      # not 16-byte aligned
     (5, 1, 16),
