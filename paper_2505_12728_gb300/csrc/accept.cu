@@ -476,7 +476,7 @@ accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, in
     const float *row = s_rows + static_cast<size_t>(here ? j - r0 : 0) * slice;
     // four tokens of a row of the slice in global memory
     auto fetch4 = [&](const float *g, int e, float pad) -> float4 {
-      if (bulk) return __ldg(reinterpret_cast<const float4 *>(g + e));
+      if (bulk) return *reinterpret_cast<const float4 *>(g + e);
       return make_float4(g[e], e + 1 < len ? g[e + 1] : pad, e + 2 < len ? g[e + 2] : pad,
                          e + 3 < len ? g[e + 3] : pad);
     };
@@ -632,7 +632,7 @@ __device__ __forceinline__ RowStat combine_records(const float4 *rr, int n, floa
 // and two passes over the records, B = 7, k = 16, V = 32000 took 54.2 us with its
 // projection and draw, against 49.8; B = 4, k = 8, V = 152064 194.3 against 192.1.
 __global__ void __launch_bounds__(32 * (SF_MAX_DRAFT + 1))
-accept_decide_kernel(const __grid_constant__ AccParams p, const SampStat *__restrict__ stats, int G) {
+accept_decide_kernel(const __grid_constant__ AccParams p, const SampStat *stats, int G) {
   __shared__ float s_rm[SF_MAX_DRAFT + 1];
   __shared__ int s_rarg[SF_MAX_DRAFT + 1];
   __shared__ ff s_rS[SF_MAX_DRAFT + 1];
@@ -930,7 +930,7 @@ __device__ __forceinline__ void run_begin(const AccParams &p, RunState &st, int 
   st.len = 0;
   st.g0 = chunk_owner(row * p.C1, U, p.NW1);
   st.n_runs = chunk_owner(row * p.C1 + p.C1 - 1, U, p.NW1) - st.g0 + 1;
-  st.tau = __ldg(p.tau + row / (p.k + 1));
+  st.tau = p.tau[row / (p.k + 1)];
   st.greedy = !(st.tau > 0.0f);
   st.scale = st.greedy ? 0.f : __fdiv_rn(1.44269504088896341f, st.tau);
   st.lm = -INFINITY;

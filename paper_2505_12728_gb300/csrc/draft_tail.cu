@@ -525,14 +525,14 @@ __global__ void __launch_bounds__(kFfThreads) sample_stats_kernel(const __grid_c
   for (int h = 0; h < kPer / 4; ++h) {
     const int i0 = e0 + h * 4 * kFfThreads + 4 * tid;
     if (p.vec4 && i0 + 3 < p.V) {
-      const float4 f = __ldg(reinterpret_cast<const float4 *>(row + i0));
+      const float4 f = *reinterpret_cast<const float4 *>(row + i0);
       x[4 * h] = f.x;
       x[4 * h + 1] = f.y;
       x[4 * h + 2] = f.z;
       x[4 * h + 3] = f.w;
     } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) x[4 * h + j] = i0 + j < p.V ? __ldg(row + i0 + j) : -INFINITY;
+      for (int j = 0; j < 4; ++j) x[4 * h + j] = i0 + j < p.V ? row[i0 + j] : -INFINITY;
     }
   }
   float bv = -INFINITY;

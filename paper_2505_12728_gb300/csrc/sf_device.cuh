@@ -186,6 +186,9 @@ __device__ __forceinline__ void grid_launch_dependents() {
 
 // ... and wait until the previous kernel on the stream has completed and its
 // memory operations are visible (a no-op when launched without the attribute).
+// What that kernel may write is read after the wait by ordinary loads: the
+// non-coherent path (ld.global.nc, __ldg) is for memory that nothing writes while
+// the kernel runs, and this kernel runs already while it waits.
 __device__ __forceinline__ void grid_dependency_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

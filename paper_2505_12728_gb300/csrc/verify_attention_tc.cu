@@ -706,7 +706,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
       const uint4 *src = reinterpret_cast<const uint4 *>(q_row(pc));
 #pragma unroll
       for (int u = 0; u < D / 8; ++u) {
-        const uint4 v = valid ? __ldg(src + u) : make_uint4(0u, 0u, 0u, 0u);
+        const uint4 v = valid ? src[u] : make_uint4(0u, 0u, 0u, 0u);
         qw[4 * u] = v.x; qw[4 * u + 1] = v.y; qw[4 * u + 2] = v.z; qw[4 * u + 3] = v.w;
       }
     };

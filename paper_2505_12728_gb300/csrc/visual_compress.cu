@@ -108,7 +108,7 @@ compress_softmax_kernel(const __grid_constant__ VcSoftmaxParams p) {
   auto token = [&](int i) { return kT > 32 ? t + kT * i : 64 * (i / 2) + 2 * t + i % 2; };
   float x[2 * kPairs];
 #pragma unroll
-  for (int i = 0; i < kOwn; ++i) x[i] = token(i) < p.N ? __ldg(row + token(i)) : -INFINITY;
+  for (int i = 0; i < kOwn; ++i) x[i] = token(i) < p.N ? row[token(i)] : -INFINITY;
 #pragma unroll 1
   for (int s0 = 1; s0 < p.ks; s0 += kFly) {
     float v[kFly][kOwn];
@@ -117,7 +117,7 @@ compress_softmax_kernel(const __grid_constant__ VcSoftmaxParams p) {
       const float *part = row + (s0 + u) * p.part_stride;
 #pragma unroll
       for (int i = 0; i < kOwn; ++i)
-        v[u][i] = s0 + u < p.ks && token(i) < p.N ? __ldg(part + token(i)) : 0.f;
+        v[u][i] = s0 + u < p.ks && token(i) < p.N ? part[token(i)] : 0.f;
     }
 #pragma unroll
     for (int u = 0; u < kFly; ++u) {
