@@ -200,8 +200,10 @@ def test_sample_on_both_sides_of_the_streaming_size(oracle_mod, V):
     (1, 65537),    # 33: a thread for each, scalar accesses
     (4, 70000),    # the same with several rows
     (2, 155648),   # 304 CTAs: two per SM
-    (2, 155652),   # 306: one warp again
-    (1, 311296),   # the most chunks that the block combines (152)
+    (2, 155652),   # spans of 2048 tokens: 154
+    (1, 311296),   # 152 chunks
+    (4, 311296),   # spans of 4096 tokens, the longest at two CTAs per SM
+    (4, 311300),   # five per SM: one warp again
 ])
 def test_sample_combination_by_a_warp_or_the_block(oracle_mod, R, V):
     rng = np.random.default_rng(V + R)
