@@ -212,6 +212,10 @@ __device__ __forceinline__ void lm_epilogue_step(uint32_t taddr, float *logits, 
     if (tau == 1.f) {  // one branch for all: the divisions are skipped together
 #pragma unroll
       for (int e = 0; e < 16; ++e) xv[e] = term_of(xv[e], ref, 1.f);
+    } else if (tau >= kRecipTauMin && tau <= kRecipTauMax) {
+      const float inv = __fdiv_rn(1.f, tau);
+#pragma unroll
+      for (int e = 0; e < 16; ++e) xv[e] = exp_diff_recip(xv[e], ref, tau, inv);
     } else {
 #pragma unroll
       for (int e = 0; e < 16; ++e) xv[e] = term_of(xv[e], ref, tau);

@@ -95,6 +95,22 @@ __device__ __forceinline__ float exp_diff_accurate(float x, float m, float tau) 
   return __fmul_rn(expf(hi), __fadd_rn(1.0f, lo));
 }
 
+// The same with 1 / tau at hand (rounded; tau from 2^-64 to 2^64), for loops over
+// many tokens of one temperature: the quotient's high part is a product, off by up
+// to 1.5 units in its last place, and its low part, from the exact remainder, makes
+// up for that, so that hi + lo is as close to the quotient as after a division.
+constexpr float kRecipTauMin = 5.421010862427522e-20f, kRecipTauMax = 1.8446744073709552e19f;
+
+__device__ __forceinline__ float exp_diff_recip(float x, float m, float tau, float inv_tau) {
+  if (x == -INFINITY) return 0.f;
+  const float d = __fsub_rn(x, m);
+  const float v = __fsub_rn(d, x);
+  const float lo = __fadd_rn(__fsub_rn(x, __fsub_rn(d, v)), __fsub_rn(-m, v));
+  const float hi = __fmul_rn(d, inv_tau);
+  const float rest = __fmaf_rn(-hi, tau, d);  // d - hi * tau, exact
+  return __fmul_rn(expf(hi), __fmaf_rn(__fadd_rn(rest, lo), inv_tau, 1.0f));
+}
+
 // exp((x - m) / tau), x <= m, as a float-float number with a relative error of
 // about 1e-8, for factors that scale a whole partial sum (where the error of
 // many terms averages out and that of one factor would not).  Cody and Waite's

@@ -225,6 +225,16 @@ def test_uniform_of_one_draws_the_last_token_with_mass():
         assert (tokens == V - 3001).all()
 
 
+@pytest.mark.parametrize("V", [700, 5000])
+def test_temperatures_at_the_ends_of_the_reciprocal(oracle_mod, V):
+    # the statistics multiply by 1 / tau for tau from 2^-64 to 2^64 and divide
+    # outside; between the last token's zero weight and equal weights
+    tau = np.array([2.0 ** -65, 2.0 ** -64, 2.0 ** -20, 0.37, 1.9, 2.0 ** 20, 2.0 ** 64, 2.0 ** 65], np.float32)
+    case = make_draft_tail_case(len(tau), 64, V, seed=V, temperature=tau, exact=True)
+    logits, probs, tokens = run_fused(case)
+    check_sampler(oracle_mod, logits, case.uniforms, tau, probs, tokens)
+
+
 def test_sample_masked_tokens_and_ties(oracle_mod):
     R, V = 6, 7000
     logits, u, temp = make_sample_case(R, V, seed=5)
