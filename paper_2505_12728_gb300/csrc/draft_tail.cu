@@ -456,32 +456,26 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     }
     if (stats) {
       named_bar_sync(1, kLmEpiThreads);
-      // the eight warps' statistics of a draft row, all rescaled at once
-      for (int c = tid; c < p.R; c += kLmEpiThreads) {
-        SampStat st{-INFINITY, INT_MAX, ff_of(0.f)};
+      // the eight warps' statistics of a draft row, a lane for each: rescaled at
+      // once, by float-float factors (a warp's 32 rows are few of a chunk, and the
+      // errors of as many plain factors showed in the probabilities), and summed
+      // as a tree
+      for (int i0 = 32 * warp; i0 < kLmEpiWarps * p.R; i0 += kLmEpiThreads) {
+        const int c = min((i0 + lane) / kLmEpiWarps, p.R - 1), w = lane % kLmEpiWarps;
+        const SampStat o = run[w * p.NP + c];
+        SampStat st = o;
 #pragma unroll
-        for (int w = 0; w < kLmEpiWarps; ++w) {
-          const SampStat o = run[w * p.NP + c];
-          if (better(o.m, o.arg, st.m, st.arg)) {
-            st.m = o.m;
-            st.arg = o.arg;
+        for (int n = kLmEpiWarps / 2; n >= 1; n >>= 1) {
+          const float om = __shfl_xor_sync(0xffffffffu, st.m, n);
+          const int oa = __shfl_xor_sync(0xffffffffu, st.arg, n);
+          if (better(om, oa, st.m, st.arg)) {
+            st.m = om;
+            st.arg = oa;
           }
         }
-        if (s_tau[c] > 0.f) {
-          ff t[kLmEpiWarps];
-#pragma unroll
-          for (int w = 0; w < kLmEpiWarps; ++w) {
-            const SampStat o = run[w * p.NP + c];
-            t[w] = o.m == -INFINITY || o.m == st.m ? o.S : ff_mul(o.S, exp_diff_accurate(o.m, st.m, s_tau[c]));
-          }
-#pragma unroll
-          for (int n = kLmEpiWarps / 2; n >= 1; n >>= 1) {
-#pragma unroll
-            for (int w = 0; w < n; ++w) t[w] = ff_add(t[w], t[w + n]);
-          }
-          st.S = t[0];
-        }
-        p.stats[static_cast<size_t>(c) * p.G + grp] = st;
+        if (s_tau[c] > 0.f && o.m != -INFINITY && o.m != st.m) st.S = ff_mul(o.S, exp_diff_ff(o.m, st.m, s_tau[c]));
+        st.S = warp_sum_ff<kLmEpiWarps>(st.S);
+        if (w == 0 && i0 + lane < kLmEpiWarps * p.R) p.stats[static_cast<size_t>(c) * p.G + grp] = st;
       }
     }
   }
@@ -633,7 +627,7 @@ sample_finish_kernel(const __grid_constant__ SampleParams p) {
     warp_argmax(m, arg);
     if (!greedy) {
       // chunk masses relative to m, and their prefix over the threads
-      const ff mass = rec.x == -INFINITY ? ff_of(0.f) : ff_mul(ff{rec.z, rec.w}, term_of(rec.x, m, tau));
+      const ff mass = rec.x == -INFINITY ? ff_of(0.f) : ff_mul(ff{rec.z, rec.w}, exp_diff_ff(rec.x, m, tau));
       ff total, next;
       const ff ex = block_scan2(mass, s_scan, &total, &next);
       invS = ff_div_to_f(1.f, total);
@@ -681,7 +675,7 @@ sample_finish_kernel(const __grid_constant__ SampleParams p) {
         // lane is, bit for bit, incl of the lane before
         ff incl = ff_of(0.f);
         for (int c = c_lo; c < c_hi; ++c) {
-          const ff w = s_st[c].m == -INFINITY ? ff_of(0.f) : ff_mul(s_st[c].S, term_of(s_st[c].m, m, tau));
+          const ff w = s_st[c].m == -INFINITY ? ff_of(0.f) : ff_mul(s_st[c].S, exp_diff_ff(s_st[c].m, m, tau));
           s_st[c].S = w;
           incl = ff_add(incl, w);
         }

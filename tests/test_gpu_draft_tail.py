@@ -22,7 +22,7 @@ import pytest
 import torch
 
 from paper_2505_12728_gb300 import specflash_verify as sfv
-from paper_2505_12728_gb300.workloads import (WORKLOADS, bf16_bits_to_f32,
+from paper_2505_12728_gb300.workloads import (WORKLOADS, bf16_bits_to_f32, f32_to_bf16_bits,
                                               make_draft_tail_case, make_draft_tail_inputs,
                                               make_sample_case)
 from tests.gpu_helpers import MARGIN, bf16_tensor, require_gpu
@@ -223,6 +223,27 @@ def test_uniform_of_one_draws_the_last_token_with_mass():
         logits[:, V - 3000:] = -np.inf
         _, tokens = run_sample(logits, np.ones(2, np.float32), np.ones(2, np.float32))
         assert (tokens == V - 3001).all()
+
+
+@pytest.mark.parametrize("V", [1000, 20000])
+def test_probabilities_show_little_but_their_own_rounding(V):
+    """Flat distributions (hundreds of tokens carry the row sum): the largest
+    probability is 1 / S rounded to fp32, 2^-24 at most.  S averages the errors of
+    its terms (2^-23 at most each, a tenth of that or less over a hundred of them:
+    2^-26), and the factors that bring the warps' and the chunks' partial sums
+    together, of which a row has few, must add nothing to that."""
+    R = 256
+    rng = np.random.default_rng(V)
+    tau = (2.7 * (1.0 + 0.1 * rng.random(R))).astype(np.float32)
+    hidden, weight = rng.integers(-8, 9, (R, 64)), rng.integers(-8, 9, (V, 64))
+    logits = hidden @ weight.T / 128.0
+    h, w = (bf16_tensor(f32_to_bf16_bits(x.astype(np.float32))) for x in (hidden, weight / 128.0))
+    got, probs, _ = sfv.draft_sample(h, w, torch.rand(R, device="cuda"), torch.from_numpy(tau).cuda())
+    np.testing.assert_array_equal(got.cpu().numpy(), logits)
+    z = logits / tau.astype(np.float64)[:, None]
+    want = 1.0 / np.exp(z - z.max(axis=1, keepdims=True)).sum(axis=1)
+    top = probs.cpu().numpy().max(axis=1).astype(np.float64)
+    assert np.abs(top / want - 1.0).max() <= 2.0 ** -24 + 2.0 ** -26
 
 
 @pytest.mark.parametrize("V", [700, 5000])
