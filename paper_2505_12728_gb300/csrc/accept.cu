@@ -199,8 +199,9 @@ __device__ __forceinline__ DraftEntry load_draft(const AccParams &p, int b) {
 //     time (one bulk copy per row; with q_ahead also the draft rows' slices, of
 //     which the draw needs one that is not known yet), and the draft tokens'
 //     logits and probabilities are on their way meanwhile;
-//  2. per row the slice's maximum and first index, then the float-float sum of
-//     exp((x - max)/tau), pushed into every CTA of the cluster;
+//  2. per row and warp the maximum, its first index and the float-float sum of
+//     exp((x - max)/tau), combined over the slice and pushed into every CTA of
+//     the cluster;
 //  3. after the first cluster barrier every CTA combines the cs records of
 //     each row in rank order and takes the decisions, identically; CTA 0
 //     writes them.  Greedy clusters leave here;
@@ -238,6 +239,13 @@ static_assert(sizeof(ClusterRec) == 16 && sizeof(ClusterDraw) == 16, "record siz
 // Dynamic shared memory: `bufs` rows' slices, then the k draft rows'.
 static size_t cluster_smem(int k, int slice, int bufs, bool ahead) {
   return sizeof(float) * static_cast<size_t>(slice) * (bufs + (ahead ? k : 0));
+}
+
+// A partial sum relative to the maximum m, relative to the larger maximum to.
+template <bool kExact>
+__device__ __forceinline__ ff scale_sum(ff S, float m, float to, float tau) {
+  if constexpr (kExact) return ff_mul(S, exp_diff_ff(m, to, tau));
+  else return ff_mul(S, exp_diff_accurate(m, to, tau));
 }
 
 // kExact (behind the fused LM head): the row sums have the precision of the
@@ -362,22 +370,9 @@ accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, in
         if (better(v[t], e, bv, bi)) { bv = v[t]; bi = e; }
       }
       warp_argmax(bv, bi);
-      if (lane == 0) {
-        s_wm[r0 + i][warp] = bv;
-        s_wi[r0 + i][warp] = bi;
-      }
-    }
-    __syncthreads();
-    if (!greedy) {
-#pragma unroll 1
-      for (int i = 0; i < n; ++i) {
-        float m = s_wm[r0 + i][0];
-#pragma unroll
-        for (int w = 1; w < kAccWarps; ++w) m = fmaxf(m, s_wm[r0 + i][w]);
-        const float ref = m == -INFINITY ? 0.f : m;  // all masked: every term is 0
-        float v[8];
-        load8(i, v);
-        ff S;
+      ff S = ff_of(0.f);
+      if (!greedy) {
+        const float ref = bv == -INFINITY ? 0.f : bv;  // all masked: every term is 0
         if constexpr (kExact) {
           if (tau == 1.0f) {  // one branch for all: the divisions are skipped together
 #pragma unroll
@@ -399,7 +394,11 @@ accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, in
           S = two_sum(sum4(v[0], v[1], v[2], v[3]), sum4(v[4], v[5], v[6], v[7]));
         }
         S = warp_sum_ff(S);
-        if (lane == 0) s_part[r0 + i][warp] = S;
+      }
+      if (lane == 0) {
+        s_wm[r0 + i][warp] = bv;
+        s_wi[r0 + i][warp] = bi;
+        s_part[r0 + i][warp] = S;
       }
     }
     if (r0 + bufs > k) break;
@@ -412,10 +411,12 @@ accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, in
   cluster_wait();  // every peer has started
   for (int r = warp; r <= k; r += kAccWarps) {
     // the eight warps' records of row r, in warp order
-    float mv = lane < kAccWarps ? s_wm[r][lane] : -INFINITY;
+    const float wm = lane < kAccWarps ? s_wm[r][lane] : -INFINITY;
+    float mv = wm;
     int mi = lane < kAccWarps ? s_wi[r][lane] : INT_MAX;
     warp_argmax(mv, mi);
-    ff S = lane < kAccWarps && !greedy ? s_part[r][lane] : ff_of(0.f);
+    ff S = lane < kAccWarps ? s_part[r][lane] : ff_of(0.f);
+    if (ff_pos(S)) S = scale_sum<kExact>(S, wm, mv, tau);
     S = shfl_ff(warp_sum_ff<kAccWarps>(S), 0);
     if (lane < cs) {
       const uint32_t at = dsmem_addr(smem_addr(&s_all[rank][r]), static_cast<uint32_t>(lane));
@@ -440,10 +441,7 @@ accept_cluster_kernel(const __grid_constant__ AccParams p, int cs, int slice, in
     warp_argmax(mv, mi);
     ff Sr = ff_of(0.f);
     if (!greedy && mv != -INFINITY) {
-      if (lane < cs && ff_pos(cS)) {
-        if constexpr (kExact) Sr = ff_mul(cS, exp_diff_ff(cm, mv, tau));
-        else Sr = ff_mul(cS, exp_diff_accurate(cm, mv, tau));
-      }
+      if (lane < cs && ff_pos(cS)) Sr = scale_sum<kExact>(cS, cm, mv, tau);
       Sr = warp_sum_ff<kClusterMax>(Sr);
     }
     if (lane == 0) {

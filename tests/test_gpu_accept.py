@@ -463,3 +463,37 @@ def test_greedy_calls_back_to_back_on_one_workspace(oracle_mod, V, graph):
         n, toks, ratio = (t.cpu().numpy() for t in o.values())
         assert compare_accept(oracle_accept(oracle_mod, c), n, toks, ratio) == 0
     assert sfv.read_device_status(ws) == 0
+
+
+@pytest.mark.parametrize("V", [8000, 32000])
+def test_row_sums_are_taken_relative_to_near_maxima(V):
+    """A token at logit 0 in every 2000 (a CTA's slice), so in one of the slice's
+    eight warps, and the others at -a, with a / tau a little above 8 and its fp32
+    rounding error as large as it gets, of one sign in a row.  A warp without a
+    token at 0 sums terms exp(0) and scales them once by expf of a float-float
+    argument; only the other warp's terms show the fp32 quotient.
+
+    The bound: p(0) = 1 / S (and q = 1), of which the share s comes from the tokens
+    at -a, shows s (7/8 (2^-23 + 2^-24) + 1/8 (2^-21 + 2.4e-7, the error of the
+    fast 2^x)), and the quotient's rounding, 2^-24."""
+    rng = np.random.default_rng(V)
+    B, k = 16, 1
+    logits = np.empty((B, k + 1, V), np.float32)
+    a, tau = np.empty(B), np.empty(B, np.float32)
+    for b in range(B):
+        a[b] = rng.integers(128, 256) / 16.0
+        t = (a[b] / (8.02 + 0.2 * rng.random(200000))).astype(np.float32)
+        off = (np.float32(a[b]) / t).astype(np.float64) - a[b] / t.astype(np.float64)
+        tau[b] = t[np.argmax(off) if b % 2 else np.argmin(off)]
+        logits[b] = -a[b]
+    logits[:, :, ::2000] = 0.0
+    inp = AcceptInputs(target_logits=logits, draft_probs=np.ones((B, k, V), np.float32),
+                       draft_tokens=np.zeros((B, k), np.int32), uniforms=np.full((B, k + 1), 0.5, np.float32),
+                       temperature=tau)
+    ratio = run_accept(inp)[2]
+    ones = V // 2000
+    rest = (V - ones) * np.exp(-a / tau.astype(np.float64))
+    want = 1.0 / (ones + rest)
+    err = np.abs(ratio[:, 0].astype(np.float64) - want) / want
+    term = 7 / 8 * (2.0 ** -23 + 2.0 ** -24) + 1 / 8 * (2.0 ** -21 + 2.4e-7)
+    assert (err <= rest * want * term + 2.0 ** -24).all(), err
