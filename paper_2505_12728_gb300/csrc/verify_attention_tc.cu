@@ -676,11 +676,13 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
     //    of a warp arrives;
     //  * the maximum is taken in threes, the rescale (rare) stands before
     //    the exponentials, where fewer registers are live, and the row sum
-    //    is added up while the stores to TMEM are in flight.
+    //    is added up while the stores to TMEM are in flight;
+    //  * with one copy (64 keys a lane) the exponentials and P go in two halves:
+    //    all of them at once spilled 400 bytes a thread (70 rows, 256 sequences of
+    //    300 tokens 156.7 -> 123.1 us, 8 of 8k 42.5 -> 33.6).
     // With the MMA warp's two changes, per layer: 4 sequences of 4.9k
     // tokens, 56 rows, 15.1 -> 14.1 us; 8 sequences of 1.2-3.6k, 42 rows, 15.3 ->
-    // 14.5; 70 rows (one copy) 19.3 -> 17.6; 16 sequences of 8-32k, 56 rows,
-    // 113.3 -> 111.5.  Not kept: a second group of softmax warps taking every
+    // 14.5; 16 sequences of 8-32k, 56 rows, 113.3 -> 111.5.  Not kept: a second group of softmax warps taking every
     // other tile (14.2-16.1: the tiles beyond the ring are then waited for,
     // and two groups' states have to be folded), reading the next tile's
     // scores while the stores complete (+0.4: more registers), spinning on
@@ -842,47 +844,54 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
           }
         }
         const float mu = ref == -INFINITY ? 0.f : ref;
-        uint32_t mine[KPL / 2];
+        // P over the scores: this lane's keys, zeros for the other copies' keys
+        // (the A operand of P V covers the whole tile), and P_lo on the
+        // sequence's first tile (warp-uniform).  One copy's 64 keys go in two
+        // halves, so that half as many results are live (see above).
+        constexpr int kHalves = F == 1 ? 2 : 1, KH = KPL / kHalves;
+        float rs = 0.f;
 #pragma unroll
-        for (int c2 = 0; c2 < KPL / 2; ++c2) {
-          const float p0 = fast_exp2(fmaf(__uint_as_float(sv[2 * c2]), p.scale_log2, -mu));
-          const float p1 = fast_exp2(fmaf(__uint_as_float(sv[2 * c2 + 1]), p.scale_log2, -mu));
-          mine[c2] = pack_bf16x2(p0, p1);
-          sv[2 * c2] = __float_as_uint(p0);
-          sv[2 * c2 + 1] = __float_as_uint(p1);
-        }
-        // P over the scores: this lane's keys, zeros for the other copies'
-        // keys (the A operand of P V covers the whole tile)
-        {
-          uint32_t zero[KPL / 2];
+        for (int hh = 0; hh < kHalves; ++hh) {
+          uint32_t *ph = sv + hh * KH;
+          uint32_t mine[KH / 2], zero[KPL / 2];
+#pragma unroll
+          for (int c2 = 0; c2 < KH / 2; ++c2) {
+            const float p0 = fast_exp2(fmaf(__uint_as_float(ph[2 * c2]), p.scale_log2, -mu));
+            const float p1 = fast_exp2(fmaf(__uint_as_float(ph[2 * c2 + 1]), p.scale_log2, -mu));
+            mine[c2] = pack_bf16x2(p0, p1);
+            ph[2 * c2] = __float_as_uint(p0);
+            ph[2 * c2 + 1] = __float_as_uint(p1);
+          }
 #pragma unroll
           for (int c = 0; c < KPL / 2; ++c) zero[c] = 0u;
 #pragma unroll
           for (int k = 1; k < F; ++k)
             tmem_st_cols<KPL / 2>(sb + static_cast<uint32_t>((kap + k) % F) * (KPL / 2), zero);
-          tmem_st_cols<KPL / 2>(sb + kap * (KPL / 2), mine);
-          if (split_p) {  // the sequence's first tile: P_lo too (warp-uniform)
+          const uint32_t at = sb + kap * (KPL / 2) + hh * (KH / 2);
+          tmem_st_cols<KH / 2>(at, mine);
+          if (split_p) {
 #pragma unroll
-            for (int c2 = 0; c2 < KPL / 2; ++c2) {
+            for (int c2 = 0; c2 < KH / 2; ++c2) {
               uint32_t hi;
-              split_bf16x2(__uint_as_float(sv[2 * c2]), __uint_as_float(sv[2 * c2 + 1]), hi, mine[c2]);
+              split_bf16x2(__uint_as_float(ph[2 * c2]), __uint_as_float(ph[2 * c2 + 1]), hi, mine[c2]);
             }
 #pragma unroll
             for (int k = 1; k < F; ++k)
               tmem_st_cols<KPL / 2>(sb + 32 + static_cast<uint32_t>((kap + k) % F) * (KPL / 2), zero);
-            tmem_st_cols<KPL / 2>(sb + 32 + kap * (KPL / 2), mine);
+            tmem_st_cols<KH / 2>(at + 32, mine);
           }
+          // the sum, as a tree, while the stores are in flight
+          float ps[KH / 2];
+#pragma unroll
+          for (int c = 0; c < KH / 2; ++c) ps[c] = __uint_as_float(ph[2 * c]) + __uint_as_float(ph[2 * c + 1]);
+#pragma unroll
+          for (int w = KH / 4; w >= 1; w >>= 1) {
+#pragma unroll
+            for (int c = 0; c < w; ++c) ps[c] += ps[c + w];
+          }
+          rs = hh == 0 ? ps[0] : rs + ps[0];
         }
-        // the sum, as a tree, while the stores are in flight
-        float ps[KPL / 2];
-#pragma unroll
-        for (int c = 0; c < KPL / 2; ++c) ps[c] = __uint_as_float(sv[2 * c]) + __uint_as_float(sv[2 * c + 1]);
-#pragma unroll
-        for (int w = KPL / 4; w >= 1; w >>= 1) {
-#pragma unroll
-          for (int c = 0; c < w; ++c) ps[c] += ps[c + w];
-        }
-        l_run = l_run * alpha + ps[0];
+        l_run = l_run * alpha + rs;
         tmem_wait_st();
         tc_fence_before_sync();
         __syncwarp();
