@@ -227,8 +227,9 @@ __device__ __forceinline__ void tc_segment(const TcPartition &tp, const AttnPara
 
 // The same partition decided by one warp alone, for at most 32 sequences: lane
 // b holds sequence b, and nothing goes through shared memory or a block
-// barrier.  Every warp of a CTA takes it for itself, so that the producers
-// reach their first copies without waiting for the other roles.
+// barrier.  Every warp of a split CTA takes it for itself, so that the producers
+// reach their first copies without waiting for the other roles; the merge
+// kernel computes the block's (both give the same pieces).
 constexpr int kTcWarpBatch = 32;
 
 struct TcWarpPartition {
@@ -682,9 +683,10 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
     //    300 tokens 156.7 -> 123.1 us, 8 of 8k 42.5 -> 33.6).
     // With the MMA warp's two changes, per layer: 4 sequences of 4.9k
     // tokens, 56 rows, 15.1 -> 14.1 us; 8 sequences of 1.2-3.6k, 42 rows, 15.3 ->
-    // 14.5; 16 sequences of 8-32k, 56 rows, 113.3 -> 111.5.  Not kept: a second group of softmax warps taking every
-    // other tile (14.2-16.1: the tiles beyond the ring are then waited for,
-    // and two groups' states have to be folded), reading the next tile's
+    // 14.5; 16 sequences of 8-32k, 56 rows, 113.3 -> 111.5.  Not kept: a second
+    // group of softmax warps taking every other tile (14.2-16.1: the tiles beyond
+    // the ring are then waited for, and two groups' states have to be folded),
+    // reading the next tile's
     // scores while the stores complete (+0.4: more registers), spinning on
     // the barriers without the try_wait suspension (+0.1).
     // ------------------------------------------------------------------
@@ -1067,7 +1069,7 @@ constexpr int kTcMergeBatch = 12;
 // 256 threads x 104 registers fit next to a split CTA (224 x 128) on one SM
 constexpr int kTcMergeMaxRegs = 104;
 
-template <int D, bool kWarpPart>
+template <int D>
 __global__ void __maxnreg__(kTcMergeMaxRegs)
 verify_tc_merge_kernel(const __grid_constant__ AttnParams p) {
   constexpr float kLn2 = 0.6931471805599453f;
@@ -1078,15 +1080,13 @@ verify_tc_merge_kernel(const __grid_constant__ AttnParams p) {
   int *s_len = s_prefix + p.B + 1;   // [B]
   int *s_cpre = s_len + p.B;         // [B+1]
   grid_launch_dependents();
-  TcWarpPartition wp{};
-  TcPartition tp{};
-  if constexpr (kWarpPart) {
-    wp = tc_warp_partition(p);
-  } else {
-    tile_prefix<kTcMergeThreads>(p, s_prefix, s_len, s_scratch + 8);
-    __syncthreads();
-    tp = tc_partition<kTcMergeThreads>(p, s_prefix, s_cpre, s_scratch + 8);
-  }
+  // The partition by the block, also where the split kernel's warps take it for
+  // themselves: it is hidden behind that kernel here, and held in a warp's
+  // registers it cost the loop below some (1 sequence of 8k, 21 rows 27.1 -> 25.5 us a
+  // call, 32 of 300 tokens, 128 rows 38.2 -> 34.9).
+  tile_prefix<kTcMergeThreads>(p, s_prefix, s_len, s_scratch + 8);
+  __syncthreads();
+  const TcPartition tp = tc_partition<kTcMergeThreads>(p, s_prefix, s_cpre, s_scratch + 8);
   grid_dependency_wait();
   // work units of kTcMergeThreads items of one segment (32-bit indices:
   // the units of all segments number fewer than 2^31)
@@ -1098,12 +1098,12 @@ verify_tc_merge_kernel(const __grid_constant__ AttnParams p) {
   for (int unit = blockIdx.x; unit < units; unit += gridDim.x) {
     const int seg = unit / units_per_seg;
     const int rem = (unit - seg * units_per_seg) * kTcMergeThreads + threadIdx.x;
+    if (rem >= per_seg) continue;
     const int c4 = rem / p.R, r = rem - c4 * p.R;
     const int b = seg / p.H_kv, h_kv = seg - b * p.H_kv;
     int c_first, n_pieces;
-    if constexpr (kWarpPart) tc_warp_segment(wp, p, b, h_kv, c_first, n_pieces);
-    else tc_segment(tp, p, s_prefix, s_cpre, b, h_kv, c_first, n_pieces);
-    if (n_pieces <= 1 || rem >= per_seg) continue;  // one piece: the split kernel wrote the output
+    tc_segment(tp, p, s_prefix, s_cpre, b, h_kv, c_first, n_pieces);
+    if (n_pieces <= 1) continue;  // the split kernel wrote the output
     const int F = p.R <= 32 ? 4 : (p.R <= 64 ? 2 : 1);  // key-split copies per piece
     const float *slot0 = p.partials + (size_t)(c_first + seg) * F * stride;
     n_pieces *= F;
@@ -1229,10 +1229,8 @@ int tc_launch(int head_dim, int G, int smem, const CUtensorMap &tk, const CUtens
   cfg.gridDim = dim3(static_cast<unsigned>(ctas));
   cfg.blockDim = dim3(kTcMergeThreads);
   cfg.dynamicSmemBytes = 4 * (3 * prm.B + 2);
-  void (*merge)(const AttnParams) =
-      head_dim == 64 ? (warp_part ? verify_tc_merge_kernel<64, true> : verify_tc_merge_kernel<64, false>)
-                     : (warp_part ? verify_tc_merge_kernel<128, true> : verify_tc_merge_kernel<128, false>);
-  e = cudaLaunchKernelEx(&cfg, merge, prm);
+  e = head_dim == 64 ? cudaLaunchKernelEx(&cfg, verify_tc_merge_kernel<64>, prm)
+                     : cudaLaunchKernelEx(&cfg, verify_tc_merge_kernel<128>, prm);
   if (e != cudaSuccess) return fail(SF_ERR_CUDA, "verify merge launch: %s", cudaGetErrorString(e));
   return SF_OK;
 }
