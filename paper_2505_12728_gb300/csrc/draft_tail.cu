@@ -26,7 +26,7 @@
 //    coalesced along the vocabulary and, for the fused path, reduce each
 //    draft row over the tile to (max, first argmax, float-float sum of
 //    exp((x - max)/tau)), merged across the CTA's tiles.
-//    Tiles of 256 rows, not 128: the hidden-state box is re-read from L2 for
+//    Tiles of 256 rows, not 128 (but see launch_lm_head): the hidden-state box is re-read from L2 for
 //    every tile, and a CTA of V = 32000 (210 rows) has one tile and one
 //    exposed epilogue instead of two.  Measured with 128 and 256 rows:
 //    5 rows x 32000 x 4096 50.8 -> 41.1 us (6.4 TB/s), 36 x 152064 x 3584
@@ -86,7 +86,8 @@ struct LmParams {
   int G;             // CTAs; CTA c owns vocabulary rows [c*V/G, (c+1)*V/G)
   int ha, hb;        // box heights of the two last-tile weight maps
   int KC;            // hidden chunks of 64
-  int halves;        // 128-row halves of a tile in use (1: no CTA owns more than 128 rows)
+  int tile;          // vocabulary rows per tile: kLmTileV or kLmHalf
+  int halves;        // 128-row halves of a tile in use (1: tiles or ranges of at most 128 rows)
   int nbuf;          // accumulator buffers in tensor memory (2, or 1)
   int stages;
   uint32_t w_bytes;      // weight box of the tallest tile
@@ -258,17 +259,17 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
   const int grp = static_cast<int>(blockIdx.x) % p.G, split = static_cast<int>(blockIdx.x) / p.G;
   const int v0 = static_cast<int>(static_cast<long long>(grp) * p.V / p.G);
   const int v1 = static_cast<int>(static_cast<long long>(grp + 1) * p.V / p.G);
-  const int n_tiles = (v1 - v0 + kLmTileV - 1) / kLmTileV;
-  const int last_h = v1 - v0 - (n_tiles - 1) * kLmTileV;  // rows of the last tile
+  const int n_tiles = (v1 - v0 + p.tile - 1) / p.tile;
+  const int last_h = v1 - v0 - (n_tiles - 1) * p.tile;  // rows of the last tile
   const int kc0 = split * p.KC / p.ks;                      // this CTA's hidden chunks
   const int nkc = (split + 1) * p.KC / p.ks - kc0;
   float *const logits = p.logits + static_cast<long long>(split) * p.part_stride;
   const uint32_t total = static_cast<uint32_t>(n_tiles) * static_cast<uint32_t>(nkc);
   // weight map and box height of tile i
   auto tile_map = [&](int i, uint32_t &bytes) -> const CUtensorMap * {
-    const int h = i == n_tiles - 1 ? last_h : kLmTileV;
+    const int h = i == n_tiles - 1 ? last_h : p.tile;
     bytes = static_cast<uint32_t>(h) * (kLmChunkK * 2) + static_cast<uint32_t>(p.NP) * (kLmChunkK * 2);
-    return h == kLmTileV ? &tmap_w : (h == p.ha ? &tmap_wa : &tmap_wb);
+    return h == p.tile ? &tmap_w : (h == p.ha ? &tmap_wa : &tmap_wb);
   };
 
   grid_launch_dependents();
@@ -331,7 +332,7 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
       const CUtensorMap *mw = tile_map(i, bytes);
       if (elect_one()) {
         mbar_arrive_expect_tx(bar(FULL + q), bytes);
-        tma_load_2d(ring + static_cast<uint32_t>(q) * p.stage_bytes, mw, (kc0 + kc) * kLmChunkK, v0 + i * kLmTileV,
+        tma_load_2d(ring + static_cast<uint32_t>(q) * p.stage_bytes, mw, (kc0 + kc) * kLmChunkK, v0 + i * p.tile,
                     bar(FULL + q), pol_w);
       }
       __syncwarp();
@@ -354,7 +355,7 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
       const CUtensorMap *mw = tile_map(i, bytes);
       if (elect_one()) {
         mbar_arrive_expect_tx(bar(FULL + slot), bytes);
-        tma_load_2d(dst, mw, (kc0 + kc) * kLmChunkK, v0 + i * kLmTileV, bar(FULL + slot), pol_w);
+        tma_load_2d(dst, mw, (kc0 + kc) * kLmChunkK, v0 + i * p.tile, bar(FULL + slot), pol_w);
         tma_load_2d(dst + p.w_bytes, &tmap_h, (kc0 + kc) * kLmChunkK, 0, bar(FULL + slot), pol_h);
       }
       __syncwarp();
@@ -378,7 +379,7 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     bool ok = true;
     for (int i = 0; i < n_tiles && ok; ++i) {
       const int buf = i % p.nbuf;
-      const int halves = (i == n_tiles - 1 ? last_h : kLmTileV) > kLmHalf ? 2 : 1;
+      const int halves = (i == n_tiles - 1 ? last_h : p.tile) > kLmHalf ? 2 : 1;
       if (i >= p.nbuf) {
         int w = 1;
         if (lane == 0) w = mbar_wait_or_abort(bar(DEMPTY + buf), (i / p.nbuf - 1) & 1, s_abort);
@@ -444,7 +445,7 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
       const bool ok = mbar_wait_or_abort(bar(DFULL + buf), (i / p.nbuf) & 1, s_abort);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after_sync();
-      const int vbase = v0 + i * kLmTileV + 32 * warp;  // the warp's vocabulary rows
+      const int vbase = v0 + i * p.tile + 32 * warp;  // the warp's vocabulary rows
       const bool vin = vbase + lane < v1;
       const uint32_t acc = lane_base + static_cast<uint32_t>((buf * p.halves + hf) * p.NP);
 #pragma unroll 1
@@ -850,7 +851,7 @@ static int lm_setup(const DeviceInfo &dev) {
   return SF_OK;
 }
 
-// Tensor maps of the weights {hidden, V} (box 64 x 128, 64 x ha, 64 x hb) and
+// Tensor maps of the weights {hidden, V} (box 64 x tile, 64 x ha, 64 x hb) and
 // hidden states {hidden, R} (box 64 x NP), cached by (base, rows, hidden, box
 // rows).
 static int lm_tensor_map(CUtensorMap *out, const void *base, uint64_t rows, int hidden, uint32_t box_rows) {
@@ -944,11 +945,20 @@ static int launch_lm_head(const void *hidden, const void *weight, int R, int hid
   prm.NP = NP;
   prm.G = projection_groups(V, dev.sm_count);
   const int q = V / prm.G;  // every CTA owns q or q + 1 rows
-  const int tallest = q + (V % prm.G ? 1 : 0) < kLmTileV ? q + (V % prm.G ? 1 : 0) : kLmTileV;
+  const int most = q + (V % prm.G ? 1 : 0);
+  // 128-row tiles where two 256-row accumulators don't fit tensor memory (more
+  // than 128 draft rows) and a CTA has more than two such tiles: each tile's
+  // statistics then stand between its MMAs and the next tile's, with 128 rows they
+  // overlap.  144 draft rows x 128000 x 4096 275.1 -> 228.2 us, 256 x 152064 x 3584 411.1
+  // -> 360.4; with fewer tiles the 256-row epilogue by eight warps is shorter (160 x
+  // 60000 x 1024 81.3, 99.3 us with 128 rows).  The logits alone take 256 rows at
+  // every size (256 x 152064 x 3584 245.6, 257.8 us).
+  prm.tile = stats && 4 * NP > 512 && most > 2 * kLmTileV ? kLmHalf : kLmTileV;
+  const int tallest = most < prm.tile ? most : prm.tile;
   prm.halves = tallest > kLmHalf ? 2 : 1;
   prm.w_bytes = static_cast<uint32_t>((tallest + 7) / 8 * 8) * (kLmChunkK * 2);
-  prm.ha = (q - 1) % kLmTileV + 1;
-  prm.hb = q % kLmTileV + 1;
+  prm.ha = (q - 1) % prm.tile + 1;
+  prm.hb = q % prm.tile + 1;
   prm.KC = (hidden_size + kLmChunkK - 1) / kLmChunkK;
   prm.stage_bytes = prm.w_bytes + static_cast<uint32_t>(NP) * 128u;
   prm.stages = lm_stages(dev, prm.stage_bytes, NP);
@@ -968,7 +978,7 @@ static int launch_lm_head(const void *hidden, const void *weight, int R, int hid
   if (smem > static_cast<size_t>(dev.max_smem_optin))
     return fail(SF_ERR_UNSUPPORTED, "LM-head ring needs %zu bytes of shared memory", smem);
   CUtensorMap tw, twa, twb, th;
-  st = lm_tensor_map(&tw, weight, static_cast<uint64_t>(V), hidden_size, kLmTileV);
+  st = lm_tensor_map(&tw, weight, static_cast<uint64_t>(V), hidden_size, static_cast<uint32_t>(prm.tile));
   if (st == SF_OK)
     st = lm_tensor_map(&twa, weight, static_cast<uint64_t>(V), hidden_size, static_cast<uint32_t>(prm.ha));
   if (st == SF_OK)

@@ -121,7 +121,9 @@ def test_lm_head_exact_on_small_integer_inputs(oracle_mod, R, Hd, V):
     (33, 256, 0),     # one full tile per CTA (NP = 48)
     (128, 256, 3),    # a last tile of one row in some CTAs; double-buffered accumulators
     (129, 300, 7),    # NP = 144: a single accumulator buffer
-    (256, 513, 5),    # three tiles, single-buffered, the largest N
+    (256, 513, 5),    # more than two such tiles: tiles of 128 rows, double-buffered, the largest N
+    (160, 512, 0),    # exactly two tiles, single-buffered
+    (160, 640, 1),    # five tiles of 128 rows, or six with a last one of one row
 ])
 def test_projection_and_sampling_at_tile_edges(oracle_mod, R, rows, extra):
     """Vocabulary sizes at which the CTAs' row ranges (V / SM count) meet the
