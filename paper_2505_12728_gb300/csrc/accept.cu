@@ -673,8 +673,9 @@ accept_decide_kernel(const __grid_constant__ AccParams p, const SampStat *stats,
 __device__ void draw_residual(const AccParams &p, int b, int c, int j, RowStat rs, float tau,
                               float u_k) {
   __shared__ ff s_scan[kAccWarps];
-  __shared__ ff s_base;
-  __shared__ int s_flag, s_seg, s_token;
+  __shared__ ff s_base[kAccThreads];   // of each thread that may hold the target
+  __shared__ int s_seg[kAccThreads];
+  __shared__ int s_flag, s_owner, s_token;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int k = p.k, V = p.V, NS = p.C1;
   const bool residual = j < k;
@@ -737,7 +738,7 @@ __device__ void draw_residual(const AccParams &p, int b, int c, int j, RowStat r
   __syncthreads();  // every part of this CTA is written
   if (tid == 0) {   // release this CTA's parts, acquire the others'
     s_flag = atom_add_acq_rel_gpu(p.draw_tickets + b, 1u) == static_cast<unsigned>(p.C2 - 1);
-    s_seg = -1;
+    s_owner = INT_MAX;
     s_token = INT_MAX;
   }
   __syncthreads();
@@ -766,33 +767,38 @@ __device__ void draw_residual(const AccParams &p, int b, int c, int j, RowStat r
     scan_segments();
   }
   const ff target = ff_mul(total, u_k);
-  // u S at or past the total (rounding): the last token with mass of all
-  const bool take_last = !ff_lt(target, total);
+  // u S at or past the total (rounding), or u outside [0, 1): the last token with
+  // mass of all
+  const bool take_last = !ff_lt(target, total) || ff_lt(target, ff_of(0.f));
   // the thread's first segment whose running sum passes the target (its last
-  // one with mass if rounding leaves none), and the sum before it
+  // one with mass if rounding leaves none), and the sum before it.  The prefixes
+  // are rounded one by one and may step back by a rounding behind a segment of
+  // next to no mass, so that two threads' intervals hold a target: the first
+  // thread owns it.
   auto walk = [&]() {
     ff run = ex;
 #pragma unroll 1
     for (int at = first; at < end; ++at) {
       const ff m = mass(at);
       if (!ff_pos(m)) continue;
-      s_seg = at;
-      s_base = run;
+      s_seg[tid] = at;
+      s_base[tid] = run;
       run = ff_add(run, m);
       if (!take_last && ff_lt(target, run)) break;
     }
+    atomicMin(&s_owner, tid);
   };
   const bool here = ff_pos(sum) && (take_last || !ff_lt(target, ex));
   if (!take_last && here && ff_lt(target, next)) walk();
   __syncthreads();
-  if (s_seg < 0) {  // take_last, or rounding put the target between two threads' intervals
+  if (s_owner == INT_MAX) {  // take_last, or rounding put the target between two threads' intervals
     __syncthreads();
     if (here) atomicMax(&s_flag, tid + 1);  // the last thread with mass up to the target; 1 from the ticket
     __syncthreads();
     if (here && s_flag == tid + 1) walk();
     __syncthreads();
   }
-  const int cc = s_seg;
+  const int owner = s_owner, cc = owner == INT_MAX ? -1 : s_seg[owner];
   int token = -1;
   if (cc >= 0) {  // uniform over the block
     // the segment in ascending token order: thread t owns tokens 4t .. 4t+3
@@ -813,7 +819,7 @@ __device__ void draw_residual(const AccParams &p, int b, int c, int j, RowStat r
     }
     if (!take_last) {
       ff all;
-      ff cum = ff_add(s_base, block_scan2(ff_add(two_sum(t[0], t[1]), two_sum(t[2], t[3])), s_scan, &all));
+      ff cum = ff_add(s_base[owner], block_scan2(ff_add(two_sum(t[0], t[1]), two_sum(t[2], t[3])), s_scan, &all));
       int at = INT_MAX;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {

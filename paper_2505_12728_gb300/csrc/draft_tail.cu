@@ -576,7 +576,7 @@ sample_finish_kernel(const __grid_constant__ SampleParams p) {
   __shared__ ff s_scan[kFfWarps];
   __shared__ float s_m, s_inv, s_wm[kFfWarps];
   __shared__ int s_arg, s_cross, s_crossed, s_tok, s_last, s_wi[kFfWarps];
-  __shared__ ff s_base, s_target;
+  __shared__ ff s_base, s_target, s_bases[kBlock ? kFfThreads : 1];
   constexpr int kBatch = 4;
   constexpr unsigned kAll = 0xffffffffu;
   grid_dependency_wait();  // the statistics and logits come from the previous kernels
@@ -618,7 +618,7 @@ sample_finish_kernel(const __grid_constant__ SampleParams p) {
       s_wi[warp] = arg;
     }
     if (tid == 0) {
-      s_cross = -1;
+      s_cross = INT_MAX;
       s_tok = INT_MAX;
       s_last = -1;
     }
@@ -634,25 +634,28 @@ sample_finish_kernel(const __grid_constant__ SampleParams p) {
       invS = ff_div_to_f(1.f, total);
       target = ff_mul(total, u);
       crossed = ff_lt(target, total);  // not for u >= 1 or NaN: then the last chunk with mass
-      const bool here = ff_pos(mass) && (!crossed || tid == 0 || !ff_lt(target, ex));
+      // u < 0: the first chunk, as by one warp
+      const bool here = ff_lt(target, ff_of(0.f)) ? tid == 0 : ff_pos(mass) && (!crossed || !ff_lt(target, ex));
+      // (rounded prefixes may step back behind a chunk of next to no mass, so that
+      // two chunks hold the target: the first one)
       if (crossed && here && ff_lt(target, next)) {
-        s_cross = tid;
-        s_base = ex;
+        s_bases[tid] = ex;
+        atomicMin(&s_cross, tid);
       }
       __syncthreads();
-      if (s_cross < 0) {  // nothing crossed, or rounding put the target between two chunks' intervals
+      if (s_cross == INT_MAX) {  // nothing crossed, or rounding put the target between two chunks' intervals
         if (here) atomicMax(&s_last, tid);
         __syncthreads();
         const int owner = s_last;
         __syncthreads();
         if (tid == owner) {
           s_cross = tid;
-          s_base = ex;
+          s_bases[tid] = ex;
         }
         if (tid == 0) s_last = -1;
         __syncthreads();
       }
-      cs = s_cross;
+      cs = s_cross < INT_MAX ? s_cross : -1;
     }
   } else {
     if (tid < 32) {
@@ -782,7 +785,7 @@ sample_finish_kernel(const __grid_constant__ SampleParams p) {
   if (e0 < x0 || e0 >= x1) return;
 
   // scan the chunk in ascending order, 4 consecutive tokens per thread
-  ff base = s_base;
+  ff base = kBlock ? s_bases[cs] : s_base;
   int lastpos = -1;
   for (int s0 = e0; s0 < e1; s0 += 4 * kFfThreads) {
     float t[4];

@@ -368,12 +368,12 @@ def test_draw_finds_every_token_of_a_sparse_row(V, temp):
     # The bonus row has equal mass on n tokens at the edges of segments (1024
     # tokens), of a CTA's eight segments and of the row, none elsewhere; one
     # sequence per u in the middle of each token's interval, and u = 0, the
-    # largest float below 1 and 1.  One segment per thread of the last CTA up
-    # to V = 262144, several above.
+    # largest float below 1, 1 and (out of range) -0.5.  One segment per thread
+    # of the last CTA up to V = 262144, several above.
     support = sorted({0, 1023, 1024, 1027, 8191, 8192, 20000, 32767, 32768, V // 2, V - 1})
     n = len(support)
-    u_last = [(i + 0.5) / n for i in range(n)] + [0.0, 1.0 - 2.0 ** -24, 1.0]
-    expected = support + [support[0], support[-1], support[-1]]
+    u_last = [(i + 0.5) / n for i in range(n)] + [0.0, 1.0 - 2.0 ** -24, 1.0, -0.5]
+    expected = support + [support[0], support[-1], support[-1], support[-1]]
     B, k = len(u_last), 1
     logits = np.full((B, k + 1, V), -np.inf, np.float32)
     logits[:, :, support] = 0.25

@@ -227,6 +227,14 @@ def test_uniform_of_one_draws_the_last_token_with_mass():
         assert (tokens == V - 3001).all()
 
 
+def test_uniform_below_zero_draws_the_first_token():
+    for V in (32000, 152064):                    # a warp's combination, the block's
+        logits = np.zeros((2, V), np.float32)
+        logits[:, :3000] = -np.inf
+        _, tokens = run_sample(logits, np.full(2, -0.5, np.float32), np.ones(2, np.float32))
+        assert (tokens == 0).all()
+
+
 @pytest.mark.parametrize("V", [1000, 20000])
 def test_probabilities_show_little_but_their_own_rounding(V):
     """Flat distributions (hundreds of tokens carry the row sum): the largest
