@@ -63,7 +63,7 @@ struct alignas(16) RowStat {  // a target row, or a run of its chunks (one 16-by
 };
 
 struct alignas(16) SeqState {  // what the draw needs, in one 16-byte load
-  int j;           // first rejected position (k if none)
+  int j1;          // first rejected position (k if none) + 1; 0 between calls: no decision
   float m;         // row j's largest raw logit
   ff S;            // row j's sum of exp((x - m) / tau)
 };
@@ -652,7 +652,7 @@ accept_decide_kernel(const __grid_constant__ AccParams p, const SampStat *stats,
   if (warp == 0) {
     const int r = lane <= k ? lane : 0;
     const Decision d = decide_core(p, b, tau, s_rm[r], s_rarg[r], s_rS[r], e.tok, e.u, e.lx, e.qx, true);
-    if (lane == 0) p.seqs[b] = SeqState{d.j, d.m, d.S};
+    if (lane == 0) p.seqs[b] = SeqState{d.j + 1, d.m, d.S};
   }
 }
 
@@ -845,6 +845,7 @@ __device__ void draw_residual(const AccParams &p, int b, int c, int j, RowStat r
   if (tid == 0) {
     p.out_tokens[(size_t)b * (k + 1) + j] = token;
     p.draw_tickets[b] = 0u;
+    p.seqs[b].j1 = 0;  // every CTA of the sequence has read it
   }
 }
 
@@ -862,10 +863,13 @@ accept_draw_kernel(const __grid_constant__ AccParams p) {
   const float tau = p.tau[b];
   const float u_k = p.u[(size_t)b * (k + 1) + k];
   grid_dependency_wait();
-  if (!(tau > 0.0f)) return;  // greedy sequences are complete
+  if (!(tau > 0.0f)) {  // greedy sequences are complete
+    if (c == 0 && threadIdx.x == 0) p.seqs[b].j1 = 0;
+    return;
+  }
   const int4 sq = __ldcg(reinterpret_cast<const int4 *>(p.seqs + b));
-  const int j = sq.x;
-  if (j < 0 || j > k) {       // no decision was written (a timed-out statistics pass)
+  const int j = sq.x - 1;
+  if (j < 0 || j > k) {  // no decision was written in this call (a timed-out statistics pass)
     if (c == 0 && threadIdx.x == 0) set_status(p.status, SF_DEVICE_TIMEOUT);
     return;
   }
@@ -996,7 +1000,7 @@ __device__ __forceinline__ void decide_warp(const AccParams &p, int b, float tau
     rS = ff{v.z, v.w};
   }
   const Decision d = decide_core(p, b, tau, rm, rarg, rS, e.tok, e.u, e.lx, e.qx, true);
-  if (lane == 0) p.seqs[b] = SeqState{d.j, d.m, d.S};
+  if (lane == 0) p.seqs[b] = SeqState{d.j + 1, d.m, d.S};
 }
 
 // A run record whose row ticket is taken: the row, its number of runs and

@@ -497,3 +497,19 @@ def test_row_sums_are_taken_relative_to_near_maxima(V):
     err = np.abs(ratio[:, 0].astype(np.float64) - want) / want
     term = 7 / 8 * (2.0 ** -23 + 2.0 ** -24) + 1 / 8 * (2.0 ** -21 + 2.4e-7)
     assert (err <= rest * want * term + 2.0 ** -24).all(), err
+
+
+@pytest.mark.parametrize("mode", ["sampling", "greedy"])
+def test_no_decision_outlives_its_call(mode):
+    # The draw takes a decision for this call's by its record alone, so that a
+    # statistics pass that gave up (and leaves none) is noticed: the records'
+    # first words, behind the tickets, the run and the row records, are 0 again.
+    B, k, V = 3, 4, 50000
+    inp = make_accept_case(B, k, V, seed=8, mode=mode)
+    ws = sfv.new_workspace(sfv.accept_workspace_size(B, k, V))
+    run_accept(inp, workspace=ws)
+    rows, segments = B * (k + 1), -(-V // 1024)
+    at = 256 + sum(-(-n // 256) * 256 for n in (4 * B, 4 * rows, 4 * B, 16 * rows * segments, 16 * rows))
+    records = ws[at:at + 16 * B].view(torch.int32).view(B, 4).cpu().numpy()
+    assert records[:, 1:].any()  # the largest logits and sums of this call
+    assert (records[:, 0] == 0).all()
