@@ -1006,7 +1006,7 @@ __device__ __forceinline__ void decide_warp(const AccParams &p, int b, float tau
 // A run record whose row ticket is taken: the row, its number of runs and
 // (lane 0) the ticket's value before this warp's add.
 struct PendingTicket {
-  int row;          // -1: none
+  int row;
   int n_runs;       // runs of the row
   float tau;        // its temperature
   uint32_t ticket;  // lane 0: the row ticket before this warp's add

@@ -301,7 +301,8 @@ __device__ __forceinline__ void tc_fence_after_sync() {
 
 // Shared-memory matrix descriptor (tcgen05 format): start address (its low 18
 // bits: in a cluster the address carries the CTA's rank above them), leading-
-// and stride-dimension byte offsets (all >> 4), descriptor version 1 at bit 46, base offset 0 (every swizzle atom is 1024-byte aligned), 128-byte
+// and stride-dimension byte offsets (all >> 4), descriptor version 1 at bit
+// 46, base offset 0 (every swizzle atom is 1024-byte aligned), 128-byte
 // swizzle (layout type 2 at bits 61..63).  Adding bytes >> 4 to a descriptor
 // moves its start address: code that issues several MMAs makes one
 // descriptor per operand outside the elected thread's branch, where it is

@@ -812,7 +812,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
         }
         const int key0 = tile_pos + kap * KPL;
         if (key0 + KPL - 1 > lim) {
-          // causal mask of the draft block, positions past the end, padding rows
+          // causal mask of the draft block, positions past the end
           mx = -INFINITY;
 #pragma unroll
           for (int c = 0; c < KPL; ++c) {

@@ -110,7 +110,7 @@ def test_decisions_with_a_warp_for_each_row(oracle_mod, B, k, V):
     hidden, weight, inp, ref_logits = make_case(oracle_mod, B, k, V, 64, seed=[B, k, V], mode="alternate")
     logits, n, toks, ratio = run_fused(hidden, weight, inp)
     assert np.array_equal(logits.astype(np.float64), ref_logits)
-    assert compare_accept(oracle_accept(oracle_mod, inp), n, toks, ratio) <= max(1, B // 8)
+    assert compare_accept(oracle_accept(oracle_mod, inp), n, toks, ratio) == 0
 
 
 @pytest.mark.parametrize("B,k,V", [
@@ -128,12 +128,13 @@ def test_decisions_with_a_warp_for_each_row(oracle_mod, B, k, V):
     (5, 1, 16),
 ])
 def test_routes_behind_the_projection_agree(oracle_mod, B, k, V):
-    hidden, weight, inp, ref_logits = make_case(oracle_mod, B, k, V, 64, seed=[B, k, V, 1], mode="alternate")
+    mode = "alternate" if B > 1 else "sampling"  # (alternating starts with a greedy sequence)
+    hidden, weight, inp, ref_logits = make_case(oracle_mod, B, k, V, 64, seed=[B, k, V, 1], mode=mode)
     ref = oracle_accept(oracle_mod, inp)
     for _ in range(2):
         logits, n, toks, ratio = run_fused(hidden, weight, inp)
         assert np.array_equal(logits.astype(np.float64), ref_logits)
-        assert compare_accept(ref, n, toks, ratio) <= max(1, B // 8)
+        assert compare_accept(ref, n, toks, ratio) == 0  # no sequence is excused by its margin
 
 
 @pytest.mark.parametrize("V,d", [(152064, 3584), (32000, 4096)])
