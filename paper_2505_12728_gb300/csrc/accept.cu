@@ -63,7 +63,7 @@ struct alignas(16) RowStat {  // a target row, or a run of its chunks (one 16-by
 };
 
 struct alignas(16) SeqState {  // what the draw needs, in one 16-byte load
-  int j1;          // first rejected position (k if none) + 1; 0 between calls: no decision
+  int j1;          // first rejected position (k if none) + 1; 0: no decision (between calls; greedy)
   float m;         // row j's largest raw logit
   ff S;            // row j's sum of exp((x - m) / tau)
 };
@@ -652,7 +652,7 @@ accept_decide_kernel(const __grid_constant__ AccParams p, const SampStat *stats,
   if (warp == 0) {
     const int r = lane <= k ? lane : 0;
     const Decision d = decide_core(p, b, tau, s_rm[r], s_rarg[r], s_rS[r], e.tok, e.u, e.lx, e.qx, true);
-    if (lane == 0) p.seqs[b] = SeqState{d.j + 1, d.m, d.S};
+    if (lane == 0 && tau > 0.0f) p.seqs[b] = SeqState{d.j + 1, d.m, d.S};
   }
 }
 
@@ -669,13 +669,16 @@ accept_decide_kernel(const __grid_constant__ AccParams p, const SampStat *stats,
 // So the temperature is tested once for all terms, the last index with mass
 // is looked for only where rounding asks for it, and the scans take two
 // barriers each.  From the release of the kernel to the token, 16
-// sequences of V = 152064: 9.0 -> 7.0 us.
+// sequences of V = 152064: 9.0 -> 7.0 us.  Its CTAs have to find room beside two
+// CTAs of the statistics kernel, whose rings leave 1.6 KB of the SM's 196 KB
+// configuration, 1 KB of it reserved: 3.2 KB of shared memory here cost that
+// call 1.7 us.
 __device__ void draw_residual(const AccParams &p, int b, int c, int j, RowStat rs, float tau,
                               float u_k) {
   __shared__ ff s_scan[kAccWarps];
-  __shared__ ff s_base[kAccThreads];   // of each thread that may hold the target
-  __shared__ int s_seg[kAccThreads];
-  __shared__ int s_flag, s_owner, s_token;
+  __shared__ ff s_base[kAccWarps];   // of each warp's first thread that holds the target
+  __shared__ int s_seg[kAccWarps];
+  __shared__ int s_flag, s_owner, s_token;  // s_owner: the first such warp
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int k = p.k, V = p.V, NS = p.C1;
   const bool residual = j < k;
@@ -781,15 +784,16 @@ __device__ void draw_residual(const AccParams &p, int b, int c, int j, RowStat r
     for (int at = first; at < end; ++at) {
       const ff m = mass(at);
       if (!ff_pos(m)) continue;
-      s_seg[tid] = at;
-      s_base[tid] = run;
+      s_seg[warp] = at;
+      s_base[warp] = run;
       run = ff_add(run, m);
       if (!take_last && ff_lt(target, run)) break;
     }
-    atomicMin(&s_owner, tid);
+    atomicMin(&s_owner, warp);
   };
   const bool here = ff_pos(sum) && (take_last || !ff_lt(target, ex));
-  if (!take_last && here && ff_lt(target, next)) walk();
+  const unsigned holders = __ballot_sync(0xffffffffu, !take_last && here && ff_lt(target, next));
+  if (holders && lane == __ffs(holders) - 1) walk();
   __syncthreads();
   if (s_owner == INT_MAX) {  // take_last, or rounding put the target between two threads' intervals
     __syncthreads();
@@ -854,19 +858,26 @@ accept_draw_kernel(const __grid_constant__ AccParams p) {
   // The previous kernel (the decision kernel of this call) lets this grid
   // start only after it has itself waited for the kernel before the call, so
   // the call's inputs (temperature, uniforms) are in place already; j and
-  // the row statistics are waited for.  Every CTA waits, those of greedy
-  // sequences too: the kernel after this one waits for this grid alone, and may
-  // use the call's buffers only once the decisions are complete.
+  // the row statistics are waited for.
   grid_launch_dependents();
   const int c = blockIdx.x, b = blockIdx.y;
   const int k = p.k;
   const float tau = p.tau[b];
-  const float u_k = p.u[(size_t)b * (k + 1) + k];
-  grid_dependency_wait();
-  if (!(tau > 0.0f)) {  // greedy sequences are complete
-    if (c == 0 && threadIdx.x == 0) p.seqs[b].j1 = 0;
+  if (!(tau > 0.0f)) {  // greedy sequences are complete with the decisions
+    // The kernel after this one waits for this grid alone, and may use the call's
+    // buffers only once the decisions are complete: where no sequence draws, one
+    // CTA waits for them.  (Not all: waiting CTAs have to find room beside the
+    // previous kernel's.  16 sequences of V = 152064, half of them greedy, 31.7 us,
+    // with every CTA waiting 33.4.)
+    if (b == 0 && c == 0) {
+      int sampled = 0;
+      for (int i = threadIdx.x; i < p.B; i += kAccThreads) sampled |= p.tau[i] > 0.0f;
+      if (!__syncthreads_or(sampled)) grid_dependency_wait();
+    }
     return;
   }
+  const float u_k = p.u[(size_t)b * (k + 1) + k];
+  grid_dependency_wait();  // j and row j's statistics come from the previous kernel
   const int4 sq = __ldcg(reinterpret_cast<const int4 *>(p.seqs + b));
   const int j = sq.x - 1;
   if (j < 0 || j > k) {  // no decision was written in this call (a timed-out statistics pass)
@@ -1000,7 +1011,7 @@ __device__ __forceinline__ void decide_warp(const AccParams &p, int b, float tau
     rS = ff{v.z, v.w};
   }
   const Decision d = decide_core(p, b, tau, rm, rarg, rS, e.tok, e.u, e.lx, e.qx, true);
-  if (lane == 0) p.seqs[b] = SeqState{d.j + 1, d.m, d.S};
+  if (lane == 0 && tau > 0.0f) p.seqs[b] = SeqState{d.j + 1, d.m, d.S};
 }
 
 // A run record whose row ticket is taken: the row, its number of runs and
