@@ -997,22 +997,24 @@ static int launch_lm_head(const void *hidden, const void *weight, int R, int hid
   return SF_OK;
 }
 
-// Span per finishing CTA, a multiple of kSampleSpan.  At most two CTAs per SM as
-// long as that leaves spans of at most 4 kSampleSpan: the kernel is then a chain of
-// latencies, to which every CTA adds its combination (sampling alone, 128 x 8000
+// Span per finishing CTA, a multiple of kSampleSpan.  With vector accesses at most
+// two CTAs per SM as long as that leaves spans of at most 4 kSampleSpan: the kernel
+// is then a chain of latencies, to which every CTA adds its combination (sampling alone, 128 x 8000
 // 11.7 us with 256 CTAs, 14.7 with 512; 5 x 152064 10.7 with 250, 13.0 with 745; the
 // projection and sampling of 5 x 152064 x 3584 169.9, 172.3).  Larger ones take as
 // many CTAs as fit the GPU at once: the kernel is then bound by its bytes (64 x
 // 32000 15.3 us with 512, 16.4 with 256), and a second, nearly empty wave cost 128
-// rows of 152064 tokens a third of the kernel.
-static int finish_span(int R, int V, int sm_count) {
+// rows of 152064 tokens a third of the kernel.  So do all sizes with scalar
+// accesses, of which a thread has one in flight (projection and sampling of 32 rows
+// of 33333 tokens, hidden 1024 25.3 us, 26.6 with two CTAs per SM).
+static int finish_span(int R, int V, int sm_count, bool vec4) {
   auto span_of = [&](int per_sm) {
     const long long spans = static_cast<long long>(per_sm) * sm_count / R;
     const long long n = spans > 1 ? spans : 1;
     return ((V + n - 1) / n + kSampleSpan - 1) / kSampleSpan * kSampleSpan;
   };
   long long span = span_of(2);
-  if (span > 4 * kSampleSpan) span = span_of(kFinishCtasPerSm);
+  if (!vec4 || span > 4 * kSampleSpan) span = span_of(kFinishCtasPerSm);
   return static_cast<int>(span < V ? span : (V + 3) / 4 * 4);
 }
 
@@ -1030,7 +1032,7 @@ static int launch_finish(SampleParams prm, cudaStream_t stream) {
   DeviceInfo dev;
   const int st = current_device(&dev);
   if (st != SF_OK) return st;
-  prm.span = finish_span(prm.R, prm.V, dev.sm_count);
+  prm.span = finish_span(prm.R, prm.V, dev.sm_count, prm.vec4 != 0);
   const int spans = (prm.V + prm.span - 1) / prm.span;
   // Projection and sampling of 5 rows, 32000 x 4096 (160 CTAs, 152 chunks) 52.1 ->
   // 49.8 us, 9 rows, 32000 x 2048 (288 CTAs) 31.0 -> 29.2; beyond two CTAs per SM the
