@@ -513,3 +513,20 @@ def test_no_decision_outlives_its_call(mode):
     records = ws[at:at + 16 * B].view(torch.int32).view(B, 4).cpu().numpy()
     assert records[:, 1:].any() == (mode == "sampling")  # the largest logits and sums of this call
     assert (records[:, 0] == 0).all()
+
+
+def test_first_call_of_a_size_while_capturing(oracle_mod):
+    # the question how many clusters of a size are resident is asked at the first
+    # call of that size, which may be one that is being recorded
+    run_accept(make_accept_case(1, 2, 3000, seed=1))  # the kernel has been set up
+    for B, k, V in [(2, 7, 13001), (3, 11, 21004), (6, 9, 31996)]:  # no draw within 1e-6 of a boundary
+        inp = make_accept_case(B, k, V, seed=[B, k, V], mode="sampling")
+        dev = accept_to_device(inp)
+        ws = sfv.new_workspace(sfv.accept_workspace_size(B, k, V))
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            out = sfv.accept(**dev, workspace=ws)
+        g.replay()
+        torch.cuda.synchronize()
+        assert compare_accept(oracle_accept(oracle_mod, inp), *(t.cpu().numpy() for t in out)) == 0
