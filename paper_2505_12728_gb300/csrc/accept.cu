@@ -1542,21 +1542,35 @@ int sf_verify_lm_head_accept(const void *hidden, const void *weight, const float
   uint8_t *ws = static_cast<uint8_t *>(workspace);
   const bool vec4 = (V % 4 == 0) && aligned(logits, 16) && aligned(draft_probs, 16);
   int Gl = 0;
-  // Where sf_accept is one cluster launch with the draft rows fetched ahead, it
-  // is mostly shorter than the statistics epilogue, the decisions and the draw:
-  // the projection then writes the logits alone, and the cluster sums the rows at
-  // the statistics' precision.  Those sums cost it 0.4 us a row, the statistics
-  // more with every 16 rows and at temperatures other than 1, so few drafts or many
-  // sequences go that way.  Whole calls, statistics -> cluster, at temperature 1
-  // and 0.7: B = 1, k = 2, V = 2000 18.9 -> 15.6, 24.9 -> 17.4 us; B = 1, k = 5, V = 32000
-  // 55.0 -> 55.0, 61.6 -> 59.1; B = 8, k = 5 59.3 -> 58.3, 74.4 -> 62.1; B = 16, k = 8,
-  // V = 8000 35.3 -> 31.2, 70.3 -> 36.7; the other side of the line: B = 1, k = 8, V =
-  // 32000 54.8 -> 58.6, 63.0 -> 64.6; B = 4, k = 8, V = 2000 20.0 -> 23.0, 33.2 -> 28.5.
-  // Not fetched ahead it is longer (B = 2, k = 16, V = 32000 58.1 -> 61.0 before the
-  // finer sums).
+  // Where sf_accept is one cluster launch with the draft rows fetched ahead, the
+  // projection can write the logits alone and the cluster sums the rows at the
+  // statistics' precision, in place of the statistics, the decisions and the
+  // draw.  A cluster takes its rows one after another, 0.7-1.1 us each; the
+  // statistics cost more with every 16 rows and at temperatures other than 1.  So
+  // one draft, many sequences or few rows go to the cluster, long rows of more
+  // sequences than clusters run at a time don't.  Whole calls (us at
+  // temperature 1 and 0.7, statistics -> cluster), on its side of each line:
+  //   k = 1, B = 4        V = 2000 15.6 -> 15.0, 20.5 -> 17.2; 32000 25.1 -> 23.8, 29.9 -> 26.7
+  //   k = 8, B = 12       V = 2000 27.2 -> 25.1, 32.2 -> 32.8; 16000 30.4 -> 27.0, 35.9 -> 34.5
+  //   k = 3, B = 64       V = 8000 45.8 -> 31.0, 51.2 -> 35.2
+  //   k = 3, B = 1        V = 2000 17.2 -> 16.6, 20.6 -> 20.2; 32000 25.1 -> 22.1, 31.2 -> 25.0
+  //   k = 2, B = 4        V = 8000 17.8 -> 16.2, 22.4 -> 18.8
+  //   k = 5, B = 1        V = 16000 19.6 -> 18.6, 24.5 -> 23.9; 32000 25.2 -> 23.9, 31.1 -> 28.8
+  // and beyond it:
+  //   k = 1, B = 32       V = 32000 30.3 -> 32.3, 34.6 -> 36.3
+  //   k = 16, B = 12      V = 8000 39.3 -> 39.1, 44.7 -> 45.8
+  //   k = 8, B = 8        V = 2000 23.5 -> 24.4, 28.3 -> 32.0; 32000 32.6 -> 32.7, 38.6 -> 39.0
+  //   k = 3, B = 4        V = 2000 16.3 -> 17.3, 19.9 -> 20.8; 32000 25.1 -> 25.8, 29.4 -> 30.0
+  //   k = 2, B = 4        V = 16000 19.4 -> 22.0, 24.4 -> 24.2
+  //   k = 5, B = 1        V = 8000 18.0 -> 18.6, 21.8 -> 23.3
+  //   k = 5, B = 2        V = 2000 15.9 -> 18.5, 20.5 -> 23.9; 32000 25.3 -> 25.9, 30.9 -> 31.4
+  // (d = 1024).  Not fetched ahead it is longer (B = 2, k = 16, V = 32000, d = 4096 58.1 ->
+  // 61.0 before the finer sums).
+  const bool few = (B <= 2 && k <= 3) || (k == 2 && V <= 8192) || (B == 1 && k <= 5 && V > 12288);
+  const bool many = (k == 1 || (k <= 8 && B >= 12)) && (V <= 16384 || B <= 16);
   int cs = 0, slice = 0, bufs = 0;
   bool cluster_ok = false, ahead = false;
-  if ((k <= 5 || B >= 8) && cluster_plan(V, &cs, &slice)) {
+  if ((few || many) && cluster_plan(V, &cs, &slice)) {
     st = cluster_setup(cs, true, &cluster_ok);
     if (st == SF_OK && cluster_ok) st = cluster_rows(B, k, V, cs, slice, vec4, true, &bufs, &ahead);
     if (st != SF_OK) return st;

@@ -120,9 +120,20 @@ def test_decisions_with_a_warp_for_each_row(oracle_mod, B, k, V):
     (1, 5, 32768),     # the longest rows of a cluster
     (1, 5, 32772),     # one step beyond
     (1, 8, 32772),
-    (7, 6, 8000),      # statistics, decisions and draw: six drafts
-    (8, 6, 8000),      # a cluster launch: eight sequences
-    (8, 8, 32000),     # statistics: eight clusters aren't resident with draft rows ahead
+    (1, 5, 12288),     # five drafts of one sequence: statistics up to here
+    (1, 5, 12292),     # and a cluster launch from here
+    (2, 5, 12292),
+    (2, 3, 5000),      # few rows: cluster
+    (3, 3, 5000),      # statistics
+    (4, 2, 8192),      # cluster
+    (4, 2, 8196),      # statistics
+    (11, 6, 8000),     # statistics
+    (12, 6, 8000),     # many sequences: cluster
+    (12, 9, 8000),     # statistics: nine drafts
+    (17, 2, 16384),    # cluster
+    (17, 1, 16388),    # statistics
+    (8, 8, 32000),     # statistics
+    (12, 8, 21840),    # draft rows within 8 MiB, but are twelve clusters resident with them?
     (2, 16, 32000),    # rows and draft rows don't fit shared memory together
     (3, 4, 5001),      # not 16-byte aligned
     (5, 1, 16),
