@@ -22,8 +22,9 @@
 //    accept_draw_kernel (the residual draw in C2 CTAs per sequence over row
 //    j, the last CTA of a sequence scanning for u_k * S);
 //  * behind the fused LM head, whose projection already left per-CTA row
-//    statistics: accept_decide_kernel then accept_draw_kernel (small batches
-//    of V <= 16 x 2048: the cluster kernel on the projection's logits).
+//    statistics: accept_decide_kernel then accept_draw_kernel (few rows,
+//    one draft or many sequences of V <= 16 x 2048: the cluster kernel on the
+//    projection's logits).
 // Every launch uses programmatic stream serialisation: a kernel is resident
 // while the previous one drains and waits for it (griddepcontrol.wait)
 // before reading its results.
@@ -210,8 +211,8 @@ __device__ __forceinline__ DraftEntry load_draft(const AccParams &p, int b) {
 //  5. after the second cluster barrier the CTA holding u_k * S finds the token
 //     by a float-float scan over its threads' terms.
 // Nobody touches a peer's shared memory after the second barrier.  Measured
-// back to back (V = 32000): B = 1, k = 5 17.6 -> 11.3 us, greedy 5.4 -> 4.4; B = 16,
-// k = 8 31.1 -> 24.0; B = 64, k = 4 76 -> 40 us, against the same phases with
+// back to back (V = 32000): B = 1, k = 5 17.5 -> 11.4 us, greedy 5.2 -> 4.4; B = 16,
+// k = 8 32.7 -> 23.1; B = 64, k = 4 77.3 -> 38.3 us, against the same phases with
 // four barriers, the decisions in CTA 0 alone, row j read again from memory
 // and the sums combined warp by warp.
 constexpr int kClusterMax = 16;
@@ -1330,7 +1331,7 @@ static int chunks_setup(int device) {
 // resident so; else kClusterFewBufs rows at a time: more clusters per SM are worth
 // a second round of copies (B = 16, k = 8, V = 32000: 33 us with all nine rows, 26
 // with five; draft rows ahead in two waves of clusters: B = 8, k = 8, V = 32000
-// 27.2 us, without them 18.3).
+// 27.2 us, without them 16.7).
 static int cluster_rows(int B, int k, int V, int cs, int slice, bool vec4, bool exact, int *bufs, bool *ahead) {
   int n = 0;
   int st = cluster_resident(cs, cluster_smem(k, slice, k + 1, false), exact, &n);

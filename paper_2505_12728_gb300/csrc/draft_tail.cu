@@ -26,11 +26,11 @@
 //    coalesced along the vocabulary and, for the fused path, reduce each
 //    draft row over the tile to (max, first argmax, float-float sum of
 //    exp((x - max)/tau)), merged across the CTA's tiles.
-//    Tiles of 256 rows, not 128 (but see launch_lm_head): the hidden-state box is re-read from L2 for
-//    every tile, and a CTA of V = 32000 (210 rows) has one tile and one
-//    exposed epilogue instead of two.  Measured with 128 and 256 rows:
-//    5 rows x 32000 x 4096 50.8 -> 41.1 us (6.4 TB/s), 36 x 152064 x 3584
-//    171.0 -> 161.7, 128 x 152064 x 3584 195.7 -> 183 us.
+//    Tiles of 256 rows, not 128 (but see launch_lm_head): the hidden-state box
+//    is re-read from L2 for every tile, and a CTA of V = 32000 (210 rows) has
+//    one tile and one exposed epilogue instead of two.  Measured with 128 and 256 rows:
+//    5 rows x 32000 x 4096 50.8 -> 39.8 us (6.6 TB/s), 36 x 152064 x 3584
+//    171.0 -> 161.7, 128 x 152064 x 3584 195.7 -> 184 us.
 //    Weight copies run before griddepcontrol.wait (the weights are constant);
 //    the hidden states are copied after it.
 //  * sample_stats_kernel (sf_sample only): the same per-chunk statistics

@@ -683,7 +683,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
     //    300 tokens 156.7 -> 123.1 us, 8 of 8k 42.5 -> 33.6).
     // With the MMA warp's two changes, per layer: 4 sequences of 4.9k
     // tokens, 56 rows, 15.1 -> 14.1 us; 8 sequences of 1.2-3.6k, 42 rows, 15.3 ->
-    // 14.5; 16 sequences of 8-32k, 56 rows, 113.3 -> 111.5.  Not kept: a second
+    // 14.5; 16 sequences of 8-32k, 56 rows, 113.3 -> 110.  Not kept: a second
     // group of softmax warps taking every other tile (14.2-16.1: the tiles beyond
     // the ring are then waited for, and two groups' states have to be folded),
     // reading the next tile's

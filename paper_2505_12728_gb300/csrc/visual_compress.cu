@@ -34,8 +34,9 @@
 // 128 x 144 x 3584, C 16: 55.9 -> 46.6; 1 x 576 x 4096, C 64: 36.9 -> 14.5.
 // A single launch with a cluster per frame, the scores exchanged through
 // distributed shared memory, was slower (31.7 and 48.9 us): a CTA's 147 KB of
-// partial scores and 74 KB of weights move at ~13 bytes per clock.  Computing the weights in the third kernel instead of the second:
-// 46.1 us for the video shape, 66.6 for the images.
+// partial scores and 74 KB of weights move at ~13 bytes per clock.  Computing
+// the weights in the third kernel instead of the second: 46.1 us for the video
+// shape, 66.6 for the images.
 // N is at most 768 and C at most 128.  Every wait is bounded
 // (SF_DEVICE_TIMEOUT).
 #include <cmath>
