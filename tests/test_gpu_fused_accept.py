@@ -133,7 +133,7 @@ def test_decisions_with_a_warp_for_each_row(oracle_mod, B, k, V):
     (17, 2, 16384),    # cluster
     (17, 1, 16388),    # statistics
     (8, 8, 32000),     # statistics
-    (12, 8, 21840),    # draft rows within 8 MiB, but are twelve clusters resident with them?
+    (12, 8, 21840),    # draft rows of just under 8 MiB
     (2, 16, 32000),    # rows and draft rows don't fit shared memory together
     (3, 4, 5001),      # not 16-byte aligned
     (5, 1, 16),
